@@ -224,23 +224,37 @@ struct Pool {
 
 }  // namespace
 
-// The temperature below which some species may have |G/RT| > kBigGRT, from G/RT of
-// every species on a 0.25 K grid over [kTmin, kTmax] with a threshold 10 below
-// kBigGRT: by d(G/RT)/dT = -(H/RT)/T, |G/RT| changes by at most 0.25 |H/RT| / T
-// between grid points, under 10 while |H/RT| < 40 T (8,000 at 200 K). A mechanism
-// with a larger |H/RT| anywhere in the range always takes the one-exponential path.
-// Returns 0 when no species comes near the threshold in the whole range.
-static double big_gibbs_temperature(const chem_mechanism_desc* d) {
-  const double thr = kBigGRT - 10.0;
-  double Tb = 0.0;
+// v 2^q rounded to an integer; *ok is cleared when it does not stay inside the format.
+static long long to_fixed(long double v, int q, bool* ok) {
+  const long double s = std::ldexp(v, q);
+  if (!(std::fabs(s) < 9.2e18L)) {
+    *ok = false;
+    return 0;
+  }
+  return (long long)std::llround(s);
+}
+
+// Largest |a + b ln T - c/T| over [kTmin, kFxThi), from above.
+static long double arrhenius_range(long double a, long double b, long double c) {
+  return std::fabs(a) + std::fabs(b) * 9.02L + std::fabs(c) / (long double)kTmin;
+}
+
+// The lowest temperature from which the fixed-point rate evaluation holds: |G/RT| of
+// every species at most kFxGRT from there to kFxThi. G/RT is scanned on a 0.5 K grid
+// with a threshold 10 below kFxGRT: by d(G/RT)/dT = -(H/RT)/T, |G/RT| changes by at most
+// 0.5 |H/RT| / T between grid points, under 10 while |H/RT| < 20 T (4,000 at 200 K);
+// a mechanism with a larger |H/RT| anywhere in the range does without (1e300).
+static double fixed_point_temperature(const chem_mechanism_desc* d) {
+  const double thr = kFxGRT - 10.0;
+  double Tb = kTmin;
   for (int k = 0; k < d->n_species; ++k) {
     bool found = false;
-    for (double T = kTmax; T >= kTmin; T -= 0.25) {
+    for (double T = kFxThi; T >= kTmin; T -= 0.5) {
       const double* a = (T < d->T_mid[k] ? d->nasa_lo : d->nasa_hi) + 7 * k;
       const double hrt = h_RT(a, T);
-      if (!(std::fabs(hrt) < 40.0 * T)) return 1e300;
+      if (!(std::fabs(hrt) < 20.0 * T)) return 1e300;
       if (!found && std::fabs(hrt - s_R(a, T)) > thr) {
-        Tb = std::max(Tb, T + 0.25);
+        Tb = std::max(Tb, T + 0.5);
         found = true;
       }
     }
@@ -281,21 +295,21 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
   // Each kind group is padded with null reactions to whole 32-reaction chunks, so a
   // warp's chunk never mixes kinds; chunks are dealt to warps by decreasing cost.
   std::vector<int> padded;
-  std::vector<double> chunk_cost;  // estimated FP64 instructions of one rate evaluation
+  std::vector<double> chunk_cost;  // estimated time of one rate evaluation, in FP64 warp instructions (64 cycles)
   for (int kind = 0; kind < 4; ++kind) {
     size_t first = padded.size();
     for (int i = 0; i < I; ++i)
       if (d->rxn_type[order[i]] == kind) padded.push_back(order[i]);
     if (padded.size() == first) continue;
     while (padded.size() % 32) padded.push_back(-1);
-    const double cost = kind == 0 ? 28.0 : kind == 1 ? 31.0 : kind == 2 ? 60.0 : 220.0;
+    const double cost = kind == 0 ? 9.0 : kind == 1 ? 23.0 : kind == 2 ? 34.0 : 62.0;
     for (size_t c = first; c < padded.size(); c += 32) chunk_cost.push_back(cost);
   }
   const int Ip = (int)padded.size();
   const int n_chunks = (int)chunk_cost.size();
   // Deal the chunks to warps, longest first, each to the warp with the least estimated
-  // work so far; the species loops (thermo, production rates: ~72 per 32 species) load
-  // the warps holding species and the CTA's scalar work (~60) the last warp.
+  // work so far; the species loops (thermo, production rates: ~45 per 32 species) load
+  // the warps holding species and the CTA's scalar work (~15) the last warp.
   std::vector<int> by_cost(n_chunks);
   std::iota(by_cost.begin(), by_cost.end(), 0);
   std::stable_sort(by_cost.begin(), by_cost.end(), [&](int a, int b) { return chunk_cost[a] > chunk_cost[b]; });
@@ -306,9 +320,9 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
     for (int w = 0; w < NW; ++w) {
       int cnt = 0;
       for (int k = 0; k < K; ++k) cnt += (k % NT) / 32 == w;
-      load[w] = 72.0 * ((cnt + 31) / 32);
+      load[w] = 45.0 * ((cnt + 31) / 32);
     }
-    load[NW - 1] += 60.0;
+    load[NW - 1] += 15.0;
     std::vector<std::vector<int>> own(NW);
     for (int ch : by_cost) {
       int w = 0;
@@ -411,6 +425,45 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
     for (int k = 0; k < K; ++k) ptr[k + 1] = ptr[k] + (int)v[k].size();
     for (int k = 0; k < K; ++k) ent.insert(ent.end(), v[k].begin(), v[k].end());
   };
+  // fixed-point copies for the rate evaluation; every argument has to stay inside +-2000
+  bool fx_ok = true;
+  std::vector<long long> gfx((size_t)16 * K, 0), arx(arr.size(), 0), fox(fo.size() / 2, 0);
+  for (int k = 0; k < K; ++k) {
+    if (!(d->T_mid[k] <= 2048.0)) fx_ok = false;  // t = T/2048 below T_mid
+    for (int r = 0; r < 2; ++r) {
+      const double* a = (r == 0 ? d->nasa_lo : d->nasa_hi) + 7 * k;
+      long long* o = &gfx[16 * k + 8 * r];
+      const long double S = r == 0 ? 2048.0L : 8192.0L;
+      // G/RT = (a1 - a7) - a1 ln T + a6/T - a2/2 T - a3/6 T^2 - a4/12 T^3 - a5/20 T^4
+      const long double c[4] = {-a[1] / 2.0L * S, -a[2] / 6.0L * S * S, -a[3] / 12.0L * S * S * S,
+                                -a[4] / 20.0L * S * S * S * S};
+      const long double c0 = (long double)a[0] - a[6];
+      if (!(arrhenius_range(c0, a[0], a[5]) + std::fabs(c[0]) + std::fabs(c[1]) + std::fabs(c[2]) + std::fabs(c[3]) <
+            2000.0L))
+        fx_ok = false;
+      o[0] = to_fixed(c0, 52, &fx_ok) + 2;  // + 2: the mean of the products' truncations
+      o[1] = to_fixed(-(long double)a[0], 58, &fx_ok);
+      o[2] = to_fixed(a[5], 45, &fx_ok);
+      for (int j = 0; j < 4; ++j) o[3 + j] = to_fixed(c[j], 52, &fx_ok);
+    }
+  }
+  auto fix_arrhenius = [&](long double A, double b, double E, long long* o) {
+    if (!(arrhenius_range(A, b, E) < 2000.0L)) fx_ok = false;
+    o[0] = to_fixed(A, 52, &fx_ok);
+    o[1] = to_fixed(b, 58, &fx_ok);
+    o[2] = to_fixed(E, 45, &fx_ok);
+  };
+  for (int i = 0, f = 0; i < Ip; ++i) {
+    const int o = padded[i];
+    const bool falloff = pkind[i] >= 2;
+    if (o >= 0) {
+      const long double lnA = std::log((long double)d->A[o]);
+      fix_arrhenius(lnA, d->b[o], d->Ea_R[o], &arx[4 * i]);
+      if (falloff)
+        fix_arrhenius(std::log((long double)d->A0[o]) - lnA, d->b0[o] - d->b[o], d->Ea0_R[o] - d->Ea_R[o], &fox[4 * f]);
+    }
+    if (falloff) ++f;
+  }
   std::vector<int> sp_ptr, tr_ptr;
   std::vector<int2> sp_ent, tr_ent;
   flatten2(sp, sp_ptr, sp_ent);
@@ -505,7 +558,8 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
                oJm = P.add(jmask.data(), jmask.size() * 4),
                oEf = P.add(eff_ff.data(), eff_ff.size() * 4), oiWf = P.add(invW_ff.data(), invW_ff.size() * 4),
                oEt = P.add(effT.data(), effT.size() * 8), oEtf = P.add(effT_ff.data(), effT_ff.size() * 4),
-               oTnf = P.add(tr_nu_ff.data(), tr_nu_ff.size() * 4);
+               oTnf = P.add(tr_nu_ff.data(), tr_nu_ff.size() * 4), oGx = P.add(gfx.data(), gfx.size() * 8),
+               oAx = P.add(arx.data(), arx.size() * 8), oFx = P.add(fox.data(), fox.size() * 8);
   size_t oJe[3], oJn[3], oJnf[3], oCs[3];
   for (int v = 0; v < 3; ++v) {
     oCs[v] = P.add(chunk_sched[v].data(), chunk_sched[v].size() * 4);
@@ -526,7 +580,10 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
   m.i_tb0 = i_tb0;
   m.i_fo0 = i_fo0;
   m.i_troe0 = i_troe0;
-  m.T_bigG = big_gibbs_temperature(d);
+  m.T_fx = fx_ok ? fixed_point_temperature(d) : 1e300;
+  m.gfx = reinterpret_cast<const long long*>(b + oGx);
+  m.arx = reinterpret_cast<const long long*>(b + oAx);
+  m.fox = reinterpret_cast<const long long*>(b + oFx);
   m.W = reinterpret_cast<const double*>(b + oW);
   m.invW = reinterpret_cast<const double*>(b + oiW);
   m.nasa = reinterpret_cast<const double*>(b + oN);

@@ -29,6 +29,7 @@
 #include <type_traits>
 
 #include "chem.h"
+#include "chem_fixed.cuh"
 #include "chem_internal.h"
 #include "chem_kernels.h"
 #include "rodas4.h"
@@ -443,6 +444,7 @@ static __device__ __noinline__ double exp_outside(double x) { return exp(x); }
 
 constexpr double kInvLn10 = 0.43429448190325176;  // 1 / ln 10
 constexpr double kLnRcP0 = 4.407418589020958;  // ln(Rc / P0), cgs
+constexpr long long kLnRcP0_Q52 = 19849248715180584ll;
 
 __device__ __forceinline__ double xexp(double x) {
   if ((__double2hiint(x) & 0x7fffffff) >= 0x40850000) return exp_outside(x);  // |x| >= 672, inf, NaN
@@ -707,7 +709,7 @@ struct Layout {
 __host__ __device__ inline int odd_ld(int n) { return n | 1; }
 
 // vectors (double): y, yn, ys, f0, fv, rr, u[6], sc  -> 13 n
-// species (double): C, hRT, cpR, eg, dcp, dk, akT, ek, ieg -> 9 K
+// species (8 bytes): C, hRT, cpR, g, dcp, dk, akT, ek -> 8 K
 // reactions (double): q, D, dTc, P, dqs[4] -> 8 I
 // m0_global: the mixed form's assembled matrix lives in a global-memory slot of
 // the CTA instead of shared memory (large mechanisms, persistent schedulers).
@@ -723,7 +725,7 @@ __host__ __device__ inline Layout make_layout(int Kmax, int Imax, int prec, bool
   L.off_vec = o;
   o += (size_t)13 * L.nmax * sizeof(double);
   L.off_sp = o;
-  o += (size_t)9 * Kmax * sizeof(double);
+  o += (size_t)8 * Kmax * sizeof(double);
   L.off_rx = o;
   if (prec == PREC_FP64) {
     o += (size_t)8 * Imax * sizeof(double);
@@ -765,7 +767,7 @@ struct Cta {
   // vectors
   double *y, *yn, *ys, *f0, *fv, *rr, *u, *sc;
   // species
-  double *C, *hRT, *cpR, *eg, *dcp, *dk, *akT, *ek, *ieg;
+  double *C, *hRT, *cpR, *g, *dcp, *dk, *akT, *ek;
   // reactions
   double *q, *D, *dTc, *P, *dqs;
   void* M;
@@ -793,12 +795,11 @@ struct Cta {
     C = s;
     hRT = s + K;
     cpR = s + 2 * K;
-    eg = s + 3 * K;
+    g = s + 3 * K;
     dcp = s + 4 * K;
     dk = s + 5 * K;
     akT = s + 6 * K;
     ek = s + 7 * K;
-    ieg = s + 8 * K;
     double* r = reinterpret_cast<double*>(base + L.off_rx);
     const int I = L.Imax;
     q = r;
@@ -895,7 +896,7 @@ __device__ __forceinline__ int warps_for(int count) {
 
 // Cell-level scalars shared by all threads of the CTA (identical in every thread).
 struct Scal {
-  double T, invT, logT, rho, irho, Wbar, cpm, icpm, fT, dcpm, Scpw;
+  double T, invT, rho, irho, Wbar, cpm, icpm, fT, dcpm, Scpw;
 };
 
 // ---------------------------------------------------------------------------
@@ -905,22 +906,41 @@ struct Scal {
 // Jacobian assembly needs: per reaction the slot derivatives dq/dC, dq/dT at
 // fixed C, sum_k C_k dq/dC_k (D), and the third-body/falloff coefficient P of
 // eff_j in dq/dC_j; per species d_k = sum_i nu_ki D_i and a_kT = sum nu dTc.
-// BIG: the cell's T is below the mechanism's T_bigG, where some species may have
-// |G/RT| > kBigGRT (very low T with large formation enthalpies): the reverse-rate
-// ratio then takes one exponential of the summed exponent per reaction instead of
-// the product of four species factors, whose partial products could overflow or
-// underflow. A separate instantiation, so that the common path carries no trace of it.
+// Rate constants come from one exponential each: kf from ln A + b ln T - Theta/T
+// (+ the falloff terms), kr from that argument + dG/RT + dnu ln(Rc T/P0).
+// FX: arguments, logarithms and exponentials in 64-bit fixed point (chem_fixed.cuh),
+// for T in [m.T_fx, kFxThi), where every argument fits; otherwise (FX = false, out of
+// line) the same formulas in FP64. One RHS of the 54-species mechanism issues 196 FP64
+// warp instructions with FX, 546 with FP64 exponentials and species factors
+// exp(+-G/RT) (counted in the source); the FP64 pipe bounded the rate evaluation.
 // FF (the forms with FP32 factors): the third-body sums [M] in float-float, and the
 // slot derivatives and P stored as float-float pairs for the assembly.
-template <int NW, bool JAC, bool FF, bool BIG>
+template <bool FX>
+__device__ __forceinline__ double rate_exp(typename std::conditional<FX, long long, double>::type a) {
+  if constexpr (FX) return fx_exp(a);
+  else return xexp(a);
+}
+template <bool FX>
+__device__ __forceinline__ double rate_log(double x) {
+  if constexpr (FX) {
+    const int hx = __double2hiint(x);
+    if (hx < 0x00100000 || hx >= 0x7ff00000) return log_outside(x);
+    return fx_to_double(fx_log<52>(x));
+  } else {
+    return xlog(x);
+  }
+}
+
+template <int NW, bool JAC, bool FF, bool FX>
 __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double p, double* f) {
   constexpr int NT = NW * 32;
+  using Arg = typename std::conditional<FX, long long, double>::type;
   const int K = m.K;
   Scal s;
   s.T = y[0];
   // the scalar warp: ln T and 1/T for every thread (read after the reduction's barriers)
   if (c.warp == Cta<NW>::SW) {
-    const double lg = xlog(s.T);
+    const double lg = FX ? __longlong_as_double(fx_log<58>(s.T)) : xlog(s.T);
     const double iT = xrcp(s.T);
     if (c.lane == 0) {
       c.red[SC_LOGT] = lg;
@@ -943,35 +963,42 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
     s.rho = o[1];
     s.irho = o[2];
   }
-  s.logT = c.red[SC_LOGT];
+  const double lgT = c.red[SC_LOGT];
   s.invT = c.red[SC_INVT];
-  const double T = s.T, invT = s.invT, logT = s.logT;
-  // species: thermo, exp(G/RT), concentrations
+  const double T = s.T, invT = s.invT;
+  // ln T (Q58), 1/T (Q71) and ln(Rc T/P0) (Q52), or their FP64 forms
+  const unsigned long long LT = (unsigned long long)__double_as_longlong(lgT);
+  const unsigned long long IT = fx_scale(invT, 19);
+  const Arg lc = FX ? (Arg)((long long)(LT >> 6) + kLnRcP0_Q52) : (Arg)(lgT + kLnRcP0);
+  Arg* const g_RT = reinterpret_cast<Arg*>(c.g);
+  // species: thermo, G/RT, concentrations
   for (int k = c.tid; k < K; k += NT) {
     const double* a = m.nasa + 36 * k;
-    a += (T < a[34]) ? 0 : 17;
+    const bool low = T < a[34];
+    a += low ? 0 : 17;
     double cp = a[0] + T * (a[1] + T * (a[2] + T * (a[3] + T * a[4])));
     double h = a[5] + T * (a[6] + T * (a[7] + T * (a[8] + T * a[9]))) + a[10] * invT;
-    double sr = a[11] * logT + T * (a[12] + T * (a[13] + T * (a[14] + T * a[15]))) + a[16];
     c.cpR[k] = cp;
     c.hRT[k] = h;
-    const double g = h - sr;
-    const double e = xexp(g);
-    c.eg[k] = e;
-    c.ieg[k] = xrcp(e);
-    if (BIG) c.ek[k] = g;  // G/RT (the slot is the Jacobian assembly's, unused until then)
+    if constexpr (FX) {
+      // T / 2048 below T_mid, T / 8192 above (Q64)
+      const unsigned long long t = fx_scale(T, low ? 1 : -1);
+      const longlong2* q = reinterpret_cast<const longlong2*>(m.gfx + 16 * k + (low ? 0 : 8));
+      const longlong2 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3];
+      const long long poly = fx_mul(q1.y + fx_mul(q2.x + fx_mul(q2.y + fx_mul(q3.x, t), t), t), t);
+      g_RT[k] = q0.x + fx_mul(q0.y, LT) + fx_mul(q1.x, IT) + poly;
+    } else {
+      const double sr = a[11] * lgT + T * (a[12] + T * (a[13] + T * (a[14] + T * a[15]))) + a[16];
+      g_RT[k] = h - sr;
+    }
     const double Ck = s.rho * y[1 + k] * m.invW[k];
     c.C[k] = Ck;
     // float-float copy of C for the third-body sums (the slot of d_k, which the
     // Jacobian evaluation writes only after the reaction loop)
     if (FF) reinterpret_cast<ff2*>(c.dk)[k] = ff_split(Ck);
     if (JAC) c.dcp[k] = a[1] + T * (2.0 * a[2] + T * (3.0 * a[3] + T * 4.0 * a[4]));
-    // without Jacobian data the reverse term needs only C_k exp(G_k/RT) (the dcp slot)
-    if (!JAC && !BIG) c.dcp[k] = Ck * e;
   }
   __syncthreads();
-  const double cRT = kRc * T / kP0;  // (P0 / (Rc T))^-1
-  const double icRT = kP0 * invT / kRc;
   // 32-reaction chunks of one kind each, dealt to the warps by estimated work
   const int* cs = m.chunk_sched[NW == 2 ? 0 : NW == 4 ? 1 : 2];
   for (int pos = cs[c.warp]; pos < cs[c.warp + 1]; ++pos) {
@@ -985,38 +1012,29 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
       }
       continue;
     }
-    const double* arp = m.arr + 4 * i;
-    const double2 a01 = reinterpret_cast<const double2*>(arp)[0];
-    const double2 a23 = reinterpret_cast<const double2*>(arp)[1];
-    const struct { double x, y, z, w; } ar = {a01.x, a01.y, a23.x, a23.y};
-    double kf = xexp(ar.x + ar.y * logT - ar.z * invT);
+    Arg ka;  // ln kf
+    double b_rx = 0.0, th_rx = 0.0, dnu = 0.0;
+    if (!FX || JAC) {
+      const double2 a01 = reinterpret_cast<const double2*>(m.arr + 4 * i)[0];
+      const double2 a23 = reinterpret_cast<const double2*>(m.arr + 4 * i)[1];
+      b_rx = a01.y;
+      th_rx = a23.x;
+      dnu = a23.y;
+      if (!FX) ka = (Arg)(a01.x + a01.y * lgT - a23.x * invT);
+    }
+    if constexpr (FX) {
+      const longlong2 x01 = reinterpret_cast<const longlong2*>(m.arx + 4 * i)[0];
+      const long long x2 = m.arx[4 * i + 2];
+      ka = fx_clamp(x01.x + fx_mul(x01.y, LT) - fx_mul(x2, IT), 1100);
+    }
     const double Ca = c.C[sl.x];
     const double Cb = sl.y >= 0 ? c.C[sl.y] : 1.0;
     const double Cc = c.C[sl.z];
     const double Cd = sl.w >= 0 ? c.C[sl.w] : 1.0;
-    const double Pf = Ca * Cb, Pb = Cc * Cd;
-    // 1/Kc = exp(dG/RT) (Rc T/P0)^dnu with exp(dG/RT) from the species factors
-    // (formed here only where kr itself is needed: Jacobian data, large-|G/RT| path)
-    constexpr bool FAST = !JAC && !BIG;
-    double ratio = 0.0;
     const int rv = m.rev[i];
-    if (!FAST && (rv & 1)) {
-      if (!BIG) {
-        ratio = c.eg[sl.z] * c.ieg[sl.x];
-        if (sl.w >= 0) ratio *= c.eg[sl.w];
-        if (sl.y >= 0) ratio *= c.ieg[sl.y];
-        ratio *= (rv >> 1) == 2 ? cRT : (rv >> 1) == 0 ? icRT : 1.0;
-      } else {
-        double dg = c.ek[sl.z] - c.ek[sl.x];
-        if (sl.w >= 0) dg += c.ek[sl.w];
-        if (sl.y >= 0) dg -= c.ek[sl.y];
-        const double lc = logT + kLnRcP0;  // ln(Rc T / P0)
-        dg += (rv >> 1) == 2 ? lc : (rv >> 1) == 0 ? -lc : 0.0;
-        ratio = xexp(dg);
-      }
-    }
-    double Mc = 0.0, phi = 1.0;
-    double dk_dM = 0.0, dlnk = (ar.y + ar.z * invT) * invT, dk_dT = 0.0;
+    // factor of the mass-action rate: 1, [M], or [M] / (1 + Pr) (falloff)
+    double Mc = 0.0, phi = 1.0, red1 = 1.0;
+    double dlnk = (b_rx + th_rx * invT) * invT, gM = 1.0;  // d ln k/dT; d ln q/d ln[M]
     if (i >= m.i_tb0) {
       // efficiencies species-major: the warp's 32 reactions read one row per species
       const int r = i - m.i_tb0, ntb = m.n_tb;
@@ -1030,112 +1048,121 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
         const double* e = m.effT + r;
         for (int k = 0; k < K; ++k) Mc += e[(size_t)k * ntb] * c.C[k];
       }
-      if (i < m.i_fo0) phi = Mc;
+      phi = Mc;
     }
     if (i >= m.i_fo0) {
-      // fo[0..2] hold the low-pressure minus the high-pressure Arrhenius parameters,
-      // so one exponential gives k0 / kinf
+      // k = k0 F / (1 + Pr) [M] with Pr = (k0/kinf) [M]; the tables hold the low-pressure
+      // minus the high-pressure Arrhenius parameters, so ln k0 = ln kinf + fa
       const double* fo = m.fo + 8 * (i - m.i_fo0);
-      const double r0 = xexp(fo[0] + fo[1] * logT - fo[2] * invT);  // k0 / kinf
-      const double Pr = r0 * Mc;
-      double F = 1.0, dlgF_dL = 0.0, dlnF_dT = 0.0;
+      Arg fa;
+      if constexpr (FX) {
+        const long long* x = m.fox + 4 * (i - m.i_fo0);
+        fa = fx_clamp(x[0] + fx_mul(x[1], LT) - fx_mul(x[2], IT), 900);
+      } else {
+        fa = fo[0] + fo[1] * lgT - fo[2] * invT;
+      }
+      const double Pr = rate_exp<FX>(fa) * Mc;
+      red1 = xrcp(1.0 + Pr);
+      double dlgF_dL = 0.0, dlnF_dT = 0.0;
+      ka = ka + fa;
       if (i >= m.i_troe0) {
         const double alpha = fo[3];
         // fo[4] = 1/T***, fo[5] = 1/T*
-        const double e3 = xexp(-T * fo[4]), e1 = xexp(-T * fo[5]);
-        double Fc = (1.0 - alpha) * e3 + alpha * e1;
-        double dFc = -(1.0 - alpha) * fo[4] * e3 - alpha * fo[5] * e1;
-        if (fo[6] > 0.0) {
-          const double e2 = xexp(-fo[6] * invT);
-          Fc += e2;
-          dFc += fo[6] * invT * invT * e2;
+        const double x3 = -T * fo[4], x1 = -T * fo[5];
+        double e3, e1, e2 = 0.0;
+        if constexpr (FX) {
+          e3 = fx_exp(fx_from_double(x3));
+          e1 = fx_exp(fx_from_double(x1));
+          if (fo[6] > 0.0) e2 = fx_exp(fx_from_double(-fo[6] * invT));
+        } else {
+          e3 = xexp(x3);
+          e1 = xexp(x1);
+          if (fo[6] > 0.0) e2 = xexp(-fo[6] * invT);
         }
-        const double lF = xlog(Fc) * kInvLn10;
-        const double cc = -0.4 - 0.67 * lF, nn = 0.75 - 1.27 * lF;
-        const double x = xlog(Pr) * kInvLn10 + cc;
-        const double iden = xrcp(nn - 0.14 * x);
-        const double f1 = x * iden;
-        const double ig = xrcp(fma(f1, f1, 1.0));
-        const double lgF = lF * ig;
-        F = xexp(lgF * 2.302585092994046);  // 10^lgF
+        const double Fc = (1.0 - alpha) * e3 + alpha * e1 + e2;
+        const double lF = rate_log<FX>(Fc), lP = rate_log<FX>(Pr);  // natural logarithms
+        const double cc = fma(lF, -0.67 * kInvLn10, -0.4), nn = fma(lF, -1.27 * kInvLn10, 0.75);
+        const double x = fma(lP, kInvLn10, cc);
+        const double den = fma(x, -0.14, nn);
+        double lnF;
         if (JAC) {
+          const double iden = xrcp(den);
+          const double f1 = x * iden;
+          const double ig = xrcp(fma(f1, f1, 1.0));
+          lnF = lF * ig;
+          const double lgF = lnF * kInvLn10;
           // partial derivatives of log10 F by log10 Pr and by log10 Fc
           const double df1_dL = nn * iden * iden;
           const double df1_dlF = (-0.67 - f1 * (-1.27 + 0.14 * 0.67)) * iden;
           dlgF_dL = -2.0 * lgF * ig * f1 * df1_dL;
           const double dlgF_dlF = ig - 2.0 * lgF * ig * f1 * df1_dlF;
+          double dFc = -(1.0 - alpha) * fo[4] * e3 - alpha * fo[5] * e1;
+          if (fo[6] > 0.0) dFc += fo[6] * invT * invT * e2;
           dlnF_dT = dlgF_dlF * dFc * xrcp(Fc);  // d ln F / dT at fixed Pr
+        } else {
+          const double den2 = den * den;
+          lnF = lF * (den2 * xrcp(fma(x, x, den2)));
+        }
+        if constexpr (FX) {
+          ka = fx_clamp(ka, 1100) + fx_clamp(fx_from_double(lnF), 900);
+          if ((__double2hiint(lnF) & 0x7ff00000) == 0x7ff00000) red1 = lnF;  // NaN: no valid [M] or Fc
+        } else {
+          ka += lnF;
         }
       }
-      const double red1 = xrcp(1.0 + Pr);
-      const double kinf = kf;
-      kf = kinf * Pr * red1 * F;
+      phi = Mc * red1;
       if (JAC) {
-        // d ln k / d ln Pr = 1/(1 + Pr) + d log10 F / d log10 Pr; Pr = (k0/kinf) [M]
-        const double g = red1 + dlgF_dL;
-        dk_dM = kinf * red1 * F * g * r0;
-        dk_dT = kf * (dlnk + g * (fo[1] + fo[2] * invT) * invT + dlnF_dT);
+        gM = red1 + dlgF_dL;  // d ln k/d ln Pr
+        dlnk += gM * (fo[1] + fo[2] * invT) * invT + dlnF_dT;
       }
     }
-    const double kr = kf * ratio;
-    double net;
-    if constexpr (FAST) {
-      // kr Pb = kf c / (e_x e_y) (C_z e_z)(C_w e_w), e = exp(G/RT), c = (Rc T/P0)^dnu:
-      // q = kf (Pf - u rb) with u = c / (e_x e_y), rb = (C e)_z (C e)_w; plain
-      // third-body chunks multiply by [M], the other kinds (phi = 1) skip it
-      net = kf * Pf;
-      if (rv & 1) {
-        double ri = c.ieg[sl.x];
-        if (sl.y >= 0) ri *= c.ieg[sl.y];
-        double rb = c.dcp[sl.z];
-        if (sl.w >= 0) rb *= c.dcp[sl.w];
-        const double u = ri * ((rv >> 1) == 2 ? cRT : (rv >> 1) == 0 ? icRT : 1.0);
-        net = kf * fma(-u, rb, Pf);
-      }
-      c.q[i] = (i >= m.i_tb0 && i < m.i_fo0) ? phi * net : net;
+    const double kfP = rate_exp<FX>(ka);
+    double krP = 0.0;
+    if (rv & 1) {
+      Arg dg = g_RT[sl.z] - g_RT[sl.x];
+      if (sl.w >= 0) dg += g_RT[sl.w];
+      if (sl.y >= 0) dg -= g_RT[sl.y];
+      dg += (rv >> 1) == 2 ? lc : (rv >> 1) == 0 ? -lc : Arg(0);
+      if constexpr (FX) krP = fx_exp(fx_clamp(ka, 1100) + fx_clamp(dg, 900));
+      else krP = xexp(ka + dg);
+    }
+    const double Pf = Ca * Cb, Pb = Cc * Cd;
+    if constexpr (!JAC) {
+      const double net = fma(kfP, Pf, -krP * Pb);
+      c.q[i] = i >= m.i_tb0 ? phi * net : net;
     } else {
-      net = kf * Pf - kr * Pb;
-      c.q[i] = phi * net;
-    }
-    if (JAC) {
+      const double qf = kfP * Pf, qr = krP * Pb;
+      const double net = qf - qr;
+      c.q[i] = i >= m.i_tb0 ? phi * net : net;
       // d ln Kc / dT = dH/(R T^2) - dnu/T
-      double dH = c.hRT[sl.z] + (sl.w >= 0 ? c.hRT[sl.w] : 0.0) - c.hRT[sl.x] -
-                  (sl.y >= 0 ? c.hRT[sl.y] : 0.0);
-      const double dlnKc = (dH - ar.w) * invT;
-      double dq[4];
-      dq[0] = phi * kf * Cb;
-      dq[1] = sl.y >= 0 ? phi * kf * Ca : 0.0;
-      dq[2] = -phi * kr * Cd;
-      dq[3] = sl.w >= 0 ? -phi * kr * Cc : 0.0;
+      const double dH = c.hRT[sl.z] + (sl.w >= 0 ? c.hRT[sl.w] : 0.0) - c.hRT[sl.x] -
+                        (sl.y >= 0 ? c.hRT[sl.y] : 0.0);
+      const double dlnKc = (dH - dnu) * invT;
+      const double kfp = phi * kfP, krp = -phi * krP;
+      const double dq0 = kfp * Cb, dq1 = sl.y >= 0 ? kfp * Ca : 0.0;
+      const double dq2 = krp * Cd, dq3 = sl.w >= 0 ? krp * Cc : 0.0;
       if (FF) {
         // the float-float assembly's copy (hi, lo), split once here
         ff2* dqf = reinterpret_cast<ff2*>(c.dqs) + 4 * i;
-        dqf[0] = ff_split(dq[0]);
-        dqf[1] = sl.y >= 0 ? ff_split(dq[1]) : ff2{0.0f, 0.0f};
-        dqf[2] = ff_split(dq[2]);
-        dqf[3] = sl.w >= 0 ? ff_split(dq[3]) : ff2{0.0f, 0.0f};
+        dqf[0] = ff_split(dq0);
+        dqf[1] = ff_split(dq1);
+        dqf[2] = ff_split(dq2);
+        dqf[3] = ff_split(dq3);
       } else {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) c.dqs[4 * i + u] = dq[u];
+        c.dqs[4 * i] = dq0;
+        c.dqs[4 * i + 1] = dq1;
+        c.dqs[4 * i + 2] = dq2;
+        c.dqs[4 * i + 3] = dq3;
       }
-      double Dsum = Ca * dq[0] + (sl.y >= 0 ? Cb * dq[1] : 0.0) + Cc * dq[2] + (sl.w >= 0 ? Cd * dq[3] : 0.0);
-      double dtc, Pc;
-      if (i >= m.i_fo0) {
-        const double netc = Pf - ratio * Pb;
-        dtc = dk_dT * netc + ((rv & 1) ? kr * Pb * dlnKc : 0.0);
-        Pc = dk_dM * netc;
-      } else {
-        const double dkf = kf * dlnk;
-        const double dkr = kr * (dlnk - dlnKc);
-        dtc = phi * (dkf * Pf - dkr * Pb);
-        Pc = (i >= m.i_tb0) ? net : 0.0;
-      }
-      if (i >= m.i_tb0) Dsum += Mc * Pc;
-      c.dTc[i] = dtc;
+      c.dTc[i] = phi * fma(dlnk, net, qr * dlnKc);
+      const double Pc = i >= m.i_tb0 ? gM * red1 * net : 0.0;
       if (FF)
         reinterpret_cast<ff2*>(c.P)[i] = ff_split(Pc);
       else
         c.P[i] = Pc;
+      // sum_k C_k dq/dC_k: the mass-action orders, and [M]
+      double Dsum = phi * ((sl.y >= 0 ? 2.0 * qf : qf) - (sl.w >= 0 ? 2.0 * qr : qr));
+      if (i >= m.i_tb0) Dsum = fma(Mc, Pc, Dsum);
       c.D[i] = Dsum;
     }
   }
@@ -1193,15 +1220,15 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
 }
 
 template <int NW, bool JAC, bool FF>
-__device__ __noinline__ Scal eval_rhs_big(const DevMech& m, Cta<NW>& c, const double* y, double p, double* f) {
-  return eval_rhs_t<NW, JAC, FF, true>(m, c, y, p, f);
+__device__ __noinline__ Scal eval_rhs_fp64(const DevMech& m, Cta<NW>& c, const double* y, double p, double* f) {
+  return eval_rhs_t<NW, JAC, FF, false>(m, c, y, p, f);
 }
 
 // RHS (and with JAC the Jacobian data) of the state y; T = y[0] selects the path.
 template <int NW, bool JAC, bool FF = false>
 __device__ __forceinline__ Scal eval_rhs(const DevMech& m, Cta<NW>& c, const double* y, double p, double* f) {
-  if (y[0] < m.T_bigG) return eval_rhs_big<NW, JAC, FF>(m, c, y, p, f);
-  return eval_rhs_t<NW, JAC, FF, false>(m, c, y, p, f);
+  if (!(y[0] >= m.T_fx && y[0] < kFxThi)) return eval_rhs_fp64<NW, JAC, FF>(m, c, y, p, f);
+  return eval_rhs_t<NW, JAC, FF, true>(m, c, y, p, f);
 }
 
 // ---------------------------------------------------------------------------

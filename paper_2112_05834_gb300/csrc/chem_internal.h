@@ -13,9 +13,11 @@ constexpr int kMaxJobs = 8;
 constexpr double kRc = 8.31446261815324e7;  // erg / (mol K)
 constexpr double kP0 = 1.01325e6;           // dyn / cm^2, standard state (1 atm)
 constexpr double kTmin = 200.0, kTmax = 6000.0;
-// Largest |G/RT| of a species for which the reverse-rate ratio is formed as a product
-// of per-species factors exp(+-G/RT): four factors then stay within e^+-600.
-constexpr double kBigGRT = 150.0;
+// Range of the fixed-point rate evaluation (chem_fixed.cuh): T in [kTmin, kFxThi), and
+// |G/RT| of every species at most kFxGRT there, so that the sum of a reaction's four
+// stays inside the format's +-2048.
+constexpr double kFxThi = 8192.0;
+constexpr double kFxGRT = 400.0;
 
 // FP64: everything in FP64.
 // MIXED: Jacobian assembled in float-float arithmetic (about 48 bits, FP32 pipe; kept
@@ -57,7 +59,13 @@ struct DevMech {
   int i_tb0;  // first reaction of kind >= 1 (sorted order)
   int i_fo0;  // first reaction of kind >= 2
   int i_troe0;  // first reaction of kind 3
-  double T_bigG;  // below this T some species may have |G/RT| > kBigGRT (0: never in [kTmin, kTmax])
+  double T_fx;    // the fixed-point rate evaluation holds for T in [T_fx, kFxThi) (1e300: nowhere)
+  // Fixed-point tables (value v in Qn: round(v 2^n)); ln T enters as Q58, 1/T as Q71.
+  const long long* gfx;  // [K][16]: G/RT coefficients for range r at 8 r: constant (Q52), of ln T
+                         //   (Q58), of 1/T (Q45), of t, t^2, t^3, t^4 (Q52), t = T/2048 (r = 0)
+                         //   or T/8192 (r = 1)
+  const long long* arx;  // [I][4]: ln A (Q52), b (Q58), Ea_R (Q45), 0
+  const long long* fox;  // [n_fo][4]: the first three of fo in the same formats
   const double* W;      // [K]
   const double* invW;   // [K]
   const struct ff2* invW_ff;  // [K] as float-float pairs (hi, lo)
