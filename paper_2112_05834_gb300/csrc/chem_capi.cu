@@ -225,18 +225,25 @@ struct Pool {
 }  // namespace
 
 // v 2^q rounded to an integer; *ok is cleared when it does not stay inside the format.
-static long long to_fixed(long double v, int q, bool* ok) {
-  const long double s = std::ldexp(v, q);
-  if (!(std::fabs(s) < 9.2e18L)) {
+static long long to_fixed(double v, int q, bool* ok) {
+  const double s = std::ldexp(v, q);
+  if (!(std::fabs(s) < 9.2e18)) {
     *ok = false;
     return 0;
   }
   return (long long)std::llround(s);
 }
 
+// ln A in Q52: the double logarithm l, and the residual A / e^l - 1 that its rounding
+// (2^-48 for the usual prefactors) leaves.
+static long long fixed_log(double A, bool* ok) {
+  const double l = std::log(A);
+  return to_fixed(l, 52, ok) + to_fixed(A / std::exp(l) - 1.0, 52, ok);
+}
+
 // Largest |a + b ln T - c/T| over [kTmin, kFxThi), from above.
-static long double arrhenius_range(long double a, long double b, long double c) {
-  return std::fabs(a) + std::fabs(b) * 9.02L + std::fabs(c) / (long double)kTmin;
+static double arrhenius_range(double a, double b, double c) {
+  return std::fabs(a) + std::fabs(b) * 9.02 + std::fabs(c) / kTmin;
 }
 
 // The lowest temperature from which the fixed-point rate evaluation holds: |G/RT| of
@@ -247,16 +254,14 @@ static long double arrhenius_range(long double a, long double b, long double c) 
 static double fixed_point_temperature(const chem_mechanism_desc* d) {
   const double thr = kFxGRT - 10.0;
   double Tb = kTmin;
-  for (int k = 0; k < d->n_species; ++k) {
-    bool found = false;
-    for (double T = kFxThi; T >= kTmin; T -= 0.5) {
+  for (double T = kFxThi; T >= kTmin; T -= 0.5) {
+    const double lnT = std::log(T), iT = 1.0 / T;
+    for (int k = 0; k < d->n_species; ++k) {
       const double* a = (T < d->T_mid[k] ? d->nasa_lo : d->nasa_hi) + 7 * k;
-      const double hrt = h_RT(a, T);
-      if (!(std::fabs(hrt) < 20.0 * T)) return 1e300;
-      if (!found && std::fabs(hrt - s_R(a, T)) > thr) {
-        Tb = std::max(Tb, T + 0.5);
-        found = true;
-      }
+      const double h = a[0] + T * (a[1] / 2 + T * (a[2] / 3 + T * (a[3] / 4 + T * (a[4] / 5)))) + a[5] * iT;
+      const double sr = a[0] * lnT + T * (a[1] + T * (a[2] / 2 + T * (a[3] / 3 + T * (a[4] / 4)))) + a[6];
+      if (!(std::fabs(h) < 20.0 * T)) return 1e300;
+      if (std::fabs(h - sr) > thr) Tb = std::max(Tb, T + 0.5);
     }
   }
   return Tb;
@@ -292,53 +297,69 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
     }
     nasa[36 * k + 34] = d->T_mid[k];
   }
+  std::vector<double> hcp((size_t)20 * K);
+  for (int k = 0; k < K; ++k)
+    for (int r = 0; r < 2; ++r) {
+      const double* a = &nasa[36 * k + 17 * r];
+      double* o = &hcp[20 * k + 10 * r];
+      for (int j = 0; j < 5; ++j) o[j] = a[j];
+      for (int j = 0; j < 5; ++j) o[5 + j] = a[6 + j];
+    }
   // Each kind group is padded with null reactions to whole 32-reaction chunks, so a
   // warp's chunk never mixes kinds; chunks are dealt to warps by decreasing cost.
   std::vector<int> padded;
-  std::vector<double> chunk_cost;  // estimated time of one rate evaluation, in FP64 warp instructions (64 cycles)
+  int tb_chunks = 0;
+  std::vector<double> chunk_cost;  // estimated cycles of one rate evaluation
   for (int kind = 0; kind < 4; ++kind) {
     size_t first = padded.size();
     for (int i = 0; i < I; ++i)
       if (d->rxn_type[order[i]] == kind) padded.push_back(order[i]);
     if (padded.size() == first) continue;
     while (padded.size() % 32) padded.push_back(-1);
-    const double cost = kind == 0 ? 9.0 : kind == 1 ? 23.0 : kind == 2 ? 34.0 : 62.0;
+    const double cost = kind == 0 ? 1400.0 : kind == 1 ? 1600.0 : kind == 2 ? 2600.0 : 4500.0;
+    if (kind > 0) tb_chunks += (int)(padded.size() - first) / 32;
     for (size_t c = first; c < padded.size(); c += 32) chunk_cost.push_back(cost);
   }
   const int Ip = (int)padded.size();
   const int n_chunks = (int)chunk_cost.size();
-  // Deal the chunks to warps, longest first, each to the warp with the least estimated
-  // work so far; the species loops (thermo, production rates: ~45 per 32 species) load
-  // the warps holding species and the CTA's scalar work (~15) the last warp.
-  std::vector<int> by_cost(n_chunks);
-  std::iota(by_cost.begin(), by_cost.end(), 0);
-  std::stable_sort(by_cost.begin(), by_cost.end(), [&](int a, int b) { return chunk_cost[a] > chunk_cost[b]; });
-  std::vector<int> chunk_sched[3];
-  for (int v = 0; v < 3; ++v) {
-    const int NW = 2 << v, NT = 32 * NW;
-    std::vector<double> load(NW, 0.0);
-    for (int w = 0; w < NW; ++w) {
-      int cnt = 0;
-      for (int k = 0; k < K; ++k) cnt += (k % NT) / 32 == w;
-      load[w] = 45.0 * ((cnt + 31) / 32);
-    }
-    load[NW - 1] += 15.0;
+  // Deal the chunks to warps, longest first, each to the warp with the least estimated time
+  // so far; the scalar work of that phase (the mixture's cp) loads the last warp. The
+  // third-body sums run beside the species' thermodynamics, which load the species warps.
+  auto deal = [](const std::vector<double>& cost, std::vector<double> load) {
+    const int NW = (int)load.size();
+    std::vector<int> by_cost(cost.size());
+    std::iota(by_cost.begin(), by_cost.end(), 0);
+    std::stable_sort(by_cost.begin(), by_cost.end(), [&](int a, int b) { return cost[a] > cost[b]; });
     std::vector<std::vector<int>> own(NW);
     for (int ch : by_cost) {
       int w = 0;
       for (int u = 1; u < NW; ++u)
         if (load[u] < load[w]) w = u;
       own[w].push_back(ch);
-      load[w] += chunk_cost[ch];
+      load[w] += cost[ch];
     }
-    chunk_sched[v].assign(1, 0);
-    for (int w = 0; w < NW; ++w) chunk_sched[v].push_back(chunk_sched[v].back() + (int)own[w].size());
-    for (int w = 0; w < NW; ++w) chunk_sched[v].insert(chunk_sched[v].end(), own[w].begin(), own[w].end());
+    std::vector<int> sched(1, 0);
+    for (int w = 0; w < NW; ++w) sched.push_back(sched.back() + (int)own[w].size());
+    for (int w = 0; w < NW; ++w) sched.insert(sched.end(), own[w].begin(), own[w].end());
+    return sched;
+  };
+  std::vector<int> chunk_sched[3], tb_sched[3];
+  for (int v = 0; v < 3; ++v) {
+    const int NW = 2 << v;
+    std::vector<double> scalar(NW, 0.0), species(NW, 0.0);
+    scalar[NW - 1] = 1300.0;
+    for (int w = 0; w < NW; ++w) {
+      int cnt = 0;
+      for (int k = 0; k < K; ++k) cnt += (k % (32 * NW)) / 32 == w;
+      if (cnt > 0) species[w] = 1000.0 + 1800.0 * ((cnt + 31) / 32);
+    }
+    chunk_sched[v] = deal(chunk_cost, scalar);
+    tb_sched[v] = deal(std::vector<double>(tb_chunks, 14.0 * K + 250.0), species);
   }
   h->rxn_order = padded;
   std::vector<double> arr((size_t)4 * std::max(Ip, 1), 0.0), fo, eff;
-  std::vector<int4> slots(std::max(Ip, 1), make_int4(-1, -1, -1, -1));
-  std::vector<int> rev(std::max(Ip, 1), 0);
+  std::vector<long long> rx((size_t)4 * std::max(Ip, 1), 0);  // records of 32 bytes (DevMech::rx)
+  for (size_t i = 3; i < rx.size(); i += 4) rx[i] = 0xffffffffll;
   std::vector<std::vector<int2>> sp(K), tr(K);
   std::vector<std::vector<int4>> jr(K);
   int n_tb = 0, n_fo = 0, i_tb0 = Ip, i_fo0 = Ip, i_troe0 = Ip;
@@ -378,12 +399,14 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
         dnu += side ? nu[2 * o + s] : -nu[2 * o + s];
       }
     }
-    slots[i] = make_int4(sl[0], sl[1], sl[2], sl[3]);
+    unsigned packed = 0u;
+    for (int w = 0; w < 4; ++w) packed |= (unsigned)(sl[w] & 255) << (8 * w);
+    const int rev = (d->reversible[o] ? 1 : 0) | ((dnu + 1) << 1);
+    rx[4 * i + 3] = (long long)((unsigned long long)rev << 32 | packed);
     arr[4 * i + 0] = std::log(d->A[o]);
     arr[4 * i + 1] = d->b[o];
     arr[4 * i + 2] = d->Ea_R[o];
     arr[4 * i + 3] = (double)dnu;
-    rev[i] = (d->reversible[o] ? 1 : 0) | ((dnu + 1) << 1);
     if (t >= 1) {
       ++n_tb;
       for (int k = 0; k < K; ++k) eff.push_back(d->eff[(size_t)o * K + k]);
@@ -427,29 +450,28 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
   };
   // fixed-point copies for the rate evaluation; every argument has to stay inside +-2000
   bool fx_ok = true;
-  std::vector<long long> gfx((size_t)16 * K, 0), arx(arr.size(), 0), fox(fo.size() / 2, 0);
+  std::vector<long long> gfx((size_t)16 * K, 0), fox(fo.size() / 2, 0);
   for (int k = 0; k < K; ++k) {
     if (!(d->T_mid[k] <= 2048.0)) fx_ok = false;  // t = T/2048 below T_mid
     for (int r = 0; r < 2; ++r) {
       const double* a = (r == 0 ? d->nasa_lo : d->nasa_hi) + 7 * k;
       long long* o = &gfx[16 * k + 8 * r];
-      const long double S = r == 0 ? 2048.0L : 8192.0L;
+      const double S = r == 0 ? 2048.0 : 8192.0;
       // G/RT = (a1 - a7) - a1 ln T + a6/T - a2/2 T - a3/6 T^2 - a4/12 T^3 - a5/20 T^4
-      const long double c[4] = {-a[1] / 2.0L * S, -a[2] / 6.0L * S * S, -a[3] / 12.0L * S * S * S,
-                                -a[4] / 20.0L * S * S * S * S};
-      const long double c0 = (long double)a[0] - a[6];
+      const double c[4] = {-a[1] / 2.0 * S, -a[2] / 6.0 * S * S, -a[3] / 12.0 * S * S * S, -a[4] / 20.0 * S * S * S * S};
+      const double c0 = a[0] - a[6];
       if (!(arrhenius_range(c0, a[0], a[5]) + std::fabs(c[0]) + std::fabs(c[1]) + std::fabs(c[2]) + std::fabs(c[3]) <
-            2000.0L))
+            2000.0))
         fx_ok = false;
-      o[0] = to_fixed(c0, 52, &fx_ok) + 2;  // + 2: the mean of the products' truncations
-      o[1] = to_fixed(-(long double)a[0], 58, &fx_ok);
+      o[0] = to_fixed(a[0], 52, &fx_ok) - to_fixed(a[6], 52, &fx_ok) + 2;  // + 2: the mean of the products' truncations
+      o[1] = to_fixed(-a[0], 58, &fx_ok);
       o[2] = to_fixed(a[5], 45, &fx_ok);
       for (int j = 0; j < 4; ++j) o[3 + j] = to_fixed(c[j], 52, &fx_ok);
     }
   }
-  auto fix_arrhenius = [&](long double A, double b, double E, long long* o) {
-    if (!(arrhenius_range(A, b, E) < 2000.0L)) fx_ok = false;
-    o[0] = to_fixed(A, 52, &fx_ok);
+  auto fix_arrhenius = [&](long long lnA, double b, double E, long long* o) {
+    if (!(arrhenius_range(std::ldexp((double)lnA, -52), b, E) < 2000.0)) fx_ok = false;
+    o[0] = lnA;
     o[1] = to_fixed(b, 58, &fx_ok);
     o[2] = to_fixed(E, 45, &fx_ok);
   };
@@ -457,25 +479,51 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
     const int o = padded[i];
     const bool falloff = pkind[i] >= 2;
     if (o >= 0) {
-      const long double lnA = std::log((long double)d->A[o]);
-      fix_arrhenius(lnA, d->b[o], d->Ea_R[o], &arx[4 * i]);
+      const long long lnA = fixed_log(d->A[o], &fx_ok);
+      fix_arrhenius(lnA, d->b[o], d->Ea_R[o], &rx[4 * i]);
       if (falloff)
-        fix_arrhenius(std::log((long double)d->A0[o]) - lnA, d->b0[o] - d->b[o], d->Ea0_R[o] - d->Ea_R[o], &fox[4 * f]);
+        fix_arrhenius(fixed_log(d->A0[o], &fx_ok) - lnA, d->b0[o] - d->b[o], d->Ea0_R[o] - d->Ea_R[o], &fox[4 * f]);
     }
     if (falloff) ++f;
   }
-  std::vector<int> sp_ptr, tr_ptr;
-  std::vector<int2> sp_ent, tr_ent;
-  flatten2(sp, sp_ptr, sp_ent);
+  std::vector<int> tr_ptr;
+  std::vector<int2> tr_ent;
   flatten2(tr, tr_ptr, tr_ent);
+  // production sums: the largest power-of-two lane group per species that one pass allows
+  std::vector<unsigned short> ps_ent[3];
+  int ps_g[3], ps_passes[3], ps_quads[3];
+  for (int v = 0; v < 3; ++v) {
+    const int NT = 64 << v;
+    int g = 1;
+    while (g < 8 && 2 * g * K <= NT) g *= 2;
+    ps_g[v] = g;
+    ps_passes[v] = (K * g + NT - 1) / NT;
+    std::vector<std::vector<unsigned short>> own((size_t)ps_passes[v] * NT);
+    size_t rows = 1;
+    for (size_t t = 0; t < own.size(); ++t) {
+      const size_t k = t / g;
+      if (k >= (size_t)K) continue;
+      size_t pos = 0;
+      for (const int2& e : sp[k])
+        for (int c = 0; c < std::abs(e.y); ++c, ++pos)
+          if (pos % g == t % g) own[t].push_back((unsigned short)(e.x << 1 | (e.y < 0 ? 1 : 0)));
+      rows = std::max(rows, own[t].size());
+    }
+    const int q = (int)(rows + 3) / 4;
+    ps_quads[v] = q;
+    ps_ent[v].assign((size_t)ps_passes[v] * q * NT * 4, 0xffffu);
+    for (size_t t = 0; t < own.size(); ++t)
+      for (size_t r = 0; r < own[t].size(); ++r)
+        ps_ent[v][(((t / NT) * q + r / 4) * NT + t % NT) * 4 + r % 4] = own[t][r];
+  }
   // Mass-action Jacobian terms grouped by (row k, column j) pair in a fixed order,
   // then dealt to the threads of a CTA (longest pair first, to the thread with the
   // fewest terms so far, lowest thread on ties) for each block size.
-  const int U = (K + 31) / 32, ldm = (K + 1) | 1;
+  const int U = (K + 31) / 32;
   std::vector<unsigned> jmask((size_t)K * U, 0u);
   struct Pair {
     int k, j;
-    std::vector<int2> ents;  // (4 i + slot, nu_ki)
+    std::vector<unsigned> ents;  // (4 i + slot) << 1 | (nu_ki < 0), |nu_ki| times
   };
   std::vector<Pair> pairs;
   for (int k = 0; k < K; ++k) {
@@ -483,7 +531,9 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
     std::stable_sort(ents.begin(), ents.end(), [](const int4& a, const int4& b) { return a.x < b.x; });
     for (size_t e = 0; e < ents.size();) {
       Pair pr{k, ents[e].x, {}};
-      for (; e < ents.size() && ents[e].x == pr.j; ++e) pr.ents.push_back(make_int2(4 * ents[e].y + ents[e].w, ents[e].z));
+      for (; e < ents.size() && ents[e].x == pr.j; ++e) 
+        for (int c = 0; c < std::abs(ents[e].z); ++c)
+          pr.ents.push_back((unsigned)(4 * ents[e].y + ents[e].w) << 1 | (ents[e].z < 0 ? 1u : 0u));
       jmask[(size_t)k * U + pr.j / 32] |= 1u << (pr.j % 32);
       pairs.push_back(std::move(pr));
     }
@@ -492,8 +542,7 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
   std::iota(by_len.begin(), by_len.end(), 0);
   std::stable_sort(by_len.begin(), by_len.end(),
                    [&](int a, int b) { return pairs[a].ents.size() > pairs[b].ents.size(); });
-  std::vector<int2> js_ent[3];
-  std::vector<double> js_nu[3];
+  std::vector<uint2> js_ent[3];
   int js_rounds[3];
   for (int v = 0; v < 3; ++v) {
     const int NT = 64 << v;
@@ -506,25 +555,24 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
       own[t].push_back(q);
       load[t] += (int)pairs[q].ents.size();
     }
-    const int R = std::max(1, *std::max_element(load.begin(), load.end()));
+    const int R = (std::max(1, *std::max_element(load.begin(), load.end())) + 3) & ~3;
     js_rounds[v] = R;
-    js_ent[v].assign((size_t)R * NT, make_int2(-1, -1));
-    js_nu[v].assign((size_t)R * NT, 0.0);
+    js_ent[v].assign((size_t)R * NT, make_uint2(~0u, ~0u));
     for (int t = 0; t < NT; ++t) {
       int r = 0;
       for (int q : own[t]) {
         const Pair& pr = pairs[q];
         for (size_t e = 0; e < pr.ents.size(); ++e, ++r) {
           const bool last = e + 1 == pr.ents.size();
-          js_ent[v][(size_t)r * NT + t] = make_int2(pr.ents[e].x, last ? (1 + pr.k) * ldm + 1 + pr.j : -1);
-          js_nu[v][(size_t)r * NT + t] = pr.ents[e].y * d->W[pr.k];
+          js_ent[v][(size_t)r * NT + t] = make_uint2(pr.ents[e], last ? (unsigned)(pr.k << 8 | pr.j) : ~0u);
         }
       }
     }
   }
 
-  std::vector<double> sp_nu(sp_ent.size()), tr_nu(tr_ent.size());
-  for (size_t e = 0; e < sp_ent.size(); ++e) sp_nu[e] = sp_ent[e].y;
+  std::vector<double> tr_nu(tr_ent.size());
+  std::vector<int> tr_row(tr_ent.size() + 3, 0);
+  for (size_t e = 0; e < tr_ent.size(); ++e) tr_row[e] = (tr_ent[e].x - i_tb0) * K;
   for (int k = 0; k < K; ++k)
     for (int e = tr_ptr[k]; e < tr_ptr[k + 1]; ++e) tr_nu[e] = tr_ent[e].y * d->W[k];
   // float-float (hi, lo) copies of the constants the mixed form's assembly multiplies by
@@ -537,35 +585,33 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
     }
     return o;
   };
-  const std::vector<float> eff_ff = split(eff), invW_ff = split(invW), tr_nu_ff = split(tr_nu);
+  const std::vector<float> eff_ff = split(eff), invW_ff = split(invW), W_ff = split(W), tr_nu_ff = split(tr_nu);
   // the efficiencies species-major as well: the rate evaluation's [M] sums read one
   // species for 32 consecutive reactions at a time (coalesced), the assembly one
   // reaction for 32 consecutive species
-  std::vector<double> effT(eff.size());
+  std::vector<double> effT(eff.size() + (size_t)8 * n_tb, 0.0);  // + 8 rows that the batched loads may reach
   for (int r = 0; r < n_tb; ++r)
     for (int k = 0; k < K; ++k) effT[(size_t)k * n_tb + r] = eff[(size_t)r * K + k];
   const std::vector<float> effT_ff = split(effT);
-  std::vector<float> js_nu_ff[3];
-  for (int v = 0; v < 3; ++v) js_nu_ff[v] = split(js_nu[v]);
   Pool P;
   const size_t oW = P.add(W.data(), W.size() * 8), oiW = P.add(invW.data(), invW.size() * 8),
                oN = P.add(nasa.data(), nasa.size() * 8), oA = P.add(arr.data(), arr.size() * 8),
-               oS = P.add(slots.data(), slots.size() * sizeof(int4)), oR = P.add(rev.data(), rev.size() * 4),
+               oR = P.add(rx.data(), rx.size() * 8),
                oF = P.add(fo.data(), fo.size() * 8), oE = P.add(eff.data(), eff.size() * 8),
-               oSp = P.add(sp_ptr.data(), sp_ptr.size() * 4), oSe = P.add(sp_ent.data(), sp_ent.size() * 8),
                oTp = P.add(tr_ptr.data(), tr_ptr.size() * 4), oTe = P.add(tr_ent.data(), tr_ent.size() * 8),
-               oSn = P.add(sp_nu.data(), sp_nu.size() * 8), oTn = P.add(tr_nu.data(), tr_nu.size() * 8),
+               oTn = P.add(tr_nu.data(), tr_nu.size() * 8),
                oJm = P.add(jmask.data(), jmask.size() * 4),
                oEf = P.add(eff_ff.data(), eff_ff.size() * 4), oiWf = P.add(invW_ff.data(), invW_ff.size() * 4),
                oEt = P.add(effT.data(), effT.size() * 8), oEtf = P.add(effT_ff.data(), effT_ff.size() * 4),
                oTnf = P.add(tr_nu_ff.data(), tr_nu_ff.size() * 4), oGx = P.add(gfx.data(), gfx.size() * 8),
-               oAx = P.add(arx.data(), arx.size() * 8), oFx = P.add(fox.data(), fox.size() * 8);
-  size_t oJe[3], oJn[3], oJnf[3], oCs[3];
+               oFx = P.add(fox.data(), fox.size() * 8), oHc = P.add(hcp.data(), hcp.size() * 8), oWf = P.add(W_ff.data(), W_ff.size() * 4), oTr = P.add(tr_row.data(), tr_row.size() * 4),
+               oTm = P.add(d->T_mid, (size_t)K * 8);
+  size_t oJe[3], oCs[3], oTs[3], oPe[3];
   for (int v = 0; v < 3; ++v) {
     oCs[v] = P.add(chunk_sched[v].data(), chunk_sched[v].size() * 4);
-    oJe[v] = P.add(js_ent[v].data(), js_ent[v].size() * sizeof(int2));
-    oJn[v] = P.add(js_nu[v].data(), js_nu[v].size() * 8);
-    oJnf[v] = P.add(js_nu_ff[v].data(), js_nu_ff[v].size() * 4);
+    oTs[v] = P.add(tb_sched[v].data(), tb_sched[v].size() * 4);
+    oPe[v] = P.add(ps_ent[v].data(), ps_ent[v].size() * 2);
+    oJe[v] = P.add(js_ent[v].data(), js_ent[v].size() * sizeof(uint2));
   }
   CHEM_CUDA(h, cudaMalloc(&h->d_tables, P.host.size()));
   CHEM_CUDA(h, cudaMemcpy(h->d_tables, P.host.data(), P.host.size(), cudaMemcpyHostToDevice));
@@ -582,34 +628,36 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
   m.i_troe0 = i_troe0;
   m.T_fx = fx_ok ? fixed_point_temperature(d) : 1e300;
   m.gfx = reinterpret_cast<const long long*>(b + oGx);
-  m.arx = reinterpret_cast<const long long*>(b + oAx);
+  m.hcp = reinterpret_cast<const double2*>(b + oHc);
+  m.T_mid = reinterpret_cast<const double*>(b + oTm);
   m.fox = reinterpret_cast<const long long*>(b + oFx);
   m.W = reinterpret_cast<const double*>(b + oW);
   m.invW = reinterpret_cast<const double*>(b + oiW);
   m.nasa = reinterpret_cast<const double*>(b + oN);
   m.arr = reinterpret_cast<const double*>(b + oA);
-  m.slots = reinterpret_cast<const int4*>(b + oS);
-  m.rev = reinterpret_cast<const int*>(b + oR);
+  m.rx = reinterpret_cast<const longlong2*>(b + oR);
   m.fo = reinterpret_cast<const double*>(b + oF);
   m.eff = reinterpret_cast<const double*>(b + oE);
-  m.sp_ptr = reinterpret_cast<const int*>(b + oSp);
-  m.sp_ent = reinterpret_cast<const int2*>(b + oSe);
   m.tr_ptr = reinterpret_cast<const int*>(b + oTp);
   m.tr_ent = reinterpret_cast<const int2*>(b + oTe);
-  m.sp_nu = reinterpret_cast<const double*>(b + oSn);
   m.tr_nu = reinterpret_cast<const double*>(b + oTn);
   m.eff_ff = reinterpret_cast<const chem::ff2*>(b + oEf);
   m.effT = reinterpret_cast<const double*>(b + oEt);
   m.effT_ff = reinterpret_cast<const chem::ff2*>(b + oEtf);
   m.invW_ff = reinterpret_cast<const chem::ff2*>(b + oiWf);
+  m.W_ff = reinterpret_cast<const chem::ff2*>(b + oWf);
+  m.tr_row = reinterpret_cast<const int*>(b + oTr);
   m.tr_nu_ff = reinterpret_cast<const chem::ff2*>(b + oTnf);
   m.jmask = reinterpret_cast<const unsigned*>(b + oJm);
   for (int v = 0; v < 3; ++v) {
-    m.js_ent[v] = reinterpret_cast<const int2*>(b + oJe[v]);
-    m.js_nu[v] = reinterpret_cast<const double*>(b + oJn[v]);
-    m.js_nu_ff[v] = reinterpret_cast<const chem::ff2*>(b + oJnf[v]);
+    m.js_ent[v] = reinterpret_cast<const uint2*>(b + oJe[v]);
     m.js_rounds[v] = js_rounds[v];
     m.chunk_sched[v] = reinterpret_cast<const int*>(b + oCs[v]);
+    m.tb_sched[v] = reinterpret_cast<const int*>(b + oTs[v]);
+    m.ps_ent[v] = reinterpret_cast<const uint2*>(b + oPe[v]);
+    m.ps_quads[v] = ps_quads[v];
+    m.ps_g[v] = ps_g[v];
+    m.ps_passes[v] = ps_passes[v];
   }
   return CHEM_OK;
 }
@@ -880,7 +928,7 @@ chem_status chem_internal_integrate(const chem_job* jobs, int32_t n_jobs, double
   // the mixed form may keep its assembled matrix in global memory on persistent grids when
   // that lets more CTAs share an SM (large mechanisms)
   const bool m0g_ok = h0->precision == PREC_MIXED && a.sched != SCHED_PLAIN;
-  int block = h0->block ? h0->block : chem_internal_pick_block(h0, a.smem_K, a.smem_I, m0g_ok);
+  int block = h0->block ? h0->block : chem_internal_pick_block(h0, a.smem_K, a.smem_I, a.n_total, m0g_ok);
   int tuned_ctas = 0, tuned_m0g = -1;  // the autotuner's resident CTAs per SM and matrix layout
   if (h0->autotune) {
     s = chem_internal_autotune(h0, a, st, &block, &tuned_ctas, &tuned_m0g);
@@ -910,8 +958,7 @@ chem_status chem_internal_integrate(const chem_job* jobs, int32_t n_jobs, double
     if (h0->ctas_per_sm > 0) occ = std::min(occ, h0->ctas_per_sm);
     grid = (int)std::min<int64_t>(total, (int64_t)occ * h0->num_sms);
     if (m0g) {
-      const int nmax = a.smem_K + 1;
-      const int64_t stride = (int64_t)nmax * (nmax | 1);
+      const int64_t stride = matrix_slot_entries(a.smem_K);
       const size_t bytes = (size_t)grid * stride * sizeof(double);
       if (bytes > h0->m0_cap) {
         cudaStreamSynchronize(st);
@@ -950,26 +997,23 @@ chem_status chem_internal_integrate(const chem_job* jobs, int32_t n_jobs, double
   return CHEM_OK;
 }
 
-// Block size with the most resident warps per SM for this mechanism size and
-// precision (ties: 128, then 64, then 256 threads).
-int chem_internal_pick_block(chem_handle h, int K, int I, bool allow_m0_global) {
-  int best = 128, best_w = -1;
-  for (int b : {128, 64, 256}) {
+// Threads per cell. The work of a cell lies in loops over its n = K + 1 entries and its
+// 32-reaction chunks, so the CTA grows with n: 64 threads up to n = 32, 128 up to n = 64
+// (the sizes of the register Gauss-Jordan), 256 beyond. A launch with at most one cell per
+// SM has no other cells to fill the SM, and takes twice the threads per cell.
+int chem_internal_pick_block(chem_handle h, int K, int I, int64_t n_cells, bool allow_m0_global) {
+  const int n = K + 1;
+  int best = n <= 32 ? 64 : n <= 64 ? 128 : 256;
+  if (n_cells <= h->num_sms) best = std::min(256, 2 * best);
+  // the preferred size first, then any that fits an SM
+  for (int b : {best, 128, 64, 256}) {
     int occ = 0;
-    if (occupancy_integrate(b, h->precision, K, I, &occ) != cudaSuccess) {
-      cudaGetLastError();
-      continue;
-    }
-    int occ_g = 0;
-    if (allow_m0_global && occupancy_integrate(b, h->precision, K, I, &occ_g, true) == cudaSuccess)
-      occ = std::max(occ, occ_g);
+    if (occupancy_integrate(b, h->precision, K, I, &occ) == cudaSuccess && occ > 0) return b;
+    if (allow_m0_global && occupancy_integrate(b, h->precision, K, I, &occ, true) == cudaSuccess && occ > 0) return b;
     cudaGetLastError();
-    if (occ * b / 32 > best_w) {
-      best_w = occ * b / 32;
-      best = b;
-    }
   }
-  return best;
+  cudaGetLastError();
+  return 128;
 }
 
 // Launch (optionally through a cached CUDA graph).

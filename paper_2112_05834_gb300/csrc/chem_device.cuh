@@ -630,18 +630,19 @@ __device__ __forceinline__ double xlog(double x) {
   return t + fma(md, kLn2Lo, __ldg(e + 2) + l1p);
 }
 
-// 1/x by Newton's iteration r <- r + r (1 - x r) from the hardware's approximate
-// reciprocal (two steps take its error below one ulp); magnitudes outside
+// 1/x from the hardware's approximate reciprocal r (relative error below 2^-20) by one
+// cubic step r <- r + r (e + e^2), e = 1 - x r, whose truncation e^3 is below 2^-60: three
+// dependent FP64 instructions, where two Newton steps take four; magnitudes outside
 // [2^-1000, 2^1000], zero, infinities and NaN take the IEEE division.
+static __device__ __noinline__ double rcp_outside(double x) { return 1.0 / x; }
+
 __device__ __forceinline__ double xrcp(double x) {
   const int ex = (__double2hiint(x) >> 20) & 0x7ff;
-  if (ex < 23 || ex > 2023) return 1.0 / x;
+  if (ex < 23 || ex > 2023) return rcp_outside(x);
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  double e = fma(-x, r, 1.0);
-  r = fma(r, e, r);
-  e = fma(-x, r, 1.0);
-  return fma(r, e, r);
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
 }
 
 
@@ -676,6 +677,19 @@ struct Meth<METHOD_ROS34PW2> {
   __device__ static double e(const IntegrateArgs& g, int j) { return g.tab.e[j]; }
 };
 
+// Loads of tables that stream through once per step: they do not displace the rate
+// evaluation's tables, which every right-hand side reads, from the L1 cache.
+__device__ __forceinline__ uint2 ld_stream(const uint2* p) {
+  uint2 v;
+  asm("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ ff2 ld_stream(const ff2* p) {
+  ff2 v;
+  asm("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.hi), "=f"(v.lo) : "l"(p));
+  return v;
+}
+
 // Precision policy: LU = type of the factorised matrix, ASM = type the Jacobian is
 // assembled in; IR = refine each solve against the assembled matrix.
 template <int PREC>
@@ -703,30 +717,38 @@ struct Policy<PREC_FP32ASM> {
 struct Layout {
   int nmax, ld;            // matrix dimension bound and leading dimension (odd)
   int Kmax, Imax;
-  size_t off_vec, off_sp, off_rx, off_M, off_M0, off_piv, off_red, total;
+  size_t off_vec, off_M, off_M0, off_piv, total;
+  bool x_tab;
 };
 
 __host__ __device__ inline int odd_ld(int n) { return n | 1; }
+// 8-byte entries of a CTA's global-memory slot: the matrix by columns and the mass-action sums
+__host__ __device__ inline int slot_ld(int n) { return (n + 7) & ~3; }
+__host__ __device__ inline size_t slot_entries(int K) {
+  return ((size_t)(K + 1) * slot_ld(K + 1) + (size_t)K * K + 3) & ~(size_t)3;
+}
 
 // vectors (double): y, yn, ys, f0, fv, rr, u[6], sc  -> 13 n
-// species (8 bytes): C, hRT, cpR, g, dcp, dk, akT, ek -> 8 K
+// species (8 bytes): C, hRT, cpR, g, dcp, dk, akT, ek, 1/W -> 9 K
 // reactions (double): q, D, dTc, P, dqs[4] -> 8 I
 // m0_global: the mixed form's assembled matrix lives in a global-memory slot of
 // the CTA instead of shared memory (large mechanisms, persistent schedulers).
-__host__ __device__ inline Layout make_layout(int Kmax, int Imax, int prec, bool m0_global = false) {
+// want_xt: the exponential's table (2 KB) in shared memory, where that still fits.
+constexpr size_t kMaxSmem = 227 * 1024;
+__host__ __device__ inline Layout make_layout(int Kmax, int Imax, int prec, bool m0_global = false,
+                                              bool want_xt = false) {
   Layout L;
   L.nmax = Kmax + 1;
   L.ld = odd_ld(L.nmax);
   L.Kmax = Kmax;
   L.Imax = Imax;
   size_t o = 0;
-  L.off_red = o;
   o += 64 * sizeof(double);
+  L.x_tab = want_xt;
+  if (want_xt) o += 256 * sizeof(double);
   L.off_vec = o;
   o += (size_t)13 * L.nmax * sizeof(double);
-  L.off_sp = o;
-  o += (size_t)8 * Kmax * sizeof(double);
-  L.off_rx = o;
+  o += (size_t)9 * Kmax * sizeof(double);
   if (prec == PREC_FP64) {
     o += (size_t)8 * Imax * sizeof(double);
     L.off_M = o;
@@ -749,71 +771,122 @@ __host__ __device__ inline Layout make_layout(int Kmax, int Imax, int prec, bool
   o += (size_t)L.nmax * sizeof(double);   // inverse diagonal of U
   o = (o + 15) & ~(size_t)15;
   L.total = o;
-  return L;
+  return want_xt && o > kMaxSmem ? make_layout(Kmax, Imax, prec, m0_global) : L;
 }
 
 
 // Scalars kept in the reduction area (its first 32 slots are unused).
 // SC_OUT: 8 broadcast results of Cta::reduce; SC_PIV: pivot search slots (12 NW bytes)
 // (SC_INVT during the rate evaluation, SC_INVP during the LU: never live together)
-enum { SC_OUT = 32, SC_LOGT = 48, SC_INVT = 49, SC_INVP = 49, SC_FLAG = 50, SC_MISC = 51, SC_PIV = 52 };
+enum { SC_OUT = 32, SC_LOGT = 48, SC_INVT = 49, SC_INVP = 49, SC_ICPM = 50, SC_DCPM = 51, SC_PIV = 52 };
+
+// A CTA's view of its shared memory. Arrays are functions of a few 32-bit sizes, so that
+// an address is one or two integer instructions and a shared-memory access: as stored
+// pointers they would take 60 registers, or local memory.
+extern __shared__ __align__(16) unsigned char smem[];
 
 template <int NW>
 struct Cta {
   static constexpr int NT = NW * 32;
   static constexpr int SW = NW - 1;  // the warp that computes CTA scalars (ln T, 1/T, the FP64 solve)
   int tid, lane, warp;
-  double* red;
-  // vectors
-  double *y, *yn, *ys, *f0, *fv, *rr, *u, *sc;
-  // species
-  double *C, *hRT, *cpR, *g, *dcp, *dk, *akT, *ek;
-  // reactions
-  double *q, *D, *dTc, *P, *dqs;
-  void* M;
-  void* M0;
-  int *piv, *perm;
-  double* invd;
+  unsigned vec, n8, k8, i8, off_M, off_piv;  // byte offsets; bytes of n, K and I 8-byte entries
+  bool x_tab;
+  void* M0;     // mixed forms: the assembled matrix by columns, entry (i, j) at j ld0 + i0 + i
+  int ld0, i0;
+  int Km;       // species of the mechanism the matrix geometry is set for
+  double p_rc, rc_p;  // p/Rc and Rc/p of the cell
 
-  __device__ void bind(unsigned char* base, const Layout& L) {
+  __device__ __forceinline__ static double* at(unsigned off) { return reinterpret_cast<double*>(smem + off); }
+  __device__ __forceinline__ double* red() const { return at(0); }
+  // vectors of n
+  __device__ __forceinline__ double* y() const { return at(vec); }
+  __device__ __forceinline__ double* yn() const { return at(vec + n8); }
+  __device__ __forceinline__ double* ys() const { return at(vec + 2 * n8); }
+  __device__ __forceinline__ double* f0() const { return at(vec + 3 * n8); }
+  __device__ __forceinline__ double* fv() const { return at(vec + 4 * n8); }
+  __device__ __forceinline__ double* rr() const { return at(vec + 5 * n8); }
+  __device__ __forceinline__ double* u() const { return at(vec + 6 * n8); }  // 6 n
+  __device__ __forceinline__ double* sc() const { return at(vec + 12 * n8); }
+  // species
+  __device__ __forceinline__ unsigned sp(int a) const { return vec + 13 * n8 + a * k8; }
+  __device__ __forceinline__ double* C() const { return at(sp(0)); }
+  __device__ __forceinline__ double* hRT() const { return at(sp(1)); }
+  __device__ __forceinline__ double* cpR() const { return at(sp(2)); }
+  __device__ __forceinline__ double* g() const { return at(sp(3)); }
+  __device__ __forceinline__ double* dcp() const { return at(sp(4)); }
+  __device__ __forceinline__ double* dk() const { return at(sp(5)); }
+  __device__ __forceinline__ double* akT() const { return at(sp(6)); }
+  __device__ __forceinline__ double* ek() const { return at(sp(7)); }
+  __device__ __forceinline__ double* iW() const { return at(sp(8)); }
+  // reactions
+  __device__ __forceinline__ double* q() const { return at(sp(9)); }
+  __device__ __forceinline__ double* D() const { return at(sp(9) + i8); }
+  __device__ __forceinline__ double* dTc() const { return at(sp(9) + 2 * i8); }
+  __device__ __forceinline__ double* P() const { return at(sp(9) + 3 * i8); }
+  __device__ __forceinline__ double* dqs() const { return at(sp(9) + 4 * i8); }
+  __device__ __forceinline__ void* M() const { return smem + off_M; }
+  __device__ __forceinline__ int* piv() const { return reinterpret_cast<int*>(smem + off_piv); }
+  __device__ __forceinline__ int* perm() const { return reinterpret_cast<int*>(smem + off_piv + n8 / 2); }
+  __device__ __forceinline__ double* invd() const { return at(off_piv + n8); }
+  // the exponential's table
+  __device__ __forceinline__ const unsigned long long* xt() const {
+    return x_tab ? reinterpret_cast<const unsigned long long*>(smem + 64 * sizeof(double)) : g_fx_exp_tab;
+  }
+  // float-float assembly: mass-action sum (k, j), see set_matrix
+  __device__ __forceinline__ ff2& pair(int k, int j) const {
+    ff2* a = reinterpret_cast<ff2*>(M0);
+    return i0 ? a[(size_t)(Km + 1) * ld0 + k * Km + j] : a[(1 + j) * ld0 + 1 + k];
+  }
+
+  __device__ void bind(const Layout& L) {
     tid = threadIdx.x;
     lane = tid & 31;
     warp = tid >> 5;
-    red = reinterpret_cast<double*>(base + L.off_red);
-    double* v = reinterpret_cast<double*>(base + L.off_vec);
-    const int n = L.nmax;
-    y = v;
-    yn = v + n;
-    ys = v + 2 * n;
-    f0 = v + 3 * n;
-    fv = v + 4 * n;
-    rr = v + 5 * n;
-    u = v + 6 * n;   // 6 n
-    sc = v + 12 * n;
-    double* s = reinterpret_cast<double*>(base + L.off_sp);
-    const int K = L.Kmax;
-    C = s;
-    hRT = s + K;
-    cpR = s + 2 * K;
-    g = s + 3 * K;
-    dcp = s + 4 * K;
-    dk = s + 5 * K;
-    akT = s + 6 * K;
-    ek = s + 7 * K;
-    double* r = reinterpret_cast<double*>(base + L.off_rx);
-    const int I = L.Imax;
-    q = r;
-    D = r + I;
-    dTc = r + 2 * I;
-    P = r + 3 * I;
-    dqs = r + 4 * I;
-    M = base + L.off_M;
-    M0 = base + L.off_M0;
-    piv = reinterpret_cast<int*>(base + L.off_piv);
-    perm = piv + L.nmax;
-    invd = reinterpret_cast<double*>(perm + L.nmax);
+    vec = (unsigned)L.off_vec;
+    n8 = 8 * L.nmax;
+    k8 = 8 * L.Kmax;
+    i8 = 8 * L.Imax;
+    off_M = (unsigned)L.off_M;
+    off_piv = (unsigned)L.off_piv;
+    M0 = smem + L.off_M0;
+    ld0 = L.ld;
+    i0 = 0;
+    Km = L.Kmax;
+    x_tab = L.x_tab;
+    if (x_tab) {
+      unsigned long long* t = reinterpret_cast<unsigned long long*>(smem + 64 * sizeof(double));
+#pragma unroll 1
+      for (int i = tid; i < 256; i += NT) t[i] = g_fx_exp_tab[i];
+      __syncthreads();
+    }
   }
 
+  // The mechanism's matrix geometry. In the CTA's global-memory slot (slot != null) a
+  // column starts at a 32-byte boundary for row 1, so that four rows of a column are one
+  // sector, and the mass-action sums have rows of their own behind the matrix; in shared
+  // memory the odd leading dimension avoids bank conflicts and the sums take the places of
+  // the finished entries.
+  __device__ void set_matrix(int K, double* slot) {
+    Km = K;
+    if (slot) {
+      ld0 = slot_ld(K + 1);
+      i0 = 3;
+      M0 = slot;
+    } else {
+      ld0 = odd_ld(K + 1);
+      i0 = 0;
+    }
+  }
+
+  // A cell's pressure and the mechanism's 1/W, which every rate evaluation reads (from
+  // shared memory: the tables' L1 lines are evicted between evaluations).
+  __device__ void set_cell(const DevMech& m, double p) {
+    p_rc = p / kRc;
+    rc_p = kRc / p;
+#pragma unroll 1
+    for (int k = tid; k < m.K; k += NT) iW()[k] = m.invW[k];
+  }
 
   // Sum of NV (1, 2 or 4) values over the CTA; every thread receives the same
   // totals (fixed summation order: deterministic). Only the first nw warps may hold
@@ -851,11 +924,12 @@ struct Cta {
           x = (h8 ? x2 : x) + __shfl_xor_sync(FULLMASK, h8 ? x : x2, 8);
         }
       }
-      if (warp > 0) sc[(warp - 1) * 32 + lane] = x;
+      if (warp > 0) sc()[(warp - 1) * 32 + lane] = x;
     }
     __syncthreads();
     if (warp == 0) {
-      for (int w = 1; w < nw; ++w) x += sc[(w - 1) * 32 + lane];
+#pragma unroll 1
+      for (int w = 1; w < nw; ++w) x += sc()[(w - 1) * 32 + lane];
 #pragma unroll
       for (int o = 16 >> LV; o; o >>= 1) x += __shfl_xor_sync(FULLMASK, x, o);
       double tot[NV];
@@ -869,12 +943,12 @@ struct Cta {
       fin(tot, o);
       if (lane == 0) {
 #pragma unroll
-        for (int b = 0; b < NO; ++b) red[SC_OUT + b] = o[b];
+        for (int b = 0; b < NO; ++b) red()[SC_OUT + b] = o[b];
       }
     }
     __syncthreads();
 #pragma unroll
-    for (int b = 0; b < NO; ++b) out[b] = red[SC_OUT + b];
+    for (int b = 0; b < NO; ++b) out[b] = red()[SC_OUT + b];
   }
 
   // Plain CTA sum of NV values (nw as in reduce).
@@ -896,7 +970,7 @@ __device__ __forceinline__ int warps_for(int count) {
 
 // Cell-level scalars shared by all threads of the CTA (identical in every thread).
 struct Scal {
-  double T, invT, rho, irho, Wbar, cpm, icpm, fT, dcpm, Scpw;
+  double T, invT, rho, irho, Wbar, icpm, fT, dcpm, Scpw;
 };
 
 // ---------------------------------------------------------------------------
@@ -916,8 +990,9 @@ struct Scal {
 // FF (the forms with FP32 factors): the third-body sums [M] in float-float, and the
 // slot derivatives and P stored as float-float pairs for the assembly.
 template <bool FX>
-__device__ __forceinline__ double rate_exp(typename std::conditional<FX, long long, double>::type a) {
-  if constexpr (FX) return fx_exp(a);
+__device__ __forceinline__ double rate_exp(typename std::conditional<FX, long long, double>::type a,
+                                           const unsigned long long* tab) {
+  if constexpr (FX) return fx_exp(a, tab);
   else return xexp(a);
 }
 template <bool FX>
@@ -925,10 +1000,26 @@ __device__ __forceinline__ double rate_log(double x) {
   if constexpr (FX) {
     const int hx = __double2hiint(x);
     if (hx < 0x00100000 || hx >= 0x7ff00000) return log_outside(x);
-    return fx_to_double(fx_log<52>(x));
+    return fx_to_double(fx_log(x, 52));
   } else {
     return xlog(x);
   }
+}
+
+// One reaction's record: Arrhenius parameters in fixed point (Q52, Q58, Q45), species
+// slots (reactants, products; 255 = empty), rev (DevMech::rx).
+struct RxRec {
+  long long lnA, b, th;
+  unsigned slots;
+  int rev;
+};
+__device__ __forceinline__ RxRec load_rec(const longlong2* rx, int i) {
+  const longlong2 a = __ldg(rx + 2 * i), b = __ldg(rx + 2 * i + 1);
+  return {a.x, a.y, b.x, (unsigned)b.y, (int)(b.y >> 32)};
+}
+// x with its sign bit flipped when sg = 2^31
+__device__ __forceinline__ double flip_sign(double x, unsigned sg) {
+  return __hiloint2double(__double2hiint(x) ^ (int)sg, __double2loint(x));
 }
 
 template <int NW, bool JAC, bool FF, bool FX>
@@ -938,48 +1029,71 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
   const int K = m.K;
   Scal s;
   s.T = y[0];
-  // the scalar warp: ln T and 1/T for every thread (read after the reduction's barriers)
+  // Phase A: Y/W of every species and its sum; ln T and 1/T on the scalar warp.
   if (c.warp == Cta<NW>::SW) {
-    const double lg = FX ? __longlong_as_double(fx_log<58>(s.T)) : xlog(s.T);
+    const double lg = FX ? __longlong_as_double(fx_log(s.T, 58)) : xlog(s.T);
     const double iT = xrcp(s.T);
     if (c.lane == 0) {
-      c.red[SC_LOGT] = lg;
-      c.red[SC_INVT] = iT;
+      c.red()[SC_LOGT] = lg;
+      c.red()[SC_INVT] = iT;
     }
   }
-  {
-    double part[1] = {0.0};
-    for (int k = c.tid; k < K; k += NT) part[0] += y[1 + k] * m.invW[k];
-    double o[3];
-    const double T = s.T;
-    // (fin runs after the reduction's first barrier: 1/T is in shared memory by then)
-    c.reduce(part, warps_for<NW>(K), [&](const double (&t)[1], double (&r)[3]) {
-      const double Wbar = xrcp(t[0]);
-      r[0] = Wbar;
-      r[1] = p * c.red[SC_INVT] * Wbar * (1.0 / kRc);  // rho = p Wbar / (Rc T)
-      r[2] = kRc * T * t[0] / p;                       // 1 / rho
-    }, o);
-    s.Wbar = o[0];
-    s.rho = o[1];
-    s.irho = o[2];
+  const int nsw = warps_for<NW>(K);  // warps that hold species
+  ff2* const yWf = reinterpret_cast<ff2*>(c.dk());
+  double part = 0.0;
+#pragma unroll 1
+  for (int k = c.tid; k < K; k += NT) {
+    const double yW = y[1 + k] * c.iW()[k];
+    c.C()[k] = yW;
+    // copy for the third-body sums, in the slot of d_k (written after the reaction loop)
+    if (FF) yWf[k] = ff_split(yW);
+    else c.dk()[k] = yW;
+    part += yW;
   }
-  const double lgT = c.red[SC_LOGT];
-  s.invT = c.red[SC_INVT];
+  if (c.warp > 0 && c.warp < nsw) c.sc()[(c.warp - 1) * 32 + c.lane] = part;
+  __syncthreads();
+  // Phase B: the species warps finish the sum (warp 0) and evaluate the species; the other
+  // warps meanwhile take the third-body sums, which need Y/W only: [M] = rho sum eff Y/W.
+  // The species warps wait for warp 0's scalars on a barrier of their own.
+  if (c.warp < nsw) {
+    if (c.warp == 0) {
+#pragma unroll 1
+      for (int w = 1; w < nsw; ++w) part += c.sc()[(w - 1) * 32 + c.lane];
+#pragma unroll
+      for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(FULLMASK, part, o);
+      const double Wbar = xrcp(part);
+      const double rho = c.p_rc * c.red()[SC_INVT] * Wbar;  // p Wbar / (Rc T)
+      const double irho = c.rc_p * s.T * part;
+      if (c.lane == 0) {
+        c.red()[SC_OUT] = Wbar;
+        c.red()[SC_OUT + 1] = rho;
+        c.red()[SC_OUT + 2] = irho;
+      }
+    }
+    if (nsw == NW) __syncthreads();
+    else if (nsw > 1) asm volatile("bar.sync 1, %0;" ::"r"(nsw * 32) : "memory");
+    else __syncwarp();
+  }
+  const double lgT = c.red()[SC_LOGT];
+  s.invT = c.red()[SC_INVT];
   const double T = s.T, invT = s.invT;
   // ln T (Q58), 1/T (Q71) and ln(Rc T/P0) (Q52), or their FP64 forms
   const unsigned long long LT = (unsigned long long)__double_as_longlong(lgT);
   const unsigned long long IT = fx_scale(invT, 19);
   const Arg lc = FX ? (Arg)((long long)(LT >> 6) + kLnRcP0_Q52) : (Arg)(lgT + kLnRcP0);
-  Arg* const g_RT = reinterpret_cast<Arg*>(c.g);
+  Arg* const g_RT = reinterpret_cast<Arg*>(c.g());
   // species: thermo, G/RT, concentrations
+  if (c.warp < nsw) s.rho = c.red()[SC_OUT + 1];
+#pragma unroll 1
   for (int k = c.tid; k < K; k += NT) {
-    const double* a = m.nasa + 36 * k;
-    const bool low = T < a[34];
-    a += low ? 0 : 17;
-    double cp = a[0] + T * (a[1] + T * (a[2] + T * (a[3] + T * a[4])));
-    double h = a[5] + T * (a[6] + T * (a[7] + T * (a[8] + T * a[9]))) + a[10] * invT;
-    c.cpR[k] = cp;
-    c.hRT[k] = h;
+    const bool low = T < m.T_mid[k];
+    double cp, h;
+    const double2* a = m.hcp + 10 * k + (low ? 0 : 5);
+    const double2 a0 = a[0], a1 = a[1], a2 = a[2], a3 = a[3], a4 = a[4];
+    cp = a0.x + T * (a0.y + T * (a1.x + T * (a1.y + T * a2.x)));
+    h = a0.x + T * (a2.y + T * (a3.x + T * (a3.y + T * a4.x))) + a4.y * invT;
+    c.cpR()[k] = cp;
+    c.hRT()[k] = h;
     if constexpr (FX) {
       // T / 2048 below T_mid, T / 8192 above (Q64)
       const unsigned long long t = fx_scale(T, low ? 1 : -1);
@@ -988,27 +1102,78 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
       const long long poly = fx_mul(q1.y + fx_mul(q2.x + fx_mul(q2.y + fx_mul(q3.x, t), t), t), t);
       g_RT[k] = q0.x + fx_mul(q0.y, LT) + fx_mul(q1.x, IT) + poly;
     } else {
-      const double sr = a[11] * lgT + T * (a[12] + T * (a[13] + T * (a[14] + T * a[15]))) + a[16];
+      const double* b = m.nasa + 36 * k + (low ? 0 : 17);
+      const double sr = b[11] * lgT + T * (b[12] + T * (b[13] + T * (b[14] + T * b[15]))) + b[16];
       g_RT[k] = h - sr;
     }
-    const double Ck = s.rho * y[1 + k] * m.invW[k];
-    c.C[k] = Ck;
-    // float-float copy of C for the third-body sums (the slot of d_k, which the
-    // Jacobian evaluation writes only after the reaction loop)
-    if (FF) reinterpret_cast<ff2*>(c.dk)[k] = ff_split(Ck);
-    if (JAC) c.dcp[k] = a[1] + T * (2.0 * a[2] + T * (3.0 * a[3] + T * 4.0 * a[4]));
+    c.C()[k] *= s.rho;
+    if (JAC) c.dcp()[k] = a0.y + T * (2.0 * a1.x + T * (3.0 * a1.y + T * 4.0 * a2.x));
+  }
+  // third-body sums of 32 reactions at a time into their q slots, efficiencies species-
+  // major: the warp's 32 reactions read one row per species
+  constexpr int v = NW == 2 ? 0 : NW == 4 ? 1 : 2;
+#pragma unroll 1
+  for (int pos = m.tb_sched[v][c.warp]; pos < m.tb_sched[v][c.warp + 1]; ++pos) {
+    const int r = m.tb_sched[v][NW + 1 + pos] * 32 + c.lane, ntb = m.n_tb;
+    double S;
+    if (FF) {
+      // eight terms at a time, the next eight efficiencies loaded while these are summed
+      // (the table's padding rows make the loads past the last species harmless)
+      constexpr int B = 8;
+      const ff2* ef = m.effT_ff + r;
+      ff_sum acc;
+      ff2 e[B];
+#pragma unroll
+      for (int u = 0; u < B; ++u) e[u] = ef[u * ntb];
+#pragma unroll 1
+      for (int k = 0; k < K; k += B) {
+        ff2 y4[B], en[B];
+        ef += B * ntb;
+#pragma unroll
+        for (int u = 0; u < B; ++u) {
+          en[u] = ef[u * ntb];
+          y4[u] = k + u < K ? yWf[k + u] : ff2{0.0f, 0.0f};
+        }
+#pragma unroll
+        for (int u = 0; u < B; ++u) acc.add_prod(e[u], y4[u]);
+#pragma unroll
+        for (int u = 0; u < B; ++u) e[u] = en[u];
+      }
+      S = ff_value(acc.value());
+    } else {
+      const double* e = m.effT + r;
+      S = 0.0;
+#pragma unroll 6
+      for (int k = 0; k < K; ++k) S += e[(size_t)k * ntb] * c.dk()[k];
+    }
+    c.q()[m.i_tb0 + r] = S;
   }
   __syncthreads();
-  // 32-reaction chunks of one kind each, dealt to the warps by estimated work
-  const int* cs = m.chunk_sched[NW == 2 ? 0 : NW == 4 ? 1 : 2];
-  for (int pos = cs[c.warp]; pos < cs[c.warp + 1]; ++pos) {
-    const int i = cs[NW + 1 + pos] * 32 + c.lane;
-    const int4 sl = m.slots[i];
-    if (sl.x < 0) {  // null padding reaction
-      c.q[i] = 0.0;
+  s.Wbar = c.red()[SC_OUT];
+  s.rho = c.red()[SC_OUT + 1];
+  s.irho = c.red()[SC_OUT + 2];
+  // 32-reaction chunks of one kind each, dealt to the warps by estimated time; the next
+  // chunk's record is loaded while this one is evaluated
+  const int* cs = m.chunk_sched[v];
+  const int pos1 = cs[c.warp + 1];
+  int pos = cs[c.warp];
+  int i_next = pos < pos1 ? cs[NW + 1 + pos] * 32 + c.lane : 0;
+  RxRec rec_next = {};
+  if (pos < pos1) rec_next = load_rec(m.rx, i_next);
+#pragma unroll 1
+  for (; pos < pos1; ++pos) {
+    const int i = i_next;
+    const RxRec rec = rec_next;
+    if (pos + 1 < pos1) {
+      i_next = cs[NW + 2 + pos] * 32 + c.lane;
+      rec_next = load_rec(m.rx, i_next);
+    }
+    const int4 sl = make_int4(rec.slots & 255u, (rec.slots >> 8) & 255u, (rec.slots >> 16) & 255u, rec.slots >> 24);
+    if (sl.x == 255) {  // null padding reaction
+      c.q()[i] = 0.0;
       if (JAC) {
-        c.D[i] = c.dTc[i] = c.P[i] = 0.0;
-        c.dqs[4 * i] = c.dqs[4 * i + 1] = c.dqs[4 * i + 2] = c.dqs[4 * i + 3] = 0.0;
+        c.D()[i] = c.dTc()[i] = c.P()[i] = 0.0;
+        c.dqs()[4 * i] = c.dqs()[4 * i + 1] = c.dqs()[4 * i + 2] = c.dqs()[4 * i + 3] = 0.0;
       }
       continue;
     }
@@ -1022,32 +1187,18 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
       dnu = a23.y;
       if (!FX) ka = (Arg)(a01.x + a01.y * lgT - a23.x * invT);
     }
-    if constexpr (FX) {
-      const longlong2 x01 = reinterpret_cast<const longlong2*>(m.arx + 4 * i)[0];
-      const long long x2 = m.arx[4 * i + 2];
-      ka = fx_clamp(x01.x + fx_mul(x01.y, LT) - fx_mul(x2, IT), 1100);
-    }
-    const double Ca = c.C[sl.x];
-    const double Cb = sl.y >= 0 ? c.C[sl.y] : 1.0;
-    const double Cc = c.C[sl.z];
-    const double Cd = sl.w >= 0 ? c.C[sl.w] : 1.0;
-    const int rv = m.rev[i];
+    if constexpr (FX) ka = fx_clamp(rec.lnA + fx_mul(rec.b, LT) - fx_mul(rec.th, IT), 1100);
+    const bool two_f = sl.y != 255, two_r = sl.w != 255;
+    const double Ca = c.C()[sl.x];
+    const double Cb = two_f ? c.C()[sl.y] : 1.0;
+    const double Cc = c.C()[sl.z];
+    const double Cd = two_r ? c.C()[sl.w] : 1.0;
+    const int rv = rec.rev;
     // factor of the mass-action rate: 1, [M], or [M] / (1 + Pr) (falloff)
     double Mc = 0.0, phi = 1.0, red1 = 1.0;
     double dlnk = (b_rx + th_rx * invT) * invT, gM = 1.0;  // d ln k/dT; d ln q/d ln[M]
     if (i >= m.i_tb0) {
-      // efficiencies species-major: the warp's 32 reactions read one row per species
-      const int r = i - m.i_tb0, ntb = m.n_tb;
-      if (FF) {
-        const ff2* ef = m.effT_ff + r;
-        const ff2* Cf = reinterpret_cast<const ff2*>(c.dk);
-        ff2 acc = {0.0f, 0.0f};
-        for (int k = 0; k < K; ++k) acc = ff_fma(ef[(size_t)k * ntb], Cf[k], acc);
-        Mc = ff_value(acc);
-      } else {
-        const double* e = m.effT + r;
-        for (int k = 0; k < K; ++k) Mc += e[(size_t)k * ntb] * c.C[k];
-      }
+      Mc = s.rho * c.q()[i];
       phi = Mc;
     }
     if (i >= m.i_fo0) {
@@ -1061,7 +1212,7 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
       } else {
         fa = fo[0] + fo[1] * lgT - fo[2] * invT;
       }
-      const double Pr = rate_exp<FX>(fa) * Mc;
+      const double Pr = rate_exp<FX>(fa, c.xt()) * Mc;
       red1 = xrcp(1.0 + Pr);
       double dlgF_dL = 0.0, dlnF_dT = 0.0;
       ka = ka + fa;
@@ -1069,18 +1220,27 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
         const double alpha = fo[3];
         // fo[4] = 1/T***, fo[5] = 1/T*
         const double x3 = -T * fo[4], x1 = -T * fo[5];
-        double e3, e1, e2 = 0.0;
-        if constexpr (FX) {
-          e3 = fx_exp(fx_from_double(x3));
-          e1 = fx_exp(fx_from_double(x1));
-          if (fo[6] > 0.0) e2 = fx_exp(fx_from_double(-fo[6] * invT));
-        } else {
-          e3 = xexp(x3);
-          e1 = xexp(x1);
-          if (fo[6] > 0.0) e2 = xexp(-fo[6] * invT);
+        // (rolled loops: one copy of the exponential and of the logarithm in the code)
+        double e3 = 0.0, e1 = 0.0, e2 = 0.0;
+        const int ne = fo[6] > 0.0 ? 3 : 2;
+#pragma unroll 1
+        for (int u = 0; u < ne; ++u) {
+          const double xa = u == 0 ? x3 : u == 1 ? x1 : -fo[6] * invT;
+          double ex;
+          if constexpr (FX) ex = fx_exp(fx_from_double(xa), c.xt());
+          else ex = xexp(xa);
+          if (u == 0) e3 = ex;
+          else if (u == 1) e1 = ex;
+          else e2 = ex;
         }
         const double Fc = (1.0 - alpha) * e3 + alpha * e1 + e2;
-        const double lF = rate_log<FX>(Fc), lP = rate_log<FX>(Pr);  // natural logarithms
+        double lF = 0.0, lP = 0.0;  // natural logarithms
+#pragma unroll 1
+        for (int u = 0; u < 2; ++u) {
+          const double l = rate_log<FX>(u == 0 ? Fc : Pr);
+          if (u == 0) lF = l;
+          else lP = l;
+        }
         const double cc = fma(lF, -0.67 * kInvLn10, -0.4), nn = fma(lF, -1.27 * kInvLn10, 0.75);
         const double x = fma(lP, kInvLn10, cc);
         const double den = fma(x, -0.14, nn);
@@ -1116,111 +1276,154 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
         dlnk += gM * (fo[1] + fo[2] * invT) * invT + dlnF_dT;
       }
     }
-    const double kfP = rate_exp<FX>(ka);
+    const double kfP = rate_exp<FX>(ka, c.xt());
     double krP = 0.0;
     if (rv & 1) {
       Arg dg = g_RT[sl.z] - g_RT[sl.x];
-      if (sl.w >= 0) dg += g_RT[sl.w];
-      if (sl.y >= 0) dg -= g_RT[sl.y];
+      if (two_r) dg += g_RT[sl.w];
+      if (two_f) dg -= g_RT[sl.y];
       dg += (rv >> 1) == 2 ? lc : (rv >> 1) == 0 ? -lc : Arg(0);
-      if constexpr (FX) krP = fx_exp(fx_clamp(ka, 1100) + fx_clamp(dg, 900));
+      if constexpr (FX) krP = fx_exp(fx_clamp(ka, 1100) + fx_clamp(dg, 900), c.xt());
       else krP = xexp(ka + dg);
     }
     const double Pf = Ca * Cb, Pb = Cc * Cd;
     if constexpr (!JAC) {
       const double net = fma(kfP, Pf, -krP * Pb);
-      c.q[i] = i >= m.i_tb0 ? phi * net : net;
+      c.q()[i] = i >= m.i_tb0 ? phi * net : net;
     } else {
       const double qf = kfP * Pf, qr = krP * Pb;
       const double net = qf - qr;
-      c.q[i] = i >= m.i_tb0 ? phi * net : net;
+      c.q()[i] = i >= m.i_tb0 ? phi * net : net;
       // d ln Kc / dT = dH/(R T^2) - dnu/T
-      const double dH = c.hRT[sl.z] + (sl.w >= 0 ? c.hRT[sl.w] : 0.0) - c.hRT[sl.x] -
-                        (sl.y >= 0 ? c.hRT[sl.y] : 0.0);
+      const double dH = c.hRT()[sl.z] + (two_r ? c.hRT()[sl.w] : 0.0) - c.hRT()[sl.x] -
+                        (two_f ? c.hRT()[sl.y] : 0.0);
       const double dlnKc = (dH - dnu) * invT;
       const double kfp = phi * kfP, krp = -phi * krP;
-      const double dq0 = kfp * Cb, dq1 = sl.y >= 0 ? kfp * Ca : 0.0;
-      const double dq2 = krp * Cd, dq3 = sl.w >= 0 ? krp * Cc : 0.0;
+      const double dq0 = kfp * Cb, dq1 = two_f ? kfp * Ca : 0.0;
+      const double dq2 = krp * Cd, dq3 = two_r ? krp * Cc : 0.0;
       if (FF) {
         // the float-float assembly's copy (hi, lo), split once here
-        ff2* dqf = reinterpret_cast<ff2*>(c.dqs) + 4 * i;
+        ff2* dqf = reinterpret_cast<ff2*>(c.dqs()) + 4 * i;
         dqf[0] = ff_split(dq0);
         dqf[1] = ff_split(dq1);
         dqf[2] = ff_split(dq2);
         dqf[3] = ff_split(dq3);
       } else {
-        c.dqs[4 * i] = dq0;
-        c.dqs[4 * i + 1] = dq1;
-        c.dqs[4 * i + 2] = dq2;
-        c.dqs[4 * i + 3] = dq3;
+        c.dqs()[4 * i] = dq0;
+        c.dqs()[4 * i + 1] = dq1;
+        c.dqs()[4 * i + 2] = dq2;
+        c.dqs()[4 * i + 3] = dq3;
       }
-      c.dTc[i] = phi * fma(dlnk, net, qr * dlnKc);
+      c.dTc()[i] = phi * fma(dlnk, net, qr * dlnKc);
       const double Pc = i >= m.i_tb0 ? gM * red1 * net : 0.0;
       if (FF)
-        reinterpret_cast<ff2*>(c.P)[i] = ff_split(Pc);
+        reinterpret_cast<ff2*>(c.P())[i] = ff_split(Pc);
       else
-        c.P[i] = Pc;
+        c.P()[i] = Pc;
       // sum_k C_k dq/dC_k: the mass-action orders, and [M]
-      double Dsum = phi * ((sl.y >= 0 ? 2.0 * qf : qf) - (sl.w >= 0 ? 2.0 * qr : qr));
+      double Dsum = phi * ((two_f ? 2.0 * qf : qf) - (two_r ? 2.0 * qr : qr));
       if (i >= m.i_tb0) Dsum = fma(Mc, Pc, Dsum);
-      c.D[i] = Dsum;
+      c.D()[i] = Dsum;
+    }
+  }
+  const uint2* ps = m.ps_ent[v] + c.tid;
+  uint2 en = ps[0];  // (in flight across the barrier)
+  // cp (and d cp/dT) of the mixture, on the scalar warp: mean over C, rho sum Y/W x = sum C x
+  if (c.warp == Cta<NW>::SW) {
+    double cs1 = 0.0, cs2 = 0.0;
+#pragma unroll 1
+    for (int k = c.lane; k < K; k += 32) {
+      cs1 += c.C()[k] * c.cpR()[k];
+      if (JAC) cs2 += c.C()[k] * c.dcp()[k];
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      cs1 += __shfl_xor_sync(FULLMASK, cs1, o);
+      if (JAC) cs2 += __shfl_xor_sync(FULLMASK, cs2, o);
+    }
+    const double rr = kRc * s.irho;
+    const double icpm = xrcp(cs1 * rr);
+    if (c.lane == 0) {
+      c.red()[SC_ICPM] = icpm;
+      if (JAC) c.red()[SC_DCPM] = cs2 * rr;
     }
   }
   __syncthreads();
-  // species: production rates, f_k, enthalpy and heat-capacity sums
-  double part[JAC ? 4 : 2];
-  part[0] = part[1] = 0.0;
-  if (JAC) part[2] = part[3] = 0.0;
-  for (int k = c.tid; k < K; k += NT) {
+  // Production rates: each species' reactions over a group of ps_g adjacent lanes, from a
+  // table of 16-bit entries (reaction << 1 | sign), four to a load and padded to the
+  // longest list; the signed terms are added one FP64 instruction each.
+#pragma unroll 1
+  for (int pass = 0; pass < m.ps_passes[v]; ++pass) {
+    const int g = m.ps_g[v];
     double w = 0.0, dd = 0.0, at = 0.0;
-    for (int e = m.sp_ptr[k]; e < m.sp_ptr[k + 1]; ++e) {
-      const int2 en = m.sp_ent[e];
-      const double nu = m.sp_nu[e];
-      w += nu * c.q[en.x];
+    auto add = [&](unsigned e) {
+      if (e != 0xffffu) {
+        const unsigned i = e >> 1, sg = e << 31;
+        w += flip_sign(c.q()[i], sg);
+        if (JAC) {
+          dd += flip_sign(c.D()[i], sg);
+          at += flip_sign(c.dTc()[i], sg);
+        }
+      }
+    };
+#pragma unroll 1
+    for (int r = 0; r < m.ps_quads[v]; ++r) {
+      const uint2 e = en;
+      const int nx = pass * m.ps_quads[v] + r + 1;
+      if (nx < m.ps_passes[v] * m.ps_quads[v]) en = ps[(size_t)nx * NT];
+      add(e.x & 0xffffu);
+      add(e.x >> 16);
+      add(e.y & 0xffffu);
+      add(e.y >> 16);
+    }
+#pragma unroll 1
+    for (int o = 1; o < g; o <<= 1) {
+      w += __shfl_xor_sync(FULLMASK, w, o);
       if (JAC) {
-        dd += nu * c.D[en.x];
-        at += nu * c.dTc[en.x];
+        dd += __shfl_xor_sync(FULLMASK, dd, o);
+        at += __shfl_xor_sync(FULLMASK, at, o);
       }
     }
-    f[1 + k] = m.W[k] * w * s.irho;
-    part[0] += c.hRT[k] * w;                  // Qh / (Rc T)
-    part[1] += y[1 + k] * c.cpR[k] * m.invW[k];  // cpm / Rc
-    if (JAC) {
-      c.dk[k] = dd;
-      c.akT[k] = at;
-      part[2] += y[1 + k] * c.dcp[k] * m.invW[k];  // dcpm/dT / Rc
-      part[3] += c.cpR[k] * w;                      // sum cp_k omega_k / Rc
+    const int k = (pass * NT + c.tid) / g;
+    if ((c.tid & (g - 1)) == 0 && k < K) {
+      c.ek()[k] = w;
+      if (JAC) {
+        c.dk()[k] = dd;
+        c.akT()[k] = at;
+      }
     }
   }
+  __syncthreads();
+  // species: f_k and the enthalpy sums
+  s.icpm = c.red()[SC_ICPM];
+  if (JAC) s.dcpm = c.red()[SC_DCPM];
   {
-    double o[5];
-    const double T = s.T, irho = s.irho;
-    c.reduce(part, warps_for<NW>(K), [&](const double (&t)[JAC ? 4 : 2], double (&r)[5]) {
-      const double cpm = kRc * t[1];
-      const double icpm = xrcp(cpm);
+    double part2[JAC ? 2 : 1] = {};
+#pragma unroll 1
+    for (int k = c.tid; k < K; k += NT) {
+      const double w = c.ek()[k];
+      f[1 + k] = m.W[k] * w * s.irho;
+      part2[0] += c.hRT()[k] * w;  // Qh / (Rc T)
+      if (JAC) part2[JAC ? 1 : 0] += c.cpR()[k] * w;  // sum cp_k omega_k / Rc
+    }
+    double o[2];
+    const double T = s.T, irho = s.irho, icpm = s.icpm;
+    c.reduce(part2, nsw, [&](const double (&t)[JAC ? 2 : 1], double (&r)[2]) {
       const double fT = -kRc * T * t[0] * irho * icpm;  // -Qh / (rho cp), Qh = Rc T sum hRT_k w_k
-      r[0] = cpm;
-      r[1] = icpm;
-      r[2] = fT;
-      if constexpr (JAC) {
-        r[3] = kRc * t[2];
-        r[4] = kRc * t[3];
-      } else {
-        r[3] = r[4] = 0.0;
-      }
+      r[0] = fT;
+      r[1] = JAC ? kRc * t[JAC ? 1 : 0] : 0.0;
       if (c.lane == 0) f[0] = fT;  // visible after the reduction's last barrier
     }, o);
-    s.cpm = o[0];
-    s.icpm = o[1];
-    s.fT = o[2];
-    s.dcpm = o[3];
-    s.Scpw = o[4];
+    s.fT = o[0];
+    s.Scpw = o[1];
   }
   return s;
 }
 
+// (The CTA's pointers are passed by value: a reference to them that leaves the caller
+// would keep them in local memory there, to be read again after every store.)
 template <int NW, bool JAC, bool FF>
-__device__ __noinline__ Scal eval_rhs_fp64(const DevMech& m, Cta<NW>& c, const double* y, double p, double* f) {
+__device__ __noinline__ Scal eval_rhs_fp64(const DevMech& m, Cta<NW> c, const double* y, double p, double* f) {
   return eval_rhs_t<NW, JAC, FF, false>(m, c, y, p, f);
 }
 
@@ -1263,31 +1466,35 @@ __device__ __forceinline__ double rx_data(const double* a, int i) {
   else return a[i];
 }
 
+// Entry (i, j) of the assembled matrix at i si + j sj.
 template <int NW, class R, bool JO, int U, bool FFD>
-__device__ void assemble_rows(const DevMech& m, Cta<NW>& c, R* A, int K, int ld, R rf) {
+__device__ void assemble_rows(const DevMech& m, Cta<NW>& c, R* A, int K, int si, int sj, R rf) {
   constexpr double SG = JO ? 1.0 : -1.0;
+#pragma unroll 1
   for (int k = c.warp; k < K; k += NW) {
-    R* row = A + (1 + k) * ld + 1;
-    const R beta = R(c.akT[k]);
+    R* row = A + (1 + k) * si + sj;
+    const R beta = R(c.akT()[k]), Wk = R(SG * m.W[k]);
     R acc[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const unsigned msk = m.jmask[k * U + u];
-      acc[u] = ((msk >> c.lane) & 1u) ? beta + row[c.lane + 32 * u] : beta;
+      acc[u] = ((msk >> c.lane) & 1u) ? fmaR(Wk, row[(c.lane + 32 * u) * sj], beta) : beta;
     }
     // third-body / falloff part: 32 row coefficients sg nu_ki W_k P_i at a time,
     // broadcast from their lanes
     const int t1 = m.tr_ptr[k + 1];
+#pragma unroll 1
     for (int tb = m.tr_ptr[k]; tb < t1; tb += 32) {
       const int t = tb + c.lane;
       R cl = R(0);
       int rl = 0;
       if (t < t1) {
         const int ri = m.tr_ent[t].x;
-        cl = R(SG * m.tr_nu[t] * rx_data<FFD>(c.P, ri));
+        cl = R(SG * m.tr_nu[t] * rx_data<FFD>(c.P(), ri));
         rl = ri - m.i_tb0;
       }
       const int cnt = min(32, t1 - tb);
+#pragma unroll 1
       for (int q = 0; q < cnt; ++q) {
         const R coef = __shfl_sync(FULLMASK, cl, q);
         const double* e = m.eff + (size_t)__shfl_sync(FULLMASK, rl, q) * K;
@@ -1301,66 +1508,97 @@ __device__ void assemble_rows(const DevMech& m, Cta<NW>& c, R* A, int K, int ld,
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int j = c.lane + 32 * u;
-      if (u < U - 1 || j < K) row[j] = fmaR(acc[u], R(m.invW[j]), j == k ? rf : R(0));
+      if (u < U - 1 || j < K) row[j * sj] = fmaR(acc[u], R(c.iW()[j]), j == k ? rf : R(0));
     }
   }
 }
 
-template <int NW, class R, bool JO, bool FFD = false>
+// Mass-action sums sum_i nu_ki dq_i/dC_j, one per existing (k, j), on the thread-balanced
+// schedule js: entry x = (dq index) << 1 | sign (~0: padding), y = k << 8 | j where the
+// finished sum goes (~0: it continues); put(k, j, sum) stores it. The entries are loaded
+// four rounds ahead: the table streams through once per step and misses the L1 cache.
+template <int NW, class Acc, class Get, class Put>
+__device__ void mass_action_sums(const DevMech& m, Cta<NW>& c, Get get, Put put) {
+  constexpr int NT = NW * 32, v = NT == 64 ? 0 : NT == 128 ? 1 : 2, B = 4;
+  const uint2* se = m.js_ent[v] + c.tid;
+  const int rounds = m.js_rounds[v];  // a multiple of B
+  uint2 e[B], en[B];
+#pragma unroll
+  for (int u = 0; u < B; ++u) en[u] = ld_stream(se + u * NT);
+  Acc a{};
+#pragma unroll 1
+  for (int r = 0; r < rounds; r += B) {
+#pragma unroll
+    for (int u = 0; u < B; ++u) e[u] = en[u];
+    if (r + B < rounds) {
+#pragma unroll
+      for (int u = 0; u < B; ++u) en[u] = ld_stream(se + (size_t)(r + B + u) * NT);
+    }
+#pragma unroll
+    for (int u = 0; u < B; ++u) {
+      if (e[u].x != 0xffffffffu) get(a, (int)(e[u].x >> 1), e[u].x << 31);
+      if (e[u].y != 0xffffffffu) {
+        put((int)(e[u].y >> 8), (int)(e[u].y & 255u), a);
+        a = Acc{};
+      }
+    }
+  }
+}
+
+// FP64 form: row-major in the LU matrix (BYCOL = false); FP32-assembled form: by columns.
+template <int NW, class R, bool JO, bool FFD = false, bool BYCOL = false>
 __device__ void assemble(const DevMech& m, Cta<NW>& c, const Scal& s, const double* f, double fac, void* target) {
   constexpr int NT = NW * 32;
   constexpr double SG = JO ? 1.0 : -1.0;
   const int K = m.K, n = K + 1, ld = odd_ld(n);
+  const int si = BYCOL ? 1 : ld, sj = BYCOL ? ld : 1;
   R* A = reinterpret_cast<R*>(target);
   const R rf = JO ? R(0) : R(fac);
   // (1) species pass
   const double eT = kRc * s.T * s.icpm, wr = s.Wbar * s.irho;
+#pragma unroll 1
   for (int k = c.tid; k < K; k += NT) {
-    c.ek[k] = c.hRT[k] * eT * m.invW[k];
-    const double Wk = m.W[k], dk = c.dk[k], fk = f[1 + k];
-    A[(1 + k) * ld] = R(SG * (Wk * s.irho * (c.akT[k] - dk * s.invT) + fk * s.invT));
-    c.akT[k] = SG * (fk * s.Wbar - Wk * wr * dk);  // beta_k (a_kT is consumed)
+    c.ek()[k] = c.hRT()[k] * eT * c.iW()[k];
+    const double Wk = m.W[k], dk = c.dk()[k], fk = f[1 + k];
+    A[(1 + k) * si] = R(SG * (Wk * s.irho * (c.akT()[k] - dk * s.invT) + fk * s.invT));
+    c.akT()[k] = SG * (fk * s.Wbar - Wk * wr * dk);  // beta_k (a_kT is consumed)
   }
-  {
-    const int v = NT == 64 ? 0 : NT == 128 ? 1 : 2;
-    const int2* se = m.js_ent[v] + c.tid;
-    const double* sn = m.js_nu[v] + c.tid;
-    const int rounds = m.js_rounds[v];
-    R a = R(0);
-    for (int r = 0; r < rounds; ++r) {
-      const int2 e = se[r * NT];
-      if (e.x >= 0) a = fmaR(R(SG * sn[r * NT]), R(rx_data<FFD>(c.dqs, e.x)), a);
-      if (e.y >= 0) {
-        A[e.y] = a;
-        a = R(0);
-      }
-    }
-  }
+  mass_action_sums<NW, R>(
+      m, c,
+      [&](R& a, int i, unsigned sg) {
+        if constexpr (FFD)
+          a += __uint_as_float(__float_as_uint(reinterpret_cast<const ff2*>(c.dqs())[i].hi) ^ sg);
+        else
+          a += flip_sign(c.dqs()[i], sg);
+      },
+      [&](int k, int j, R a) { A[(1 + k) * si + (1 + j) * sj] = a; });
   __syncthreads();
   // (2) species rows
   switch ((K + 31) >> 5) {
-    case 1: assemble_rows<NW, R, JO, 1, FFD>(m, c, A, K, ld, rf); break;
-    case 2: assemble_rows<NW, R, JO, 2, FFD>(m, c, A, K, ld, rf); break;
-    case 3: assemble_rows<NW, R, JO, 3, FFD>(m, c, A, K, ld, rf); break;
-    case 4: assemble_rows<NW, R, JO, 4, FFD>(m, c, A, K, ld, rf); break;
-    case 5: assemble_rows<NW, R, JO, 5, FFD>(m, c, A, K, ld, rf); break;
-    case 6: assemble_rows<NW, R, JO, 6, FFD>(m, c, A, K, ld, rf); break;
-    case 7: assemble_rows<NW, R, JO, 7, FFD>(m, c, A, K, ld, rf); break;
-    default: assemble_rows<NW, R, JO, 8, FFD>(m, c, A, K, ld, rf); break;
+    case 1: assemble_rows<NW, R, JO, 1, FFD>(m, c, A, K, si, sj, rf); break;
+    case 2: assemble_rows<NW, R, JO, 2, FFD>(m, c, A, K, si, sj, rf); break;
+    case 3: assemble_rows<NW, R, JO, 3, FFD>(m, c, A, K, si, sj, rf); break;
+    case 4: assemble_rows<NW, R, JO, 4, FFD>(m, c, A, K, si, sj, rf); break;
+    case 5: assemble_rows<NW, R, JO, 5, FFD>(m, c, A, K, si, sj, rf); break;
+    case 6: assemble_rows<NW, R, JO, 6, FFD>(m, c, A, K, si, sj, rf); break;
+    case 7: assemble_rows<NW, R, JO, 7, FFD>(m, c, A, K, si, sj, rf); break;
+    default: assemble_rows<NW, R, JO, 8, FFD>(m, c, A, K, si, sj, rf); break;
   }
   __syncthreads();
   // (3) temperature row; with acc = sum_k e_k S_kj, sum_k e_k J_kj = sg (acc - rf e_(j-1)),
   //     so S_0j = rf e_(j-1) - acc - sg extra_j (j >= 1) and S_00 = rf - acc - sg extra_0
   const double ft = s.fT * s.icpm;
+#pragma unroll 1
   for (int j = NT - 1 - c.tid; j < n; j += NT) {  // from the last warp down, as the residual rows
     R acc = R(0);
-    for (int k = 0; k < K; ++k) acc = fmaR(R(c.ek[k]), A[(1 + k) * ld + j], acc);
+#pragma unroll 1
+    for (int k = 0; k < K; ++k) acc = fmaR(R(c.ek()[k]), A[(1 + k) * si + j * sj], acc);
     R v;
     if (j == 0)
       v = rf - acc - R(SG * (s.Scpw * s.irho * s.icpm + ft * s.dcpm));
     else
-      v = rf * R(c.ek[j - 1]) - acc - R(SG * ft * c.cpR[j - 1] * kRc * m.invW[j - 1]);
-    A[j] = v;
+      v = rf * R(c.ek()[j - 1]) - acc - R(SG * ft * c.cpR()[j - 1] * kRc * c.iW()[j - 1]);
+    A[j * sj] = v;
   }
   __syncthreads();
 }
@@ -1372,48 +1610,101 @@ __device__ void assemble(const DevMech& m, Cta<NW>& c, const Scal& s, const doub
 // scalars are formed in FP64 and split once per species. A holds (hi, lo) per entry;
 // its error is a few units of 2^-48 relative to the sums' terms, far below the FP32
 // factorisation's, so the refinement converges to the same solutions.
-template <int NW, bool JO, int U>
-__device__ void assemble_rows_ff(const DevMech& m, Cta<NW>& c, ff2* A, int K, int ld, ff2 rf) {
-  const ff2* beta_ff = reinterpret_cast<const ff2*>(c.akT);
-  const ff2* Pf = reinterpret_cast<const ff2*>(c.P);
+//
+// A warp takes RG consecutive rows (lanes on the columns, all sums in registers), so that
+// a lane finishes RG entries of a column side by side (one 32-byte sector for RG = 4), and
+// adds e_k S_kj to its share of the temperature row; the warps' shares meet in shared
+// memory (the vectors rr, u and sc). Third-body coefficients sg nu_ki W_k P_i come from
+// shared memory (cf, in the place of dq once the mass-action sums have consumed it).
+template <int NW, bool JO, int U, int RG>
+__device__ void assemble_rows_ff(const DevMech& m, Cta<NW>& c, ff2* A, int K, ff2 rf) {
+  const ff2* beta_ff = reinterpret_cast<const ff2*>(c.akT());
+  const ff2* ek = reinterpret_cast<const ff2*>(c.ek());
+  const ff2* cf = reinterpret_cast<const ff2*>(c.dqs());
   const ff2 zero = {0.0f, 0.0f};
-  for (int k = c.warp; k < K; k += NW) {
-    ff2* row = A + (1 + k) * ld + 1;
-    const ff2 beta = beta_ff[k];
-    ff_sum acc[U];
+  const int ld0 = c.ld0;
+  ff2* A1 = A + c.i0 + 1;  // row of species 0
+  ff_sum accT[U], accT0;
+#pragma unroll 1
+  for (int k0 = c.warp * RG; k0 < K; k0 += NW * RG) {
+    ff2 S[RG][U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const unsigned msk = m.jmask[k * U + u];
-      acc[u] = ff_sum(beta);
-      if ((msk >> c.lane) & 1u) acc[u].add(row[c.lane + 32 * u]);
-    }
-    const int t1 = m.tr_ptr[k + 1];
-    for (int tb = m.tr_ptr[k]; tb < t1; tb += 32) {
-      const int t = tb + c.lane;
-      ff2 cl = zero;
-      int rl = 0;
-      if (t < t1) {
-        const int ri = m.tr_ent[t].x;
-        const ff2 tn = m.tr_nu_ff[t];
-        cl = ff_mul(JO ? tn : ff_neg(tn), Pf[ri]);
-        rl = ri - m.i_tb0;
-      }
-      const int cnt = min(32, t1 - tb);
-      for (int q = 0; q < cnt; ++q) {
-        const ff2 coef = {__shfl_sync(FULLMASK, cl.hi, q), __shfl_sync(FULLMASK, cl.lo, q)};
-        const ff2* e = m.eff_ff + (size_t)__shfl_sync(FULLMASK, rl, q) * K;
+    for (int rr = 0; rr < RG; ++rr) {
+      const int k = k0 + rr;
+#pragma unroll
+      for (int u = 0; u < U; ++u) S[rr][u] = zero;
+      if (k < K) {
+        const ff2 beta = beta_ff[k], Wk = m.W_ff[k];
+        ff_sum acc[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const unsigned msk = m.jmask[k * U + u];
+          acc[u] = ff_sum(beta);
+          if ((msk >> c.lane) & 1u) acc[u].add_prod(JO ? Wk : ff_neg(Wk), c.pair(k, c.lane + 32 * u));
+        }
+        const int t1 = m.tr_ptr[k + 1];
+        // four entries at a time: their efficiencies' loads overlap (row: offset of the
+        // entry's efficiencies; entries past the row's end have coefficient 0)
+#pragma unroll 1
+        for (int t = m.tr_ptr[k]; t < t1; t += 4) {
+          ff2 e[4][U];
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            const ff2* er = m.eff_ff + __ldg(m.tr_row + t + v);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const int j = c.lane + 32 * u;
+              if (u < U - 1 || j < K) {
+                const float2 x = __ldg(reinterpret_cast<const float2*>(er + j));
+                e[v][u] = {x.x, x.y};
+              } else {
+                e[v][u] = zero;
+              }
+            }
+          }
+#pragma unroll
+          for (int v = 0; v < 4; ++v) {
+            const ff2 coef = t + v < t1 ? cf[t + v] : zero;
+#pragma unroll
+            for (int u = 0; u < U; ++u) acc[u].add_prod(coef, e[v][u]);
+          }
+        }
+        const ff2 ekk = ek[k];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
           const int j = c.lane + 32 * u;
-          if (u < U - 1 || j < K) acc[u].add_prod(coef, e[j]);
+          S[rr][u] = u < U - 1 || j < K ? ff_fma(acc[u].value(), m.invW_ff[j], j == k ? rf : zero) : zero;
+          accT[u].add_prod(ekk, S[rr][u]);
         }
+        accT0.add_prod(ekk, A1[k]);
       }
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int j = c.lane + 32 * u;
-      if (u < U - 1 || j < K) row[j] = ff_fma(acc[u].value(), m.invW_ff[j], j == k ? rf : zero);
+      if (u < U - 1 || j < K) {
+        ff2* o = A1 + (size_t)(1 + j) * ld0 + k0;
+        if (RG % 2 == 0 && c.i0 != 0) {  // the slot: aligned and padded columns
+#pragma unroll
+          for (int rr = 0; rr < RG; rr += 2)
+            if (k0 + rr < K)
+              *reinterpret_cast<float4*>(o + rr) = make_float4(S[rr][u].hi, S[rr][u].lo, S[rr + 1 < RG ? rr + 1 : rr][u].hi,
+                                                               S[rr + 1 < RG ? rr + 1 : rr][u].lo);
+        } else {
+#pragma unroll
+          for (int rr = 0; rr < RG; ++rr)
+            if (k0 + rr < K) o[rr] = S[rr][u];
+        }
+      }
     }
+  }
+  // the warp's share of the temperature row: entry j (0: temperature column) at warp n + j
+  ff2* tp = reinterpret_cast<ff2*>(c.rr()) + c.warp * (K + 1);
+  if (c.lane == 0) tp[0] = accT0.value();
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int j = c.lane + 32 * u;
+    if (u < U - 1 || j < K) tp[1 + j] = accT[u].value();
   }
 }
 
@@ -1421,63 +1712,67 @@ template <int NW, bool JO>
 __device__ void assemble_ff(const DevMech& m, Cta<NW>& c, const Scal& s, const double* f, double fac, ff2* A) {
   constexpr int NT = NW * 32;
   constexpr double SG = JO ? 1.0 : -1.0;
-  const int K = m.K, n = K + 1, ld = odd_ld(n);
+  const int K = m.K, n = K + 1, ld0 = c.ld0;
   const ff2 zero = {0.0f, 0.0f};
   const ff2 rf = JO ? zero : ff_split(fac);
-  ff2* ek = reinterpret_cast<ff2*>(c.ek);
-  ff2* beta = reinterpret_cast<ff2*>(c.akT);
-  const ff2* dq = reinterpret_cast<const ff2*>(c.dqs);
+  ff2* ek = reinterpret_cast<ff2*>(c.ek());
+  ff2* beta = reinterpret_cast<ff2*>(c.akT());
+  const ff2* dq = reinterpret_cast<const ff2*>(c.dqs());
   // (1) species pass
   const double eT = kRc * s.T * s.icpm, wr = s.Wbar * s.irho;
+#pragma unroll 1
   for (int k = c.tid; k < K; k += NT) {
-    ek[k] = ff_split(c.hRT[k] * eT * m.invW[k]);
-    const double Wk = m.W[k], dk = c.dk[k], fk = f[1 + k];
-    A[(1 + k) * ld] = ff_split(SG * (Wk * s.irho * (c.akT[k] - dk * s.invT) + fk * s.invT));
+    ek[k] = ff_split(c.hRT()[k] * eT * c.iW()[k]);
+    const double Wk = m.W[k], dk = c.dk()[k], fk = f[1 + k];
+    A[c.i0 + 1 + k] = ff_split(SG * (Wk * s.irho * (c.akT()[k] - dk * s.invT) + fk * s.invT));
     beta[k] = ff_split(SG * (fk * s.Wbar - Wk * wr * dk));  // beta_k (a_kT is consumed)
   }
+  mass_action_sums<NW, ff_sum>(
+      m, c,
+      [&](ff_sum& a, int i, unsigned sg) {
+        const ff2 d = dq[i];
+        a.add({__uint_as_float(__float_as_uint(d.hi) ^ sg), __uint_as_float(__float_as_uint(d.lo) ^ sg)});
+      },
+      [&](int k, int j, const ff_sum& a) { c.pair(k, j) = a.value(); });
+  __syncthreads();
   {
-    const int v = NT == 64 ? 0 : NT == 128 ? 1 : 2;
-    const int2* se = m.js_ent[v] + c.tid;
-    const ff2* sn = m.js_nu_ff[v] + c.tid;
-    const int rounds = m.js_rounds[v];
-    ff_sum a;
-    for (int r = 0; r < rounds; ++r) {
-      const int2 e = se[r * NT];
-      if (e.x >= 0) {
-        const ff2 w = sn[r * NT];
-        a.add_prod(JO ? w : ff_neg(w), dq[e.x]);
-      }
-      if (e.y >= 0) {
-        A[e.y] = a.value();
-        a = ff_sum();
-      }
+    // third-body coefficients (tr_ptr[K] <= 4 n_tb, dq holds 4 I pairs)
+    const ff2* Pf = reinterpret_cast<const ff2*>(c.P());
+    ff2* cf = reinterpret_cast<ff2*>(c.dqs());
+    const int nt = m.tr_ptr[K];
+#pragma unroll 1
+    for (int t = c.tid; t < nt; t += NT) {
+      const ff2 tn = m.tr_nu_ff[t];
+      cf[t] = ff_mul(JO ? tn : ff_neg(tn), Pf[m.tr_ent[t].x]);
     }
   }
   __syncthreads();
   // (2) species rows
   switch ((K + 31) >> 5) {
-    case 1: assemble_rows_ff<NW, JO, 1>(m, c, A, K, ld, rf); break;
-    case 2: assemble_rows_ff<NW, JO, 2>(m, c, A, K, ld, rf); break;
-    case 3: assemble_rows_ff<NW, JO, 3>(m, c, A, K, ld, rf); break;
-    case 4: assemble_rows_ff<NW, JO, 4>(m, c, A, K, ld, rf); break;
-    case 5: assemble_rows_ff<NW, JO, 5>(m, c, A, K, ld, rf); break;
-    case 6: assemble_rows_ff<NW, JO, 6>(m, c, A, K, ld, rf); break;
-    case 7: assemble_rows_ff<NW, JO, 7>(m, c, A, K, ld, rf); break;
-    default: assemble_rows_ff<NW, JO, 8>(m, c, A, K, ld, rf); break;
+    case 1: assemble_rows_ff<NW, JO, 1, 4>(m, c, A, K, rf); break;
+    case 2: assemble_rows_ff<NW, JO, 2, 4>(m, c, A, K, rf); break;
+    case 3: assemble_rows_ff<NW, JO, 3, 2>(m, c, A, K, rf); break;
+    case 4: assemble_rows_ff<NW, JO, 4, 2>(m, c, A, K, rf); break;
+    case 5: assemble_rows_ff<NW, JO, 5, 1>(m, c, A, K, rf); break;
+    case 6: assemble_rows_ff<NW, JO, 6, 1>(m, c, A, K, rf); break;
+    case 7: assemble_rows_ff<NW, JO, 7, 1>(m, c, A, K, rf); break;
+    default: assemble_rows_ff<NW, JO, 8, 1>(m, c, A, K, rf); break;
   }
   __syncthreads();
-  // (3) temperature row, as in assemble()
+  // (3) temperature row, as in assemble(), from the warps' shares
   const double ft = s.fT * s.icpm;
-  for (int j = NT - 1 - c.tid; j < n; j += NT) {
-    ff_sum sum;
-    for (int k = 0; k < K; ++k) sum.add_prod(ek[k], A[(1 + k) * ld + j]);
-    const ff2 acc = sum.value();
+  const ff2* tp = reinterpret_cast<const ff2*>(c.rr());
+#pragma unroll 1
+  for (int j = c.tid; j < n; j += NT) {
+    ff2 acc = tp[j];
+#pragma unroll
+    for (int w = 1; w < NW; ++w) acc = ff_add(acc, tp[w * n + j]);
     ff2 v;
     if (j == 0)
       v = ff_sub(ff_sub(rf, acc), ff_split(SG * (s.Scpw * s.irho * s.icpm + ft * s.dcpm)));
     else
-      v = ff_sub(ff_sub(ff_mul(rf, ek[j - 1]), acc), ff_split(SG * ft * c.cpR[j - 1] * kRc * m.invW[j - 1]));
-    A[j] = v;
+      v = ff_sub(ff_sub(ff_mul(rf, ek[j - 1]), acc), ff_split(SG * ft * c.cpR()[j - 1] * kRc * c.iW()[j - 1]));
+    A[j * ld0 + c.i0] = v;
   }
   __syncthreads();
 }
@@ -1524,14 +1819,15 @@ template <int NW, class R>
 __device__ int lu_factor(Cta<NW>& c, R* a, int n, bool pivot = true) {
   constexpr int NT = NW * 32;
   const int ld = odd_ld(n);
-  float* pmax = reinterpret_cast<float*>(c.red + SC_PIV);
-  int* pidx = reinterpret_cast<int*>(c.red + SC_PIV + NW);
-  double* spinv = c.red + SC_INVP;
+  float* pmax = reinterpret_cast<float*>(c.red() + SC_PIV);
+  int* pidx = reinterpret_cast<int*>(c.red() + SC_PIV + NW);
+  double* spinv = c.red() + SC_INVP;
   int info = 0;
   // candidates for column 0
   {
     float v = -1.0f;
     int bi = n;
+#pragma unroll 1
     for (int i = c.tid; i < n; i += NT) {
       const float x = fabsf((float)a[i * ld]);
       if (x > v || (x == v && i < bi)) { v = x; bi = i; }
@@ -1539,15 +1835,17 @@ __device__ int lu_factor(Cta<NW>& c, R* a, int n, bool pivot = true) {
     warp_argmax_store(v, bi, c.lane, pmax, pidx, c.warp);
   }
   __syncthreads();
+#pragma unroll 1
   for (int k = 0; k < n; ++k) {
     int p = pivot ? pivot_reduce<NW>(c, pmax, pidx, n) : k;  // no pivoting: the diagonal
     if (p >= n) p = k;  // a column of NaN: the zero-pivot path below
     if (c.tid == 0) {
-      c.piv[k] = p;
+      c.piv()[k] = p;
       const double pv = (double)a[p * ld + k];
       spinv[0] = pv != 0.0 && isfinite(pv) ? 1.0 / pv : 0.0;
     }
     if (p != k)
+#pragma unroll 1
       for (int j = c.tid; j < n; j += NT) {
         const R t = a[k * ld + j];
         a[k * ld + j] = a[p * ld + j];
@@ -1558,10 +1856,12 @@ __device__ int lu_factor(Cta<NW>& c, R* a, int n, bool pivot = true) {
     if (invp == R(0) && info == 0) info = k + 1;
     float v = -1.0f;
     int bi = n;
+#pragma unroll 1
     for (int i = k + 1 + c.warp; i < n; i += NW) {
       const R l = a[i * ld + k] * invp;
       __syncwarp();
       if (c.lane == 0) a[i * ld + k] = l;
+#pragma unroll 1
       for (int j = k + 1 + c.lane; j < n; j += 32) {
         const R nv = a[i * ld + j] - l * a[k * ld + j];
         a[i * ld + j] = nv;
@@ -1576,15 +1876,17 @@ __device__ int lu_factor(Cta<NW>& c, R* a, int n, bool pivot = true) {
   }
   // composed permutation: position i of the pivoted system holds original row perm[i]
   if (c.tid == 0) {
-    for (int i = 0; i < n; ++i) c.perm[i] = i;
+    for (int i = 0; i < n; ++i) c.perm()[i] = i;
+#pragma unroll 1
     for (int k = 0; k < n; ++k) {
-      const int p = c.piv[k];
-      const int t = c.perm[k];
-      c.perm[k] = c.perm[p];
-      c.perm[p] = t;
+      const int p = c.piv()[k];
+      const int t = c.perm()[k];
+      c.perm()[k] = c.perm()[p];
+      c.perm()[p] = t;
     }
   }
-  for (int i = c.tid; i < n; i += NT) c.invd[i] = 1.0 / (double)a[i * ld + i];
+#pragma unroll 1
+  for (int i = c.tid; i < n; i += NT) c.invd()[i] = 1.0 / (double)a[i * ld + i];
   __syncthreads();
   return info;
 }
@@ -1593,18 +1895,22 @@ __device__ int lu_factor(Cta<NW>& c, R* a, int n, bool pivot = true) {
 template <class R>
 __device__ void lu_solve_warp(const R* a, int n, const double* invd, R* x, int lane) {
   const int ld = odd_ld(n);
+#pragma unroll 1
   for (int i0 = 0; i0 < n; i0 += 32) {
     const int i = i0 + lane;
     const int jend = min(i0 + 32, n);
     R xi = i < n ? x[i] : R(0);
+#pragma unroll 1
     for (int j = i0; j < jend; ++j) {
       const R xj = __shfl_sync(FULLMASK, xi, j - i0);
       if (i > j && i < n) xi -= a[i * ld + j] * xj;
     }
     if (i < n) x[i] = xi;
     __syncwarp();
+#pragma unroll 1
     for (int r = i0 + 32 + lane; r < n; r += 32) {
       R sacc = R(0);
+#pragma unroll 1
       for (int j = i0; j < jend; ++j) sacc += a[r * ld + j] * x[j];
       x[r] -= sacc;
     }
@@ -1621,6 +1927,7 @@ __device__ void lu_solve_warp(const R* a, int n, const double* invd, R* x, int l
     }
     if (i < i1) x[i] = xi;
     __syncwarp();
+#pragma unroll 1
     for (int r = lane; r < i0; r += 32) {
       R sacc = R(0);
       for (int j = i0; j < i1; ++j) sacc += a[r * ld + j] * x[j];
@@ -1639,13 +1946,14 @@ template <int NW>
 __device__ int gj_invert(Cta<NW>& c, float* a, int n) {
   constexpr int NT = NW * 32;
   const int ld = odd_ld(n);
-  float* pmax = reinterpret_cast<float*>(c.red + SC_PIV);
-  int* pidx = reinterpret_cast<int*>(c.red + SC_PIV + NW);
-  float* pr = reinterpret_cast<float*>(c.rr);  // normalised pivot row
+  float* pmax = reinterpret_cast<float*>(c.red() + SC_PIV);
+  int* pidx = reinterpret_cast<int*>(c.red() + SC_PIV + NW);
+  float* pr = reinterpret_cast<float*>(c.rr());  // normalised pivot row
   int info = 0;
   {
     float v = -1.0f;
     int bi = n;
+#pragma unroll 1
     for (int i = c.tid; i < n; i += NT) {
       const float x = fabsf(a[i * ld]);
       if (x > v || (x == v && i < bi)) { v = x; bi = i; }
@@ -1653,14 +1961,16 @@ __device__ int gj_invert(Cta<NW>& c, float* a, int n) {
     warp_argmax_store(v, bi, c.lane, pmax, pidx, c.warp);
   }
   __syncthreads();
+#pragma unroll 1
   for (int k = 0; k < n; ++k) {
     int p = pivot_reduce<NW>(c, pmax, pidx, n);
     if (p >= n) p = k;
     const float pv = a[p * ld + k];
     const float pinv = (pv != 0.0f && isfinite(pv)) ? 1.0f / pv : 0.0f;
     if (pinv == 0.0f && info == 0) info = k + 1;
-    if (c.tid == 0) c.piv[k] = p;
+    if (c.tid == 0) c.piv()[k] = p;
     // interchange rows k and p; the new row k, normalised, goes to the copy
+#pragma unroll 1
     for (int j = c.tid; j < n; j += NT) {
       const float rk = a[k * ld + j], rp = a[p * ld + j];
       if (p != k) a[p * ld + j] = rk;
@@ -1671,13 +1981,16 @@ __device__ int gj_invert(Cta<NW>& c, float* a, int n) {
     const int own = cn & 31;           // lane owning column cn in the loops below
     float v = -1.0f;
     int bi = n;
+#pragma unroll 1
     for (int i = c.warp; i < n; i += NW) {
       if (i == k) {
+#pragma unroll 1
         for (int j = c.lane; j < n; j += 32) a[k * ld + j] = pr[j];
         continue;
       }
       const float fct = a[i * ld + k];
       __syncwarp();
+#pragma unroll 1
       for (int j = c.lane; j < n; j += 32) {
         const float nv = (j == k ? 0.0f : a[i * ld + j]) - fct * pr[j];
         a[i * ld + j] = nv;
@@ -1692,9 +2005,11 @@ __device__ int gj_invert(Cta<NW>& c, float* a, int n) {
     __syncthreads();
   }
   // column interchanges in reverse order; each thread owns whole rows
+#pragma unroll 1
   for (int i = c.tid; i < n; i += NT)
+#pragma unroll 1
     for (int k = n - 1; k >= 0; --k) {
-      const int p = c.piv[k];
+      const int p = c.piv()[k];
       if (p != k) {
         const float t = a[i * ld + k];
         a[i * ld + k] = a[i * ld + p];
@@ -1708,184 +2023,260 @@ __device__ int gj_invert(Cta<NW>& c, float* a, int n) {
 // Gauss-Jordan inverse (FP32) with the matrix in registers, by columns: warp w owns
 // the columns j = w + NW c (c < CC), lane l the rows l + 32 s (s < RS). Partial
 // pivoting by index (the unused row with the largest |a_ik|, lowest row index on
-// ties; rows are not moved, the k-th pivot row is recorded instead). The warp
-// owning column k searches it, publishes the pivot row p, 1/a_pk and the column (the multipliers) through
-// shared memory (double-buffered), and every warp then broadcasts the pivot row's
-// values of its own columns by warp shuffles and updates them: one CTA barrier per
-// column. Column k is first replaced by the unit vector e_p, so it ends up holding
-// column k of the inverse (in-place Gauss-Jordan). The inverse is written back as
+// ties; rows are not moved, the k-th pivot row is recorded instead). The warp owning
+// column k publishes it through shared memory (double-buffered); every warp searches the
+// pivot in it, broadcasts the pivot row's values of its own columns by warp shuffles and
+// updates them. Column k ends up holding column k of the inverse (in-place Gauss-Jordan).
+// A pivot row keeps its values and takes its factor 1/a_pk at the end: later steps
+// subtract multiples of other rows from it, which commutes with the factor, so it is just
+// a row whose multiplier is zero in its own step. The columns rotate through the registers
+// once per NW pivots, so that the current one is always c = 0 and no register is selected
+// by a run-time index.
+// The chain from one pivot to the next (search column k, update column k + 1, publish it)
+// is all that the warps wait for: the owner of column k + 1 updates it ahead of its other
+// columns and only arrives at the barrier the others wait on; and as every warp searches
+// for itself, the chain holds one pass through shared memory and one barrier. (n = 55 on
+// four warps, alone on an SM, cycles a pivot: 908 with a search by the owner after all
+// updates; 811 with the owner ahead; 692 with the rotation and the deferred factor; the
+// search by the owner alone took 540 of these.) The inverse is written as
 // inv[Pinv[i]][P[j]] = W[i][j] (P = pivot rows in step order). Requires n <= 32 RS
-// and n <= NW CC. Returns 0 or 1 + k for a zero pivot.
-template <int NW, int RS, int CC>
-__device__ int gj_invert_wc(Cta<NW>& c, float* A, int n) {
+// and n <= NW CC. src: the matrix by columns, leading dimension ld0. Returns 0 or 1 + k
+// for a zero pivot.
+template <int NW, int RS, int CC, class A>
+__device__ int gj_invert_wc(Cta<NW>& c, const A* src, int ld0, float* inv, int n) {
   const int ld = odd_ld(n);
   const int lane = c.lane, wp = c.warp;
-  float* pcol = reinterpret_cast<float*>(c.u);          // [2][n] multipliers (u: 6 n doubles)
-  int* pp = reinterpret_cast<int*>(c.red + SC_PIV);     // [2] pivot rows
-  float* pinvb = reinterpret_cast<float*>(pp + 2);      // [2] pivot reciprocals
+  float* pcol = reinterpret_cast<float*>(c.u());  // [2][n] the published columns (u: 6 n doubles)
   float a[RS][CC];
 #pragma unroll
-  for (int s = 0; s < RS; ++s)
+  for (int cc = 0; cc < CC; ++cc)
 #pragma unroll
-    for (int cc = 0; cc < CC; ++cc) {
+    for (int s = 0; s < RS; ++s) {
       const int i = lane + 32 * s, j = wp + NW * cc;
-      a[s][cc] = (i < n && j < n) ? A[i * ld + j] : 0.0f;
+      a[s][cc] = (i < n && j < n) ? to_float(src[(size_t)j * ld0 + i]) : 0.0f;
     }
   unsigned used = 0u;  // bit s: row lane + 32 s is a pivot row already
-  // owner warp of column k: search, then publish the pivot and the column
-  auto search = [&](int k, int buf) {
-    const int ck = k / NW;
-    float v[RS];
+  float scale[RS];     // 1/a_pk of the pivot rows
 #pragma unroll
-    for (int s = 0; s < RS; ++s) v[s] = 0.0f;
+  for (int s = 0; s < RS; ++s) scale[s] = 0.0f;
+  if (wp == 0) {
 #pragma unroll
-    for (int cc = 0; cc < CC; ++cc)
-      if (cc == ck) {
-#pragma unroll
-        for (int s = 0; s < RS; ++s) v[s] = a[s][cc];
-      }
-    // argmax of |a_ik| over the unused rows, lowest row on ties, NaN never chosen: the
-    // bit pattern of a non-negative float orders like its value, so key = bits + 1
-    // (0: no candidate) goes through one warp max-reduction; the first row slot, then
-    // the lowest lane, holding the maximum is the lowest row index that has it
-    unsigned key[RS];
+    for (int s = 0; s < RS; ++s)
+      if (lane + 32 * s < n) pcol[lane + 32 * s] = a[s][0];
+  }
+#pragma unroll 1
+  for (int i = c.tid; i < n; i += NW * 32) c.perm()[i] = i;  // (a zero pivot leaves entries unset below)
+  __syncthreads();
+  int info = 0;
+#pragma unroll 1
+  for (int k = 0; k < n; ++k) {
+    const int buf = k & 1, k1 = k + 1;
+    const bool own_next = k1 < n && wp == k1 % NW;
+    // pivot of column k: argmax of |v| over the unused rows, lowest row on ties, NaN never
+    // chosen: the bit pattern of a non-negative float orders like its value, so key =
+    // bits + 1 (0: no candidate) goes through one warp max-reduction; every lane forms the
+    // reciprocal of its own candidate (one Newton step on the approximate reciprocal)
+    float v[RS], best = 0.0f;
     unsigned kmax = 0u;
+    int bs = 0;
 #pragma unroll
     for (int s = 0; s < RS; ++s) {
       const int i = lane + 32 * s;
+      v[s] = pcol[buf * n + min(i, n - 1)];
       const float x = fabsf(v[s]);
-      key[s] = (i < n && !((used >> s) & 1u) && !isnan(x)) ? __float_as_uint(x) + 1u : 0u;
-      kmax = max(kmax, key[s]);
+      const unsigned key = (i < n && !((used >> s) & 1u) && !isnan(x)) ? __float_as_uint(x) + 1u : 0u;
+      best = key > kmax ? v[s] : best;
+      bs = key > kmax ? s : bs;
+      kmax = max(key, kmax);
     }
     const unsigned km = __reduce_max_sync(FULLMASK, kmax);
-    int bi = n;
-    float bval = 0.0f;
-    if (km != 0u) {
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(best));
+    r = fmaf(r, fmaf(-best, r, 1.0f), r);
+    r = fabsf(r) < 3.4e38f ? r : 0.0f;  // zero pivot (or none): no finite reciprocal
+    unsigned win = __ballot_sync(FULLMASK, kmax == km);
+    if (RS > 1 && (win & (win - 1u))) {  // a tie: the lowest row, i.e. the lowest slot first
 #pragma unroll
-      for (int s = 0; s < RS; ++s) {
-        const unsigned b = __ballot_sync(FULLMASK, key[s] == km);
-        if (bi == n && b != 0u) {
-          const int l = __ffs(b) - 1;
-          bi = l + 32 * s;
-          bval = __shfl_sync(FULLMASK, v[s], l);
-        }
+      for (int s = RS - 1; s >= 0; --s) {
+        const unsigned w = __ballot_sync(FULLMASK, kmax == km && bs == s);
+        if (w) win = w;
       }
     }
-#pragma unroll
-    for (int s = 0; s < RS; ++s)
-      if (lane + 32 * s < n) pcol[buf * n + lane + 32 * s] = v[s];
-    if (lane == 0) {
-      const bool ok = bi < n && bval != 0.0f && isfinite(bval);
-      pp[buf] = bi < n ? bi : k;  // no candidate (NaN column): a safe index, zero pivot
-      pinvb[buf] = ok ? 1.0f / bval : 0.0f;
-    }
-  };
-  if (wp == 0) search(0, 0);
-  __syncthreads();
-  int info = 0;
-  for (int k = 0; k < n; ++k) {
-    const int buf = k & 1;
-    const int p = pp[buf];
-    const float pinv = pinvb[buf];
+    const int pl = __ffs(win) - 1;
+    const float pinv = __shfl_sync(FULLMASK, r, pl);
+    const int ps = RS > 1 ? __shfl_sync(FULLMASK, bs, pl) : 0;
+    const int p = pl + 32 * ps;  // (a column of NaN: some row in range, zero pivot)
     if (pinv == 0.0f && info == 0) info = k + 1;
-    if (c.tid == 0) c.piv[k] = p;
-    const int ps = p >> 5, pl = p & 31;
-    float f[RS];
+    if (c.tid == 0) c.piv()[k] = p;
+    float fp[RS];  // multipliers over the pivot: a_ij -= (a_ik / a_pk) a_pj
     bool isp[RS];
 #pragma unroll
     for (int s = 0; s < RS; ++s) {
-      isp[s] = lane + 32 * s == p;
-      f[s] = lane + 32 * s < n ? pcol[buf * n + lane + 32 * s] : 0.0f;
+      isp[s] = lane == pl && s == ps;
+      fp[s] = isp[s] || lane + 32 * s >= n ? 0.0f : v[s] * pinv;
+      used |= isp[s] ? 1u << s : 0u;
+      scale[s] = isp[s] ? pinv : scale[s];
     }
-    // column k becomes e_p (it then receives column k of the inverse)
+    auto pivot_row = [&](const float (&x)[RS]) {  // the pivot row's entry of a column
+      float r = x[0];
+#pragma unroll
+      for (int s = 1; s < RS; ++s) r = ps == s ? x[s] : r;
+      return __shfl_sync(FULLMASK, r, pl);
+    };
+    // barrier 2 + (k1 & 1): column k + 1 is published
+    if (own_next) {
+      const bool next_group = k1 % NW == 0;  // the columns rotate after this step
+      float w[RS];
+#pragma unroll
+      for (int s = 0; s < RS; ++s) w[s] = next_group ? a[s][CC > 1 ? 1 : 0] : a[s][0];
+      const float pr = pivot_row(w);
+#pragma unroll
+      for (int s = 0; s < RS; ++s)
+        if (lane + 32 * s < n) pcol[(k1 & 1) * n + lane + 32 * s] = fmaf(-fp[s], pr, w[s]);
+      __syncwarp();
+      if (k1 & 1) asm volatile("bar.arrive 3, %0;" ::"n"(NW * 32) : "memory");
+      else asm volatile("bar.arrive 2, %0;" ::"n"(NW * 32) : "memory");
+    }
+    // all broadcasts first (their latencies overlap), then the updates
+    float pr[CC];
+#pragma unroll
+    for (int cc = 0; cc < CC; ++cc) {
+      float x[RS];
+#pragma unroll
+      for (int s = 0; s < RS; ++s) x[s] = a[s][cc];
+      pr[cc] = pivot_row(x);
+    }
+#pragma unroll
+    for (int cc = 0; cc < CC; ++cc)
+#pragma unroll
+      for (int s = 0; s < RS; ++s) a[s][cc] = fmaf(-fp[s], pr[cc], a[s][cc]);
+    // column k, as from the unit vector e_p, becomes column k of the inverse
     if (wp == k % NW) {
-      const int ck = k / NW;
 #pragma unroll
-      for (int cc = 0; cc < CC; ++cc)
-        if (cc == ck) {
-#pragma unroll
-          for (int s = 0; s < RS; ++s) a[s][cc] = isp[s] ? 1.0f : 0.0f;
-        }
+      for (int s = 0; s < RS; ++s) a[s][0] = isp[s] ? 1.0f : -fp[s];
     }
+    if (k1 % NW == 0) {
 #pragma unroll
-    for (int cc = 0; cc < CC; ++cc) {
-      float src = a[0][cc];
+      for (int s = 0; s < RS; ++s) {
+        const float t = a[s][0];
 #pragma unroll
-      for (int s = 1; s < RS; ++s) src = ps == s ? a[s][cc] : src;
-      const float pr = __shfl_sync(FULLMASK, src, pl) * pinv;  // normalised pivot row
-#pragma unroll
-      for (int s = 0; s < RS; ++s) a[s][cc] = isp[s] ? pr : fmaf(-f[s], pr, a[s][cc]);
+        for (int cc = 0; cc + 1 < CC; ++cc) a[s][cc] = a[s][cc + 1];
+        a[s][CC - 1] = t;
+      }
     }
-#pragma unroll
-    for (int s = 0; s < RS; ++s)
-      if (isp[s]) used |= 1u << s;
-    const int k1 = k + 1;
-    if (k1 < n && wp == k1 % NW) search(k1, k1 & 1);
-    __syncthreads();
+    if (k1 < n && !own_next) {
+      if (k1 & 1) asm volatile("bar.sync 3, %0;" ::"n"(NW * 32) : "memory");
+      else asm volatile("bar.sync 2, %0;" ::"n"(NW * 32) : "memory");
+    }
   }
-  // inverse permutation of the pivot rows, then the scatter into the true inverse
-  for (int k = c.tid; k < n; k += NW * 32) c.perm[c.piv[k]] = k;
   __syncthreads();
+  // inverse permutation of the pivot rows, then the scatter into the true inverse
+#pragma unroll 1
+  for (int k = c.tid; k < n; k += NW * 32) c.perm()[c.piv()[k]] = k;
+  __syncthreads();
+  const int rot = n / NW % CC;  // rotations made
 #pragma unroll
-  for (int s = 0; s < RS; ++s)
+  for (int s = 0; s < RS; ++s) {
+    const int i = lane + 32 * s;
+    float* row = inv + (i < n ? c.perm()[i] * ld : 0);
 #pragma unroll
     for (int cc = 0; cc < CC; ++cc) {
-      const int i = lane + 32 * s, j = wp + NW * cc;
-      if (i < n && j < n) A[c.perm[i] * ld + c.piv[j]] = a[s][cc];
+      const int j = wp + NW * (cc + rot < CC ? cc + rot : cc + rot - CC);
+      if (i < n && j < n) row[c.piv()[j]] = a[s][cc] * scale[s];
     }
+  }
   __syncthreads();
   return info;
 }
 
-// Solve M x = b for the FP64 right-hand side b; x written as double.
+// One row of the FP32 inverse times xf (16-byte aligned).
+__device__ __forceinline__ float inv_row(const float* row, const float* xf, int n) {
+  float a0 = 0.0f, a1 = 0.0f, a2 = 0.0f, a3 = 0.0f;
+  int j = 0;
+#pragma unroll 2
+  for (; j + 4 <= n; j += 4) {
+    const float4 x = *reinterpret_cast<const float4*>(xf + j);
+    a0 = fmaf(row[j], x.x, a0);
+    a1 = fmaf(row[j + 1], x.y, a1);
+    a2 = fmaf(row[j + 2], x.z, a2);
+    a3 = fmaf(row[j + 3], x.w, a3);
+  }
+  for (; j < n; ++j) a0 = fmaf(row[j], xf[j], a0);
+  return (a0 + a1) + (a2 + a3);
+}
+
+// Solve M x = b for the FP64 right-hand side b; x written as double. b's entry i was
+// written by the thread i (mod the CTA) that reads it here.
 // FP64: LU forward/back substitution. Otherwise: x = M32^-1 b with the FP32
-// inverse, then `ir` sweeps of r = b - M0 x (FP64, against the assembled matrix
-// M0) and x += M32^-1 r. One thread per row in every matrix-vector product.
+// inverse, then `ir` sweeps of r = b - M0 x (about 48 bits, against the assembled matrix
+// M0) and x += M32^-1 r. One thread per row of the inverse; a residual row is shared by
+// up to three threads (each a range of columns), since a row costs 14 FP32 instructions
+// per entry and n rows leave half of the CTA's warps without one.
 template <int NW, int PREC>
 __device__ void solve(Cta<NW>& c, int n, const double* b, double* x, int ir) {
   constexpr int NT = NW * 32;
   using P = Policy<PREC>;
   if constexpr (!P::IR) {
-    for (int i = c.tid; i < n; i += NT) x[i] = b[c.perm[i]];
     __syncthreads();
-    if (c.warp == Cta<NW>::SW) lu_solve_warp<double>(reinterpret_cast<double*>(c.M), n, c.invd, x, c.lane);
+#pragma unroll 1
+    for (int i = c.tid; i < n; i += NT) x[i] = b[c.perm()[i]];
+    __syncthreads();
+    if (c.warp == Cta<NW>::SW) lu_solve_warp<double>(reinterpret_cast<double*>(c.M()), n, c.invd(), x, c.lane);
     __syncthreads();
   } else {
     using A = typename P::ASM;
-    const float* Ai = reinterpret_cast<const float*>(c.M);
-    const A* M0 = reinterpret_cast<const A*>(c.M0);
-    float* xf = reinterpret_cast<float*>(c.sc);  // scratch vector reused as float
-    ff2* xq = reinterpret_cast<ff2*>(c.rr);      // x as float-float pairs (rr is free in the solves)
-    const int ld = odd_ld(n);
+    const float* Ai = reinterpret_cast<const float*>(c.M());
+    const A* M0 = reinterpret_cast<const A*>(c.M0) + c.i0;
+    float* xf = reinterpret_cast<float*>(c.sc());  // scratch vector reused as float
+    ff2* xq = reinterpret_cast<ff2*>(c.rr());      // x as float-float pairs (rr is free in the solves)
+    ff2* part = reinterpret_cast<ff2*>(c.yn());    // partial residuals (yn and ys are free in the solves)
+    const int ld = odd_ld(n), ld0 = c.ld0;
+    const int nwr = (n + 31) >> 5;                    // warps that hold a row each lane
+    const int np = nwr >= NW ? 1 : min(3, NW / nwr);  // threads per row
+    const int cols = (n + np - 1) / np;
+    const int q = np > 1 ? c.warp / nwr : 0;          // this thread's range of columns
+#pragma unroll 1
     for (int i = c.tid; i < n; i += NT) xf[i] = ff_split(b[i]).hi;
     __syncthreads();
-    for (int i = c.tid; i < n; i += NT) {
-      float acc = 0.0f;
-      const float* row = Ai + i * ld;
-      for (int j = 0; j < n; ++j) acc = fmaf(row[j], xf[j], acc);
-      x[i] = f32_to_f64(acc);
-      xq[i] = {acc, 0.0f};
-    }
-    __syncthreads();
-    for (int sweep = 0; sweep < ir; ++sweep) {
-      // Residual rows r = b - M0 x from the last warp down (the first warps carry the
-      // species loops), as a compensated dot product on the FP32 pipe (Ogita, Rump and
-      // Oishi's Dot2: exact products of the hi parts, TwoSum of the running sum, the
+#pragma unroll 1
+    for (int sweep = 0;; ++sweep) {
+#pragma unroll 1
+      for (int i = c.tid; i < n; i += NT) {
+        const float acc = inv_row(Ai + i * ld, xf, n);
+        if (sweep == 0) {
+          x[i] = f32_to_f64(acc);
+          xq[i] = {acc, 0.0f};
+        } else {
+          x[i] += f32_to_f64(acc);
+          if (sweep < ir) xq[i] = ff_split(x[i]);
+        }
+      }
+      __syncthreads();
+      if (sweep == ir) break;
+      // Residual rows r = b - M0 x as a compensated dot product on the FP32 pipe (Ogita,
+      // Rump and Oishi's Dot2: exact products of the hi parts, TwoSum of the running sum, the
       // rounding errors and cross terms gathered in a second accumulator): as accurate as
       // a sum in about 48-bit arithmetic, then rounded to FP32 for the correction solve.
-      for (int i = NT - 1 - c.tid; i < n; i += NT) {
-        const ff2 bi = ff_split(b[i]);
-        float sh = bi.hi, sl = bi.lo;
-        const A* row = M0 + i * ld;
-        for (int j = 0; j < n; ++j) {
+      // M0 lies by columns: a warp reads 32 consecutive rows.
+      float sh = 0.0f, sl = 0.0f;
+#pragma unroll 1
+      for (int i = np > 1 ? c.tid - q * nwr * 32 : c.tid; i < n && q < np; i += np > 1 ? n : NT) {
+        if (q == 0) {
+          const ff2 bi = ff_split(b[i]);
+          sh = bi.hi;
+          sl = bi.lo;
+        }
+        const int j1 = min(n, (q + 1) * cols);
+#pragma unroll 4
+        for (int j = q * cols; j < j1; ++j) {
           const ff2 xj = xq[j];
           float mh, ml = 0.0f;
           if constexpr (std::is_same<A, ff2>::value) {
-            const ff2 mj = row[j];
+            const ff2 mj = M0[j * ld0 + i];
             mh = mj.hi;
             ml = mj.lo;
           } else {
-            mh = row[j];
+            mh = M0[j * ld0 + i];
           }
           const float p = __fmul_rn(mh, xj.hi);
           float pe = fmaf(mh, xj.hi, -p);
@@ -1895,17 +2286,18 @@ __device__ void solve(Cta<NW>& c, int n, const double* b, double* x, int ir) {
           sh = t.hi;
           sl = __fadd_rn(sl, __fsub_rn(t.lo, pe));
         }
-        xf[i] = __fadd_rn(sh, sl);
+        if (q > 0) part[(q - 1) * n + i] = {sh, sl};
+        else if (np == 1) xf[i] = __fadd_rn(sh, sl);
       }
       __syncthreads();
-      for (int i = c.tid; i < n; i += NT) {
-        float acc = 0.0f;
-        const float* row = Ai + i * ld;
-        for (int j = 0; j < n; ++j) acc = fmaf(row[j], xf[j], acc);
-        x[i] += f32_to_f64(acc);
-        if (sweep + 1 < ir) xq[i] = ff_split(x[i]);
+      if (np > 1) {
+        if (c.tid < n) {  // its first range's sum is still in sh + sl
+          ff_sum r(ff2{sh, sl});
+          for (int w = 0; w + 1 < np; ++w) r.add(part[w * n + c.tid]);
+          xf[c.tid] = __fadd_rn(r.s, r.c);
+        }
+        __syncthreads();
       }
-      __syncthreads();
     }
   }
 }
@@ -1914,42 +2306,43 @@ __device__ void solve(Cta<NW>& c, int n, const double* b, double* x, int ir) {
 template <int NW, int PREC>
 __device__ int factor(Cta<NW>& c, int n, bool pivot = true) {
   if constexpr (!Policy<PREC>::IR) {
-    return lu_factor<NW, double>(c, reinterpret_cast<double*>(c.M), n, pivot);
+    return lu_factor<NW, double>(c, reinterpret_cast<double*>(c.M()), n, pivot);
   } else {
-    float* A = reinterpret_cast<float*>(c.M);
+    using A = typename Policy<PREC>::ASM;
+    float* inv = reinterpret_cast<float*>(c.M());
+    const A* src = reinterpret_cast<const A*>(c.M0) + c.i0;
     if constexpr (NW == 4) {
-      if (n <= 56) return gj_invert_wc<4, 2, 14>(c, A, n);
-      if (n <= 64) return gj_invert_wc<4, 2, 16>(c, A, n);
+      if (n <= 32) return gj_invert_wc<4, 1, 8>(c, src, c.ld0, inv, n);
+      if (n <= 56) return gj_invert_wc<4, 2, 14>(c, src, c.ld0, inv, n);
+      if (n <= 64) return gj_invert_wc<4, 2, 16>(c, src, c.ld0, inv, n);
     } else if constexpr (NW == 8) {
-      if (n <= 64) return gj_invert_wc<8, 2, 8>(c, A, n);
-      if (n <= 128) return gj_invert_wc<8, 4, 16>(c, A, n);
+      if (n <= 64) return gj_invert_wc<8, 2, 8>(c, src, c.ld0, inv, n);
+      if (n <= 128) return gj_invert_wc<8, 4, 16>(c, src, c.ld0, inv, n);
     } else if constexpr (NW == 2) {
-      if (n <= 64) return gj_invert_wc<2, 2, 32>(c, A, n);
+      if (n <= 32) return gj_invert_wc<2, 1, 16>(c, src, c.ld0, inv, n);
+      if (n <= 64) return gj_invert_wc<2, 2, 32>(c, src, c.ld0, inv, n);
     }
-    return gj_invert<NW>(c, A, n);
+    const int ld = odd_ld(n);
+#pragma unroll 1
+    for (int j = c.warp; j < n; j += NW)
+#pragma unroll 1
+      for (int i = c.lane; i < n; i += 32) inv[i * ld + j] = to_float(src[(size_t)j * c.ld0 + i]);
+    __syncthreads();
+    return gj_invert<NW>(c, inv, n);
   }
 }
 
 // Assemble the iteration matrix (fac = 1/(h gamma)) or the Jacobian (JO) in the
-// policy's assembly precision, then give the LU its own copy when they differ.
+// policy's assembly precision.
 template <int NW, int PREC, bool JO>
 __device__ void build_matrix(const DevMech& m, Cta<NW>& c, const Scal& s, const double* f, double fac) {
   using P = Policy<PREC>;
-  if constexpr (!P::IR) {
-    assemble<NW, double, JO>(m, c, s, f, fac, c.M);
-  } else {
-    if constexpr (std::is_same<typename P::ASM, ff2>::value)
-      assemble_ff<NW, JO>(m, c, s, f, fac, reinterpret_cast<ff2*>(c.M0));
-    else
-      assemble<NW, typename P::ASM, JO, true>(m, c, s, f, fac, c.M0);
-    if (JO) return;
-    const int n = m.K + 1, ld = odd_ld(n);
-    const typename P::ASM* src = reinterpret_cast<const typename P::ASM*>(c.M0);
-    float* dst = reinterpret_cast<float*>(c.M);
-    for (int i = c.warp; i < n; i += NW)
-      for (int j = c.lane; j < n; j += 32) dst[i * ld + j] = to_float(src[i * ld + j]);
-    __syncthreads();
-  }
+  if constexpr (!P::IR)
+    assemble<NW, double, JO>(m, c, s, f, fac, c.M());
+  else if constexpr (std::is_same<typename P::ASM, ff2>::value)
+    assemble_ff<NW, JO>(m, c, s, f, fac, reinterpret_cast<ff2*>(c.M0));
+  else
+    assemble<NW, typename P::ASM, JO, true, true>(m, c, s, f, fac, c.M0);
 }
 
 // Iteration matrix (FP64 form) from a forward-difference Jacobian, column by column:
@@ -1961,63 +2354,93 @@ template <int NW, bool JO>
 __device__ void fd_matrix(const DevMech& m, Cta<NW>& c, double p, const double* y, const double* f0, double fac) {
   constexpr int NT = NW * 32;
   const int n = m.K + 1, ld = odd_ld(n);
-  double* A = reinterpret_cast<double*>(c.M);
+  double* A = reinterpret_cast<double*>(c.M());
   for (int j = 0; j < n; ++j) {
     const double d = 1.4901161193847656e-8 * fmax(fabs(y[j]), j == 0 ? 1.0 : 1e-6);
-    for (int i = c.tid; i < n; i += NT) c.ys[i] = y[i] + (i == j ? d : 0.0);
+#pragma unroll 1
+    for (int i = c.tid; i < n; i += NT) c.ys()[i] = y[i] + (i == j ? d : 0.0);
     __syncthreads();
-    eval_rhs<NW, false, false>(m, c, c.ys, p, c.fv);
+    eval_rhs<NW, false, false>(m, c, c.ys(), p, c.fv());
     const double id = 1.0 / d;
+#pragma unroll 1
     for (int i = c.tid; i < n; i += NT) {
-      const double J = (c.fv[i] - f0[i]) * id;
+      const double J = (c.fv()[i] - f0[i]) * id;
       A[i * ld + j] = JO ? J : -J + (i == j ? fac : 0.0);
     }
     __syncthreads();
   }
 }
 
-// WRMS norm of e with scale atol + rtol max(|ya|, |yb|). With step_fac, also the
-// step-size factor 0.9 err^(-1/q) (q = 4: RODAS4, 3: ROS34PW2; kFacMax for err = 0);
-// both come from the CTA's last warp.
-template <int NW>
-__device__ double wrms(Cta<NW>& c, int n, const double* e, const double* ya, const double* yb,
-                       double rtol, double atol, double* step_fac = nullptr, int q = 4) {
+// Sum over the CTA of (e_i / (atol + rtol max(|ya_i|, |yb_i|)))^2, finished by fin on warp 0.
+template <int NW, int NO, class F>
+__device__ void scaled_square_sum(Cta<NW>& c, int n, const double* e, const double* ya, const double* yb, double rtol,
+                                  double atol, F fin, double (&out)[NO]) {
   constexpr int NT = NW * 32;
   double part[1] = {0.0};
+#pragma unroll 1
   for (int i = c.tid; i < n; i += NT) {
     const double sc = atol + rtol * fmax(fabs(ya[i]), fabs(yb[i]));
-    const double r = e[i] / sc;
+    const double r = e[i] * xrcp(sc);
     part[0] += r * r;
   }
+  c.reduce(part, warps_for<NW>(n), fin, out);
+}
+
+// WRMS norm of e with scale atol + rtol max(|ya|, |yb|).
+template <int NW>
+__device__ double wrms(Cta<NW>& c, int n, const double* e, const double* ya, const double* yb, double rtol,
+                       double atol) {
+  double o[1];
+  scaled_square_sum(c, n, e, ya, yb, rtol, atol,
+                    [&](const double (&t)[1], double (&r)[1]) { r[0] = sqrt(t[0] / n); }, o);
+  return o[0];
+}
+
+// The error test of a step: the square of the WRMS norm of e, and the step-size factor
+// 0.9 err^(-1/q) (q = 4: RODAS4, 3: ROS34PW2; kFacMax for err = 0) by the fixed-point
+// logarithm and exponential (about 300 cycles on warp 0, where the FP64 roots and
+// division took 2,500).
+template <int NW>
+__device__ double error_test(Cta<NW>& c, int n, const double* e, const double* ya, const double* yb, double rtol,
+                             double atol, double* step_fac, int q) {
   double o[2];
-  c.reduce(part, warps_for<NW>(n), [&](const double (&t)[1], double (&r)[2]) {
-    const double err = sqrt(t[0] / n);
-    r[0] = err;
-    r[1] = err > 0.0 ? kSafety / (q == 4 ? sqrt(sqrt(err)) : cbrt(err)) : kFacMax;
+  const double inv_n = xrcp((double)n);
+  scaled_square_sum(c, n, e, ya, yb, rtol, atol, [&](const double (&t)[1], double (&r)[2]) {
+    const double err2 = t[0] * inv_n;
+    r[0] = err2;
+    const int hx = __double2hiint(err2);
+    if (hx >= 0x00100000 && hx < 0x7ff00000) {
+      const long long l = fx_log(err2, 52);
+      r[1] = kSafety * fx_exp(q == 4 ? -(l >> 3) : -(l / 6), c.xt());
+    } else {
+      r[1] = kFacMax;  // zero or subnormal (a non-finite norm's factor is not used)
+    }
   }, o);
-  if (step_fac) *step_fac = o[1];
+  *step_fac = o[1];
   return o[0];
 }
 
 // Hairer-Wanner starting step (Solving ODEs I, Sec. II.4) in the WRMS norm with
 // scale atol + rtol |y0|, exponent 1/q (the method's embedded order + 1), clamped
 // to dt; a vanishing derivative selects the whole interval. Uses f0 = f(y0)
-// (already in c.f0) and c.ys, c.fv.
+// (already in c.f0()) and c.ys(), c.fv().
 template <int NW, bool FF = false>
 __device__ double starting_step(const DevMech& m, Cta<NW>& c, double p, double dt, double rtol,
                                 double atol, int q = 4) {
   constexpr int NT = NW * 32;
   const int n = m.K + 1;
-  const double d0 = wrms(c, n, c.y, c.y, c.y, rtol, atol);
-  const double d1 = wrms(c, n, c.f0, c.y, c.y, rtol, atol);
+  const double d0 = wrms(c, n, c.y(), c.y(), c.y(), rtol, atol);
+  const double d1 = wrms(c, n, c.f0(), c.y(), c.y(), rtol, atol);
   double ha = (d1 > 1e-300) ? 0.01 * d0 / d1 : dt;
   ha = fmin(ha, dt);
-  for (int i = c.tid; i < n; i += NT) c.ys[i] = c.y[i] + ha * c.f0[i];
+#pragma unroll 1
+  for (int i = c.tid; i < n; i += NT) c.ys()[i] = c.y()[i] + ha * c.f0()[i];
   __syncthreads();
-  eval_rhs<NW, false, FF>(m, c, c.ys, p, c.fv);
-  for (int i = c.tid; i < n; i += NT) c.rr[i] = c.fv[i] - c.f0[i];
+  eval_rhs<NW, false, FF>(m, c, c.ys(), p, c.fv());
+#pragma unroll 1
+  for (int i = c.tid; i < n; i += NT) c.rr()[i] = c.fv()[i] - c.f0()[i];
   __syncthreads();
-  const double d2 = wrms(c, n, c.rr, c.y, c.y, rtol, atol) / ha;
+  const double d2 = wrms(c, n, c.rr(), c.y(), c.y(), rtol, atol) / ha;
   const double mx = fmax(d1, d2);
   const double hb = (mx > 1e-300) ? (q == 4 ? pow(0.01 / mx, 0.25) : cbrt(0.01 / mx)) : dt;
   return fmin(fmin(100.0 * ha, hb), dt);
@@ -2030,6 +2453,7 @@ __device__ void h_cp_mass(const DevMech& m, Cta<NW>& c, double T, const double* 
   constexpr int NT = NW * 32;
   const double invT = 1.0 / T;
   double part[2] = {0.0, 0.0};
+#pragma unroll 1
   for (int k = c.tid; k < m.K; k += NT) {
     const double* a = m.nasa + 36 * k;
     a += (T < a[34]) ? 0 : 17;
@@ -2061,7 +2485,7 @@ __device__ void h_cp_mass(const DevMech& m, Cta<NW>& c, double T, const double* 
   } while (0)
 
 template <int NW, int PREC, int MTH>
-__device__ void integrate_cell(const Job& job, int64_t cell, const IntegrateArgs& args, Cta<NW>& c) {
+__device__ void integrate_cell(const Job& job, int64_t cell, const IntegrateArgs& args, Cta<NW>& c, double* slot) {
   using MT = Meth<MTH>;
   const bool prof = args.phase != nullptr && c.tid == 0;
   long long last_ = prof ? clock64() : 0;
@@ -2072,21 +2496,25 @@ __device__ void integrate_cell(const Job& job, int64_t cell, const IntegrateArgs
   const double p = job.p[cell];
   const double dt = args.dt, rtol = args.rtol, atol = args.atol;
   // load (coalesced over species)
-  if (c.tid == 0) c.y[0] = job.T[cell];
-  for (int k = c.tid; k < K; k += NT) c.y[1 + k] = job.Y[(size_t)cell * K + k];
+  if (c.tid == 0) c.y()[0] = job.T[cell];
+#pragma unroll 1
+  for (int k = c.tid; k < K; k += NT) c.y()[1 + k] = job.Y[(size_t)cell * K + k];
+  c.set_cell(m, p);
+  c.set_matrix(K, slot);
   __syncthreads();
   int status = CHEM_CELL_OK;
   {
     double part[1] = {0.0};
-    for (int i = c.tid; i < n; i += NT) part[0] += isfinite(c.y[i]) ? 0.0 : 1.0;
+#pragma unroll 1
+    for (int i = c.tid; i < n; i += NT) part[0] += isfinite(c.y()[i]) ? 0.0 : 1.0;
     c.sum(part, warps_for<NW>(n));
-    if (part[0] > 0.0 || !(c.y[0] > 0.0) || !(p > 0.0)) status = CHEM_CELL_NONFINITE;
+    if (part[0] > 0.0 || !(c.y()[0] > 0.0) || !(p > 0.0)) status = CHEM_CELL_NONFINITE;
   }
   int steps = 0, rejects = 0;
   double h_first = 0.0, h_next = 0.0;
   if (status == CHEM_CELL_OK) {
     double h_target, cp_dummy;
-    h_cp_mass(m, c, c.y[0], c.y + 1, h_target, cp_dummy);
+    h_cp_mass(m, c, c.y()[0], c.y() + 1, h_target, cp_dummy);
     // initial step
     double h = -1.0;
     bool guard = false;  // a supplied initial step, checked against f(y0) at the first step
@@ -2098,7 +2526,7 @@ __device__ void integrate_cell(const Job& job, int64_t cell, const IntegrateArgs
       }
     }
     if (h <= 0.0) {
-      eval_rhs<NW, false, Policy<PREC>::IR>(m, c, c.y, p, c.f0);
+      eval_rhs<NW, false, Policy<PREC>::IR>(m, c, c.y(), p, c.f0());
       h = starting_step<NW, Policy<PREC>::IR>(m, c, p, dt, rtol, atol, MT::Q);
     }
     double t = 0.0, h_unclipped = h;
@@ -2120,27 +2548,27 @@ __device__ void integrate_cell(const Job& job, int64_t cell, const IntegrateArgs
       auto apply_guard = [&]() {
         if (!guard) return;
         guard = false;
-        const double d0 = wrms(c, n, c.y, c.y, c.y, rtol, atol);
-        const double d1 = wrms(c, n, c.f0, c.y, c.y, rtol, atol);
+        const double d0 = wrms(c, n, c.y(), c.y(), c.y(), rtol, atol);
+        const double d1 = wrms(c, n, c.f0(), c.y(), c.y(), rtol, atol);
         const double ha = d1 > 1e-300 ? 0.01 * d0 / d1 : dt;
         h = fmin(fmin(fmax(h, ha), 100.0 * ha), dt - t);
         h_unclipped = h;
       };
       if (PREC == PREC_FP64 && args.jac_fd) {
-        eval_rhs<NW, false, false>(m, c, c.y, p, c.f0);
+        eval_rhs<NW, false, false>(m, c, c.y(), p, c.f0());
         apply_guard();
         PHASE(2);
-        fd_matrix<NW, false>(m, c, p, c.y, c.f0, 1.0 / (h * MT::gamma(args)));
+        fd_matrix<NW, false>(m, c, p, c.y(), c.f0(), 1.0 / (h * MT::gamma(args)));
       } else {
-        const Scal s = eval_rhs<NW, true, Policy<PREC>::IR>(m, c, c.y, p, c.f0);
+        const Scal s = eval_rhs<NW, true, Policy<PREC>::IR>(m, c, c.y(), p, c.f0());
         apply_guard();
         PHASE(2);
-        build_matrix<NW, PREC, false>(m, c, s, c.f0, 1.0 / (h * MT::gamma(args)));
+        build_matrix<NW, PREC, false>(m, c, s, c.f0(), 1.0 / (h * MT::gamma(args)));
       }
       PHASE(3);
       const int info = factor<NW, PREC>(c, n, !(PREC == PREC_FP64 && args.no_pivot));
       PHASE(6);
-      double err, step_fac = kFacMin;
+      double err, step_fac = kFacMin;  // err: square of the norm
       if (info != 0) {
         err = NAN;
       } else {
@@ -2148,43 +2576,56 @@ __device__ void integrate_cell(const Job& job, int64_t cell, const IntegrateArgs
         constexpr int S = MT::S;
 #pragma unroll 1
         for (int st = 0; st < S; ++st) {
-          const double* fs = c.f0;
           if (st > 0) {
             PHASE(6);
-            for (int i = c.tid; i < n; i += NT) {
-              double v = c.y[i];
-              for (int j = 0; j < st; ++j) v += MT::a(args, st, j) * c.u[j * n + i];
-              c.ys[i] = v;
+            // stage point y_s = y + sum_j a_sj u_j and sum_j c_sj u_j (kept in yn); with
+            // half the CTA's threads enough for n entries, each half takes one of the two
+            auto stage_sum = [&](int i, double v, auto coef) {
+#pragma unroll
+              for (int j = 0; j < S - 1; ++j)
+                if (j < st) v = fma(coef(j), c.u()[j * n + i], v);
+              return v;
+            };
+            auto ca = [&](int j) { return MT::a(args, st, j); };
+            auto cc = [&](int j) { return MT::c(args, st, j); };
+            if (n <= NT / 2) {
+              const int i = c.tid & (NT / 2 - 1);
+              if (i < n) {
+                if (c.tid < NT / 2) c.ys()[i] = stage_sum(i, c.y()[i], ca);
+                else c.yn()[i] = stage_sum(i, 0.0, cc);
+              }
+            } else {
+#pragma unroll 1
+              for (int i = c.tid; i < n; i += NT) {
+                c.ys()[i] = stage_sum(i, c.y()[i], ca);
+                c.yn()[i] = stage_sum(i, 0.0, cc);
+              }
             }
             __syncthreads();
             PHASE(4);
-            eval_rhs<NW, false, Policy<PREC>::IR>(m, c, c.ys, p, c.fv);
-            fs = c.fv;
+            eval_rhs<NW, false, Policy<PREC>::IR>(m, c, c.ys(), p, c.fv());
           }
           PHASE(6);
           // stage right-hand side f(y_s) + sum_j (c_sj / h) u_j, in place in fv
-          for (int i = c.tid; i < n; i += NT) {
-            double v = 0.0;
-            for (int j = 0; j < st; ++j) v += MT::c(args, st, j) * c.u[j * n + i];
-            c.fv[i] = fma(invh, v, fs[i]);
-          }
-          __syncthreads();
+#pragma unroll 1
+          for (int i = c.tid; i < n; i += NT) c.fv()[i] = st > 0 ? fma(invh, c.yn()[i], c.fv()[i]) : c.f0()[i];
           PHASE(5);
-          solve<NW, PREC>(c, n, c.fv, c.u + st * n, args.ir_sweeps);
+          solve<NW, PREC>(c, n, c.fv(), c.u() + st * n, args.ir_sweeps);
         }
         PHASE(6);
+#pragma unroll 1
         for (int i = c.tid; i < n; i += NT) {
-          double v = c.y[i], e = 0.0;
+          double v = c.y()[i], e = 0.0;
 #pragma unroll
           for (int j = 0; j < S; ++j) {
-            v += MT::m(args, j) * c.u[j * n + i];
-            if (!MT::E_LAST) e += MT::e(args, j) * c.u[j * n + i];
+            v += MT::m(args, j) * c.u()[j * n + i];
+            if (!MT::E_LAST) e += MT::e(args, j) * c.u()[j * n + i];
           }
-          c.yn[i] = v;
-          if (!MT::E_LAST) c.rr[i] = e;
+          c.yn()[i] = v;
+          if (!MT::E_LAST) c.rr()[i] = e;
         }
         __syncthreads();
-        err = wrms(c, n, MT::E_LAST ? c.u + (S - 1) * n : c.rr, c.y, c.yn, rtol, atol, &step_fac, MT::Q);
+        err = error_test(c, n, MT::E_LAST ? c.u() + (S - 1) * n : c.rr(), c.y(), c.yn(), rtol, atol, &step_fac, MT::Q);
       }
       if (!(err <= 1.0)) {
         ++rejects;
@@ -2193,7 +2634,8 @@ __device__ void integrate_cell(const Job& job, int64_t cell, const IntegrateArgs
         continue;
       }
       t += h;
-      for (int i = c.tid; i < n; i += NT) c.y[i] = c.yn[i];
+#pragma unroll 1
+      for (int i = c.tid; i < n; i += NT) c.y()[i] = c.yn()[i];
       __syncthreads();
       if (h_first == 0.0) h_first = h;
       const double fac = fmin(fmax(step_fac, kFacMin), after_reject ? 1.0 : kFacMax);
@@ -2206,23 +2648,25 @@ __device__ void integrate_cell(const Job& job, int64_t cell, const IntegrateArgs
     // temperature from the conserved mass enthalpy (Newton, |dT| < 1e-10 T)
     PHASE(7);
     if (status == CHEM_CELL_OK) {
-      double T = c.y[0];
+      double T = c.y()[0];
+#pragma unroll 1
       for (int it = 0; it < 50; ++it) {
         double hm, cpm;
-        h_cp_mass(m, c, T, c.y + 1, hm, cpm);
+        h_cp_mass(m, c, T, c.y() + 1, hm, cpm);
         const double dT = (hm - h_target) / cpm;
         T -= dT;
         if (fabs(dT) < 1e-10 * T) break;
       }
       if (!(T >= kTmin && T <= kTmax)) status = CHEM_CELL_T_RANGE;
-      else if (c.tid == 0) c.y[0] = T;
+      else if (c.tid == 0) c.y()[0] = T;
       __syncthreads();
     }
   }
   // store (the last accepted state for failed cells)
   if (status != CHEM_CELL_NONFINITE) {
-    if (c.tid == 0) job.T[cell] = c.y[0];
-    for (int k = c.tid; k < K; k += NT) job.Y[(size_t)cell * K + k] = c.y[1 + k];
+    if (c.tid == 0) job.T[cell] = c.y()[0];
+#pragma unroll 1
+    for (int k = c.tid; k < K; k += NT) job.Y[(size_t)cell * K + k] = c.y()[1 + k];
   }
   PHASE(7);
   if (c.tid == 0) {
@@ -2245,14 +2689,13 @@ __device__ void integrate_cell(const Job& job, int64_t cell, const IntegrateArgs
 // global-memory matrix slot makes room for (measured on 54 species: 7 % faster than
 // four CTAs; six and seven CTAs spill too much in the register Gauss-Jordan).
 template <int NW, int PREC, int MTH>
-__global__ void __launch_bounds__(NW * 32, NW == 4 ? (PREC == PREC_MIXED ? 5 : 4) : NW == 2 ? 8 : 2) k_integrate(const __grid_constant__ IntegrateArgs args) {
-  extern __shared__ __align__(16) unsigned char smem[];
+__global__ void __launch_bounds__(NW * 32, NW == 4 ? (PREC == PREC_MIXED ? 3 : 4) : NW == 2 ? 8 : 2) k_integrate(const __grid_constant__ IntegrateArgs args) {
   __shared__ long long s_work;
   const bool m0g = PREC == PREC_MIXED && args.m0_scratch != nullptr;
-  const Layout L = make_layout(args.smem_K, args.smem_I, PREC, m0g);
+  const Layout L = make_layout(args.smem_K, args.smem_I, PREC, m0g, true);
   Cta<NW> c;
-  c.bind(smem, L);
-  if (m0g) c.M0 = args.m0_scratch + (size_t)blockIdx.x * args.m0_stride;
+  c.bind(L);
+  double* const slot = m0g ? args.m0_scratch + (size_t)blockIdx.x * args.m0_stride : nullptr;
   for (long long it = 0;; ++it) {
     long long w;
     if (args.sched == SCHED_PLAIN) {
@@ -2270,7 +2713,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (PREC == PREC_MIXED ? 5 : 4
     const long long g = args.perm ? args.perm[w] : w;
     int j = 0;
     while (j + 1 < args.n_jobs && g >= args.jobs[j + 1].offset) ++j;
-    integrate_cell<NW, PREC, MTH>(args.jobs[j], g - args.jobs[j].offset, args, c);
+    integrate_cell<NW, PREC, MTH>(args.jobs[j], g - args.jobs[j].offset, args, c, slot);
   }
 }
 

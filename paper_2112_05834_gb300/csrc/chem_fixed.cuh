@@ -243,7 +243,8 @@ __device__ __forceinline__ unsigned long long fx_scale(double x, int sh) {
 // r^3/6 + r^4/24 + r^5/120); r and the bracket in Q62, r^2 from the two halves of r, the
 // cubic tail (below 2^-31) from 32-bit factors. Error before the final rounding below
 // 2^-58 relative.
-__device__ __forceinline__ double fx_exp(long long x) {
+// tab: g_fx_exp_tab or a copy of it in shared memory.
+__device__ __forceinline__ double fx_exp(long long x, const unsigned long long* tab) {
   constexpr int kInvL = 1549082005;                           // 256/ln2, Q22
   constexpr unsigned long long kL = 0x2c5c85fdf473deull;      // ln2/256, Q62, rounded down
   constexpr unsigned kLlo = 1794275565u;                      // the rest, Q94
@@ -259,7 +260,7 @@ __device__ __forceinline__ double fx_exp(long long x) {
   // (1/6)(1 + r/4 + r^2/20), Q32
   const int u = 715827883 + __mulhi(rh, 699051) + (r2 >> 23);
   const long long em1 = r + (sq >> 19) + (((long long)rh * rl) >> 40) + (((long long)r3 * u) >> 29);
-  const unsigned long long t = __ldg(&g_fx_exp_tab[N & 255]);
+  const unsigned long long t = tab[N & 255];
   const int th = (int)(t >> 32), tl = (int)((unsigned)t >> 1);
   const int eh = (int)(em1 >> 22), el = (int)((unsigned)em1 & 0x3fffffu);
   long long v = (long long)t + (((long long)eh * th) >> 8) + (((long long)eh * tl) >> 39) + (((long long)el * th) >> 30);
@@ -271,12 +272,11 @@ __device__ __forceinline__ double fx_exp(long long x) {
   return __longlong_as_double(((long long)e << 52) + ((v + 512) >> 10));
 }
 
-// ln x of a positive normal double in Q(Q) (Q = 52 or 58; |ln x| must fit): x = 2^e m,
+// ln x of a positive normal double in Q52 or Q58 (|ln x| must fit): x = 2^e m,
 // z = m c - 1 with c = 1/(1 + (j + 1/2)/256) to 31 bits, |z| < 2^-9, and ln x = e ln2 -
-// ln c + z - z^2/2 + z^3 (1/3 - z/4 + z^2/5 - z^3/6). Error below 2^-(Q - 1).
-template <int Q>
-__device__ __forceinline__ long long fx_log(double x) {
-  static_assert(Q == 52 || Q == 58, "fx_log");
+// ln c + z - z^2/2 + z^3 (1/3 - z/4 + z^2/5 - z^3/6). Error below 2^-51 (Q52), 2^-56 (Q58).
+// Out of line: it is called once or twice per rate evaluation.
+static __device__ __noinline__ long long fx_log(double x, int Q) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int e = (int)(b >> 52) - 1023;
   const int j = (int)(b >> 44) & 255;
@@ -292,9 +292,9 @@ __device__ __forceinline__ long long fx_log(double x) {
   // 1/3 - z/4 + z^2/5 - z^3/6, Q32
   const int u = 1431655765 - (zh >> 10) + (__mulhi(z2, 858993459) >> 16) - (z3 >> 29);
   const long long f = (long long)t.lnc + z - (sq >> 19) - (((long long)zh * zl) >> 40) + (((long long)z3 * u) >> 28);
-  constexpr long long kLn2 = Q == 52 ? 0xb17217f7d1cf7ll : 0x2c5c85fdf473de6ll;
-  constexpr long long kLn2lo = Q == 52 ? 2596052539ll : 2938605262ll;  // ln2 Q(Q + 32) - kLn2 2^32
-  return e * kLn2 + ((e * kLn2lo) >> 32) + (f >> (62 - Q));
+  const long long ln2 = Q == 52 ? 0xb17217f7d1cf7ll : 0x2c5c85fdf473de6ll;
+  const long long ln2_lo = Q == 52 ? 2596052539ll : 2938605262ll;  // ln2 Q(Q + 32) - ln2 2^32
+  return e * ln2 + ((e * ln2_lo) >> 32) + (f >> (62 - Q));
 }
 
 // Double to Q52, truncated; |x| >= 1024 and infinities saturate beyond +-1024 (NaN too).

@@ -54,52 +54,60 @@ struct DevMech {
   // Chunks dealt to the warps of a CTA of 64, 128 or 256 threads (table v = 0, 1, 2):
   // [NW + 1] offsets, then the chunk indices of warp 0, warp 1, ... (NW = 2 << v).
   const int* chunk_sched[3];
+  const int* tb_sched[3];  // the same for the third-body sums, in 32-row chunks of eff
   int n_tb;   // reactions with a third-body concentration (kinds 1..3)
   int n_fo;   // falloff reactions (kinds 2, 3)
   int i_tb0;  // first reaction of kind >= 1 (sorted order)
   int i_fo0;  // first reaction of kind >= 2
   int i_troe0;  // first reaction of kind 3
   double T_fx;    // the fixed-point rate evaluation holds for T in [T_fx, kFxThi) (1e300: nowhere)
-  // Fixed-point tables (value v in Qn: round(v 2^n)); ln T enters as Q58, 1/T as Q71.
   const long long* gfx;  // [K][16]: G/RT coefficients for range r at 8 r: constant (Q52), of ln T
                          //   (Q58), of 1/T (Q45), of t, t^2, t^3, t^4 (Q52), t = T/2048 (r = 0)
                          //   or T/8192 (r = 1)
-  const long long* arx;  // [I][4]: ln A (Q52), b (Q58), Ea_R (Q45), 0
-  const long long* fox;  // [n_fo][4]: the first three of fo in the same formats
+  const long long* fox;  // [n_fo][4]: the first three of fo in the formats of rx
   const double* W;      // [K]
   const double* invW;   // [K]
   const struct ff2* invW_ff;  // [K] as float-float pairs (hi, lo)
+  const struct ff2* W_ff;     // [K]
+  const double* T_mid;  // [K]
+  const double2* hcp;   // [K][2][10] as pairs, for range r: cp/R coefficients a1..a5, then H/RT
+                        //   coefficients a2/2, a3/3, a4/4, a5/5, a6 (its constant is a1)
   const double* nasa;   // [K][36]: for range r (0 below T_mid, 1 above) at 17 r:
                         //   cp/R coefficients a1..a5, H/RT coefficients a1, a2/2, a3/3,
                         //   a4/4, a5/5, a6, S/R coefficients a1, a2, a3/2, a4/3, a5/4, a7;
                         //   [34] = T_mid
   const double* arr;    // [I][4]: ln A, b, Ea_R, dnu
-  const int4* slots;    // [I]: reactant slot 0/1, product slot 0/1 species (-1 empty);
-                        //      a coefficient of 2 appears as two equal slots
-  const int* rev;       // [I] bit 0: reversible; bits 1-2: dnu + 1 (dnu = -1, 0, 1)
+  // [I] records of 32 bytes: fixed-point ln A (Q52), b (Q58), Ea_R (Q45), then four
+  // bytes of species slots (reactants 0/1, products 0/1; 255 empty; a coefficient of 2
+  // appears as two equal slots) and rev: bit 0 reversible, bits 1-2 dnu + 1 (dnu = -1, 0, 1).
+  // ln T enters as Q58, 1/T as Q71 (a value v in Qn: round(v 2^n)).
+  const longlong2* rx;
   const double* fo;     // [n_fo][8]: ln(A0/A), b0 - b, Ea0_R - Ea_R, alpha, 1/T***, 1/T*, T**, 0
   const double* eff;    // [n_tb][K] (row r belongs to reaction i_tb0 + r)
   const struct ff2* eff_ff;  // the same efficiencies as float-float pairs (hi, lo)
   const double* effT;        // [K][n_tb]: the efficiencies species-major
   const struct ff2* effT_ff;  // the same as float-float pairs
-  const int* sp_ptr;    // [K+1] species -> (reaction, nu) CSR
-  const int2* sp_ent;
-  const double* sp_nu;  // the same nu as doubles
+  // Production sums on a CTA of 64, 128 or 256 threads (table v): ps_g[v] adjacent lanes
+  // share a species, ps_passes[v] passes cover them all, ps_quads[v] loads per pass. Load r
+  // of a pass holds four 16-bit entries of thread t, at (pass ps_quads + r) NT + t: reaction
+  // << 1 | (1: consumed), 0xffff padding; a net coefficient of 2 is two entries.
+  const uint2* ps_ent[3];
+  int ps_g[3], ps_passes[3], ps_quads[3];
   // Mass-action Jacobian terms A_kj = sum nu_ki dq_i/dC_j, one sum per (row k,
   // column j) pair, dealt to the threads of a CTA of 64, 128 or 256 threads
   // (table v = 0, 1, 2) so that each thread has about as many terms as any other.
-  // Entry (r, t) of table v, at r * (64 << v) + t, is thread t's r-th term:
-  // x = index 4 i + slot into the per-reaction dq/dC data (-1: padding), y = the
-  // matrix offset the finished sum goes to (-1: the pair continues).
-  const int2* js_ent[3];
-  const double* js_nu[3];  // nu_ki W_k of the term
-  const struct ff2* js_nu_ff[3];  // the same as float-float pairs
+  // Entry (r, t) of table v, at r * (64 << v) + t, is thread t's r-th term: x = (4 i + slot)
+  // << 1 | (1: nu < 0) into the per-reaction dq/dC data (~0: padding; a coefficient of 2 is
+  // two entries), y = k << 8 | j of the finished sum (~0: it continues). js_rounds[v] is a
+  // multiple of 4.
+  const uint2* js_ent[3];
   int js_rounds[3];
   const unsigned* jmask;   // [K][ceil(K/32)]: bit l of word (k, u) set if pair (k, l + 32 u) exists
   const double* tr_nu;  // nu_ki W_k of the tr_ent entries
   const struct ff2* tr_nu_ff;  // the same as float-float pairs
   const int* tr_ptr;    // [K+1] row k -> (reaction i with [M], nu_ki)
   const int2* tr_ent;
+  const int* tr_row;    // offset of the entry's reaction in eff (3 more zeros: batched loads)
 };
 
 struct CellStats {
@@ -138,7 +146,7 @@ struct IntegrateArgs {
   int no_pivot;        // FP64 form only: 1 = Gaussian elimination without row interchanges
   int smem_K, smem_I;  // sizes the shared-memory carve-up was computed for
   unsigned long long* phase;  // optional [8] per-phase cycle counters (diagnostic)
-  double* m0_scratch;  // mixed form, persistent grids: per-CTA slots for the assembled matrix
+  double* m0_scratch;  // mixed form, persistent grids: per-CTA slots for the assembled matrix and its sums
   int64_t m0_stride;   //   (8-byte entries; null: it stays in shared memory); entries per slot
   MethodTab tab;       // the Rosenbrock method
 };

@@ -6,9 +6,11 @@
 
 namespace chem {
 
-size_t smem_bytes(int Kmax, int Imax, int prec, bool m0_global) {
-  return make_layout(Kmax, Imax, prec, m0_global).total;
+size_t smem_bytes(int Kmax, int Imax, int prec, bool m0_global, bool x_tab) {
+  return make_layout(Kmax, Imax, prec, m0_global, x_tab).total;
 }
+
+int64_t matrix_slot_entries(int Kmax) { return (int64_t)slot_entries(Kmax); }
 
 // W-method instantiations (chem_kernels_w.cu)
 cudaError_t launch_integrate_w(const IntegrateArgs& a, int block, int prec, int grid, cudaStream_t st);
@@ -26,35 +28,43 @@ struct DiagArgs {
 
 template <int NW, int PREC>
 __global__ void __launch_bounds__(NW * 32) k_diag(const __grid_constant__ DiagArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
   using A = typename Policy<PREC>::ASM;
-  const Layout L = make_layout(a.m.K, a.m.I, PREC);
+  const Layout L = make_layout(a.m.K, a.m.I, PREC, false, true);
   Cta<NW> c;
-  c.bind(smem, L);
+  c.bind(L);
 
   constexpr int NT = NW * 32;
   const int K = a.m.K, n = K + 1, ld = odd_ld(n);
+#pragma unroll 1
   for (int64_t cell = blockIdx.x; cell < a.n; cell += gridDim.x) {
-    if (c.tid == 0) c.y[0] = a.T[cell];
-    for (int k = c.tid; k < K; k += NT) c.y[1 + k] = a.Y[(size_t)cell * K + k];
-    __syncthreads();
+    if (c.tid == 0) c.y()[0] = a.T[cell];
+#pragma unroll 1
+    for (int k = c.tid; k < K; k += NT) c.y()[1 + k] = a.Y[(size_t)cell * K + k];
     const double p = a.p[cell];
+    c.set_cell(a.m, p);
+    c.set_matrix(K, nullptr);
+    __syncthreads();
     if (a.what == 0) {
-      eval_rhs<NW, false, Policy<PREC>::IR>(a.m, c, c.y, p, c.f0);
-      for (int i = c.tid; i < n; i += NT) a.out[(size_t)cell * n + i] = c.f0[i];
+      eval_rhs<NW, false, Policy<PREC>::IR>(a.m, c, c.y(), p, c.f0());
+#pragma unroll 1
+      for (int i = c.tid; i < n; i += NT) a.out[(size_t)cell * n + i] = c.f0()[i];
     } else if (a.what == 1) {
       if (PREC == PREC_FP64 && a.jac_fd) {
-        eval_rhs<NW, false, false>(a.m, c, c.y, p, c.f0);
-        fd_matrix<NW, true>(a.m, c, p, c.y, c.f0, 0.0);
+        eval_rhs<NW, false, false>(a.m, c, c.y(), p, c.f0());
+        fd_matrix<NW, true>(a.m, c, p, c.y(), c.f0(), 0.0);
       } else {
-        const Scal s = eval_rhs<NW, true, Policy<PREC>::IR>(a.m, c, c.y, p, c.f0);
-        build_matrix<NW, PREC, true>(a.m, c, s, c.f0, 0.0);
+        const Scal s = eval_rhs<NW, true, Policy<PREC>::IR>(a.m, c, c.y(), p, c.f0());
+        build_matrix<NW, PREC, true>(a.m, c, s, c.f0(), 0.0);
       }
-      const A* J = reinterpret_cast<const A*>(Policy<PREC>::IR ? c.M0 : c.M);
+      // (the mixed forms hold it by columns)
+      const A* J = reinterpret_cast<const A*>(Policy<PREC>::IR ? c.M0 : c.M());
+      const int si = Policy<PREC>::IR ? 1 : ld, sj = Policy<PREC>::IR ? ld : 1;
+#pragma unroll 1
       for (int i = c.warp; i < n; i += NW)
-        for (int j = c.lane; j < n; j += 32) a.out[(size_t)cell * n * n + i * n + j] = to_double(J[i * ld + j]);
+#pragma unroll 1
+        for (int j = c.lane; j < n; j += 32) a.out[(size_t)cell * n * n + i * n + j] = to_double(J[i * si + j * sj]);
     } else {
-      eval_rhs<NW, false, Policy<PREC>::IR>(a.m, c, c.y, p, c.f0);
+      eval_rhs<NW, false, Policy<PREC>::IR>(a.m, c, c.y(), p, c.f0());
       const double h = starting_step<NW, Policy<PREC>::IR>(a.m, c, p, a.dt, a.rtol, a.atol, a.q);
       if (c.tid == 0) a.out[cell] = h;
     }
@@ -86,28 +96,32 @@ struct LuArgs {
 
 template <int NW, int PREC>
 __global__ void __launch_bounds__(NW * 32) k_lu_solve(const __grid_constant__ LuArgs a) {
-  extern __shared__ __align__(16) unsigned char smem[];
   using P = Policy<PREC>;
   using R = typename P::LU;
   const Layout L = make_layout(a.dim - 1, 1, PREC);
   Cta<NW> c;
-  c.bind(smem, L);
+  c.bind(L);
   constexpr int NT = NW * 32;
   const int n = a.dim, ld = odd_ld(n);
-  R* M = reinterpret_cast<R*>(c.M);
+  R* M = reinterpret_cast<R*>(c.M());
+#pragma unroll 1
   for (int64_t s = blockIdx.x; s < a.n_mat; s += gridDim.x) {
     const double* As = a.A + (size_t)s * n * n;
+#pragma unroll 1
     for (int i = c.warp; i < n; i += NW)
+#pragma unroll 1
       for (int j = c.lane; j < n; j += 32) {
         const double v = As[i * n + j];
-        M[i * ld + j] = (R)v;
-        if constexpr (P::IR) reinterpret_cast<typename P::ASM*>(c.M0)[i * ld + j] = from_double<typename P::ASM>(v);
+        if constexpr (P::IR) reinterpret_cast<typename P::ASM*>(c.M0)[j * ld + i] = from_double<typename P::ASM>(v);
+        else M[i * ld + j] = v;
       }
-    for (int i = c.tid; i < n; i += NT) c.fv[i] = a.b[(size_t)s * n + i];
+#pragma unroll 1
+    for (int i = c.tid; i < n; i += NT) c.fv()[i] = a.b[(size_t)s * n + i];
     __syncthreads();
     const int info = factor<NW, PREC>(c, n);
-    if (info == 0) solve<NW, PREC>(c, n, c.fv, c.u, a.ir);
-    for (int i = c.tid; i < n; i += NT) a.x[(size_t)s * n + i] = info == 0 ? c.u[i] : NAN;
+    if (info == 0) solve<NW, PREC>(c, n, c.fv(), c.u(), a.ir);
+#pragma unroll 1
+    for (int i = c.tid; i < n; i += NT) a.x[(size_t)s * n + i] = info == 0 ? c.u()[i] : NAN;
     if (c.tid == 0 && a.info) a.info[s] = info;
     __syncthreads();
   }
@@ -206,7 +220,7 @@ cudaError_t launch_lu_solve(int64_t n_mat, int dim, const double* A, const doubl
   a.x = x;
   a.info = info;
   a.ir = ir;
-  const size_t smem = smem_bytes(dim - 1, 1, prec);
+  const size_t smem = smem_bytes(dim - 1, 1, prec, false, false);
   const int grid = (int)(n_mat < 65535 ? n_mat : 65535);
   if (prec == PREC_FP64) return launch_simple<PREC_FP64>(k_lu_solve<4, PREC_FP64>, a, smem, grid, st);
   if (prec == PREC_MIXED) return launch_simple<PREC_MIXED>(k_lu_solve<4, PREC_MIXED>, a, smem, grid, st);

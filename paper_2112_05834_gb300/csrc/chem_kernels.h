@@ -10,7 +10,10 @@
 
 namespace chem {
 
-size_t smem_bytes(int Kmax, int Imax, int prec, bool m0_global = false);
+// Dynamic shared memory of a kernel (x_tab: with the exponential's table, where it fits).
+size_t smem_bytes(int Kmax, int Imax, int prec, bool m0_global = false, bool x_tab = true);
+// 8-byte entries of a CTA's global-memory matrix slot (mixed form).
+int64_t matrix_slot_entries(int Kmax);
 cudaError_t launch_integrate(const IntegrateArgs& a, int block, int prec, int grid, cudaStream_t st);
 cudaError_t occupancy_integrate(int block, int prec, int K, int I, int* ctas_per_sm, bool m0_global = false);
 cudaError_t launch_diag(const DevMech& m, int64_t n, const double* T, const double* p, const double* Y,

@@ -130,7 +130,7 @@ extern "C" chem_status chem_integrate_noalloc(chem_handle h, int64_t n_cells, do
   a.tab = chem::method_tableau(h->method);
   a.smem_K = h->K;
   a.smem_I = h->I > 0 ? h->I : 1;
-  const int block = h->block ? h->block : chem_internal_pick_block(h, a.smem_K, a.smem_I);
+  const int block = h->block ? h->block : chem_internal_pick_block(h, a.smem_K, a.smem_I, n_cells);
   int grid;
   if (a.sched == chem::SCHED_PLAIN) {
     grid = (int)n_cells;

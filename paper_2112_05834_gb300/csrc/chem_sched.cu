@@ -295,8 +295,8 @@ chem_status chem_internal_autotune(chem_handle h, const IntegrateArgs& a, cudaSt
       }
     }
   if (cands.empty()) return CHEM_OK;
-  const int64_t stride = (int64_t)(a.smem_K + 1) * ((a.smem_K + 1) | 1);
-  const size_t sample_doubles = (size_t)S * (K + 2) * 2;
+  const int64_t stride = matrix_slot_entries(a.smem_K);
+  const size_t sample_doubles = ((size_t)S * (K + 2) * 2 + 3) & ~(size_t)3;  // the slots start at a 32-byte boundary
   const size_t slot_doubles = layouts ? (size_t)max_grid * stride : 0;
   double* buf = nullptr;
   cudaError_t e = cudaMalloc(&buf, (sample_doubles + slot_doubles) * sizeof(double));
