@@ -26,7 +26,6 @@
 namespace {
 
 constexpr int kH = 128;      // hidden width
-constexpr int kChunk = 65536;  // rows per inference chunk
 typedef __nv_bfloat16 bf16;
 
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
@@ -83,258 +82,490 @@ __global__ void k_target_stats(const int32_t* sub, const double* hf, int64_t n, 
   }
 }
 
-// Standardised BF16 features of rows [r0, r0 + rows). With zmax > 0, out[r] is set
-// to 1 for a row with a standardised feature beyond +-zmax (any thread of the row may
-// store it; all store the same value; the head kernel reads and clears it).
-__global__ void k_features(const double* T, const double* p, const double* Y, int K, int64_t r0, int64_t rows,
-                           const float* norm, bf16* X, float zmax = 0.0f, unsigned char* out = nullptr) {
-  const int D = K + 2;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < rows * D; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t r = e / D;
-    const int d = (int)(e - r * D);
-    const double x = feature(T, p, Y, K, r0 + r, d);
-    const float z = (float)((x - norm[d]) / norm[D + d]);
-    X[e] = __float2bfloat16(z);
-    if (zmax > 0.0f && !(fabsf(z) <= zmax)) out[r] = 1;
-  }
-}
-
-__global__ void k_targets(const int32_t* sub, const double* hf, int64_t n, const float* norm_t, float* Ts) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double t0 = log(fmax((double)sub[i], 1.0)), t1 = log(fmax(hf[i], 1e-300));
-    Ts[2 * i] = (float)((t0 - norm_t[0]) / norm_t[2]);
-    Ts[2 * i + 1] = (float)((t1 - norm_t[1]) / norm_t[3]);
-  }
-}
-
-__global__ void k_gather(const bf16* X, const float* Ts, const int* perm, int64_t b0, int rows, int D, bf16* Xb,
-                         float* Tb) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)rows * D; e += (int64_t)gridDim.x * blockDim.x) {
-    const int r = (int)(e / D), d = (int)(e - (int64_t)r * D);
-    Xb[e] = X[(size_t)perm[b0 + r] * D + d];
-  }
-  for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += gridDim.x * blockDim.x) {
-    Tb[2 * r] = Ts[2 * (size_t)perm[b0 + r]];
-    Tb[2 * r + 1] = Ts[2 * (size_t)perm[b0 + r] + 1];
-  }
-}
-
 // ---------------------------------------------------------------------------
-// BF16 GEMM, FP32 accumulation: C(m, n) = sum_k A(m, k) B(n, k) with general strides
-// A(m, k) = A[m sam + k sak], B(n, k) = B[n sbn + k sbk]. 64 x 64 tile per CTA,
-// 4 warps of 32 x 32, mma.sync.m16n8k16; split-K over blockIdx.z.
-// mode 0: C[z zstride + m ldc + n] = acc
-// mode 1: z = acc + bias[n]; Zout (optional) = z; Hout = bf16(GELU(z))
-// mode 2: dZout = bf16(acc * GELU'(Zin))
+// forward pass (and backward pass) of a batch in one kernel
+//
+// A warp takes 16 rows through the whole model: it standardises their features into its own
+// BF16 tile in shared memory, and since the accumulator fragment of one m16n8k16 product is
+// laid out like the A fragment of the next, both hidden layers stay in registers; the
+// weights are read from shared memory, where each CTA loads them once.
+//
+// Four kernels per pass with one FP64 logarithm and division per feature took 527 us for
+// 65,536 rows of 54 species and were bound by the FP64 pipe (3.5 M logarithms of some 25
+// operations at 19 cycles per warp and SM: 180 us) and by element-wise strided operand
+// loads. Training keeps what the backward pass needs in shared memory: a CTA's 64 rows give
+// both weight gradients as products of tiles that never leave the SM (334 us for 8,192 rows
+// in 17 launches before, with two passes over the activations in global memory per layer).
 // ---------------------------------------------------------------------------
-struct GemmP {
-  const bf16* A;
-  long long sam, sak;
-  const bf16* B;
-  long long sbn, sbk;
-  int M, N, K, kchunk, mode;
-  float* C;
-  long long ldc, zstride;
-  const float* bias;
-  float* Zout;
-  bf16* Hout;
-  const float* Zin;
-  bf16* dZout;
+struct MlpP {
+  const double *T, *p, *Y;
+  const int* perm;  // row order of a training epoch (null: as given)
+  int64_t row0, n;  // rows [row0, row0 + n) of that order
+  int K, D, Dp;     // species, features, features rounded up to 16
+  const float* norm;  // mu_x[D], sd_x[D], mu_t[2], sd_t[2]
+  const bf16* wb;     // BF16 weights
+  const float* w;     // FP32 weights (biases)
+  int64_t ob1, oW2, ob2, oW3, ob3, nw;
+  // prediction
+  float zmax;  // > 0: rows with a standardised feature beyond +-zmax get a NaN initial step
+  float *ln_cost, *ln_h0, *cost;
+  double* h0;
+  // training
+  const int32_t* sub;
+  const double* hf;
+  float inv_B;
+  float* part;  // [CTAs][part_stride]: gradient in the order of the weights, then the loss
+  int64_t part_stride;
 };
 
-__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
+constexpr int kLd = kH + 8;  // row length of the 128-wide tiles (rows 16 bytes off in banks: no conflicts)
+constexpr int kPredictWarps = 8, kTrainWarps = 4;
+constexpr size_t kMaxSmemMlp = 232448;
+constexpr int kFeatureBatch = 8;                      // loads in flight per lane
+constexpr int kListed = 32 + 32 * kFeatureBatch;  // features a warp may have waiting for FP64
+
+struct MlpSmem {  // byte offsets
+  int W2, X, norm, vec, list, H1, H2, dZ2, g1, d, total;
+};
+__host__ __device__ inline MlpSmem mlp_smem(int Dp, int warps, bool train) {
+  MlpSmem o;
+  const int ld1 = Dp + 8;
+  o.W2 = kH * ld1 * 2;
+  o.X = o.W2 + kH * kLd * 2;
+  o.norm = o.X + warps * 16 * ld1 * 2;
+  o.vec = o.norm + Dp * 8;
+  o.list = o.vec + 4 * kH * 4;
+  o.H1 = o.list + (train ? 0 : warps * kListed * 2);  // training: in the g1 area, unused by then
+  const int tile = train ? warps * 16 * kLd * 2 : 0;
+  o.H2 = o.H1 + tile;
+  o.dZ2 = o.H2 + tile;
+  o.g1 = o.dZ2 + tile;
+  o.d = o.g1 + (train ? warps * 16 * kH * 4 : 0);
+  o.total = o.d + (train ? warps * 16 * 12 : 0);
+  return o;
+}
+
+__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
       "{%0,%1,%2,%3};\n"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldsm(uint32_t (&r)[4], const bf16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm_t(uint32_t (&r)[4], const bf16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"((uint32_t)__cvta_generic_to_shared(p)) : "memory");
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-__global__ void __launch_bounds__(128) k_gemm(const GemmP p) {
-  __shared__ __align__(16) bf16 As[64][40];
-  __shared__ __align__(16) bf16 Bs[64][40];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int wm = warp >> 1, wn = warp & 1;
-  const int g = lane >> 2, t4 = lane & 3;
-  const int m0 = blockIdx.x * 64, n0 = blockIdx.y * 64;
-  const int kb = blockIdx.z * p.kchunk;
-  const int ke = min(p.K, kb + p.kchunk);
-  const bf16 zero = __float2bfloat16(0.0f);
-  float acc[2][4][4];
+// acc[16 rows][128] += A (fragments of kt16 x 16 columns) W^T for W stored [128][k]
+__device__ __forceinline__ void rows_times_wt(float (&acc)[16][4], const uint32_t (&a)[4], const bf16* W, int ld,
+                                              int k0, int lane) {
+  const bf16* w = W + ((lane & 7) + ((lane >> 4) << 3)) * ld + k0 + ((lane >> 3) & 1) * 8;
 #pragma unroll
-  for (int a = 0; a < 2; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.0f;
-  for (int k0 = kb; k0 < ke; k0 += 32) {
-    for (int e = tid; e < 64 * 32; e += 128) {
-      const int r = e >> 5, cc = e & 31;
-      const int gk = k0 + cc;
-      const int gm = m0 + r, gn = n0 + r;
-      As[r][cc] = (gm < p.M && gk < ke) ? p.A[(long long)gm * p.sam + (long long)gk * p.sak] : zero;
-      Bs[r][cc] = (gn < p.N && gk < ke) ? p.B[(long long)gn * p.sbn + (long long)gk * p.sbk] : zero;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 32; kk += 16) {
-      uint32_t a[2][4], b[4][2];
-      const int c = kk + t4 * 2;
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt) {
-        const int r = wm * 32 + mt * 16 + g;
-        a[mt][0] = *reinterpret_cast<const uint32_t*>(&As[r][c]);
-        a[mt][1] = *reinterpret_cast<const uint32_t*>(&As[r + 8][c]);
-        a[mt][2] = *reinterpret_cast<const uint32_t*>(&As[r][c + 8]);
-        a[mt][3] = *reinterpret_cast<const uint32_t*>(&As[r + 8][c + 8]);
-      }
-#pragma unroll
-      for (int nt = 0; nt < 4; ++nt) {
-        const int nn = wn * 32 + nt * 8 + g;
-        b[nt][0] = *reinterpret_cast<const uint32_t*>(&Bs[nn][c]);
-        b[nt][1] = *reinterpret_cast<const uint32_t*>(&Bs[nn][c + 8]);
-      }
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int nt = 0; nt < 4; ++nt) mma_bf16(acc[mt][nt], a[mt], b[nt]);
-    }
-    __syncthreads();
+  for (int np = 0; np < 8; ++np) {
+    uint32_t b[4];
+    ldsm(b, w + np * 16 * ld);
+    mma_bf16(acc[2 * np], a, b[0], b[1]);
+    mma_bf16(acc[2 * np + 1], a, b[2], b[3]);
   }
+}
+
+// The feature's standardised value z in FP32 arithmetic from the leading bits of v, with a
+// bound e on its distance from the FP64 result rounded to FP32; false where the arithmetic
+// does not cover v (negative, beyond FP32's range, not finite).
+// ln s = E ln 2 + ln 2 log2(m), m in [0.707, 1.414): __log2f is within 2^-22 there, E ln 2 - mu
+// is one rounding with the upper bits of ln 2, the truncated bits of v and the rounded 1e-20
+// shift s by under 2.4e-7: 4.8e-7 + 1.2e-7 |t| in all, taken as 8e-7 + 4e-7 |t|.
+enum { FEAT_Y, FEAT_P, FEAT_T };
+template <int KIND>
+__device__ __forceinline__ bool feature_fast(double v, float2 norm, float* z, float* e) {
+  const int hi = __double2hiint(v);
+  const int fe = (hi >> 20) - 896;
+  float s = __int_as_float((fe << 23) | ((hi & 0xfffff) << 3) | (int)((unsigned)__double2loint(v) >> 29));
+  bool ok = hi >= 0 && fe < 255;
+  if (KIND == FEAT_Y) s = (fe > 0 ? s : 0.0f) + 1e-20f;
+  else ok = ok && fe > 0;
+  float t, et;
+  if (KIND == FEAT_T) {
+    t = fmaf(s, 1e-3f, -norm.x);
+    et = fmaf(s, 2.5e-10f, 8e-7f);
+  } else {
+    const int b = __float_as_int(s);
+    const int E = (b - 0x3f3504f3) >> 23;
+    const float Ef = __int_as_float(0x4b400000 + E) - 12582912.0f;  // E as a float
+    const float l = __log2f(__int_as_float(b - (E << 23)));
+    t = fmaf(Ef, 0.693145751953125f, -norm.x) + fmaf(Ef, 1.42860682e-6f, 0.693147182f * l);
+    et = 8e-7f;
+  }
+  *z = t * norm.y;
+  *e = fmaf(fmaf(fabsf(t), 4e-7f, et), fabsf(norm.y), 3.2e-7f * fabsf(*z));
+  return ok && fabsf(*z) > 1e-30f && fabsf(*z) < 1e30f;
+}
+
+// One warp's 16 x D feature tile (BF16); rows beyond nr are zero. The BF16 value is that of
+// the FP64 formula: where the FP32 value's error bound reaches across a rounding boundary (or
+// across zmax), some one element in a thousand, the element is put on a list and the warp
+// goes through the formula for all of those side by side. Returns the rows beyond zmax.
+template <bool TRAIN>
+__device__ __forceinline__ uint32_t feature_tile(const MlpP& p, bf16* X, int ld, const float2* norm, uint16_t* list,
+                                                 int64_t r0, int nr, int lane) {
+  const int K = p.K, EY = 16 * K;
+  const uint32_t inv_k = (1u << 20) / (uint32_t)K + 1;  // e / K for e < 16 K, K < 256
+  const int64_t mine = p.row0 + r0 + ((lane & 15) < nr ? lane & 15 : 0);
+  const int64_t src = TRAIN && p.perm ? (int64_t)p.perm[mine] : mine;
+  uint32_t far = 0;
+  int cnt = 0;
+  auto put = [&](int r, int d, float z) {
+    X[r * ld + d] = __float2bfloat16(z);
+    if (p.zmax > 0.0f && !(fabsf(z) <= p.zmax)) far |= 1u << r;
+  };
+  auto listed = [&]() {
+    __syncwarp();
+    for (int i0 = 0; i0 < cnt; i0 += 32) {
+      const int c = list[min(i0 + lane, cnt - 1)];
+      const int q = c - EY;
+      const int r = q >= 0 ? q & 15 : (int)((uint32_t)c * inv_k >> 20);
+      const int d = q >= 0 ? q >> 4 : c - r * K + 2;
+      const int64_t row = __shfl_sync(0xffffffffu, src, r);
+      const double x = feature(p.T, p.p, p.Y, K, row, d);
+      put(r, d, (float)((x - p.norm[d]) / p.norm[p.D + d]));
+    }
+    __syncwarp();
+    cnt = 0;
+  };
+  auto take = [&](int code, int r, int d, bool valid, bool ok, float z, float e) {
+    const uint32_t h = pack_bf16(z - e, z + e);
+    const bool slow = valid && (!ok || ((h ^ (h >> 16)) & 0xffffu) || (p.zmax > 0.0f && fabsf(fabsf(z) - p.zmax) <= e));
+    if (valid && !slow) put(r, d, z);
+    const uint32_t m = __ballot_sync(0xffffffffu, slow);
+    if (m) {
+      if (slow) list[cnt + __popc(m & ((1u << lane) - 1))] = (uint16_t)code;
+      cnt += __popc(m);
+    }
+  };
+  {
+    const int r = lane & 15, d = lane >> 4;
+    const bool valid = r < nr;
+    float z, e;
+    bool ok;
+    if (d == 0) ok = feature_fast<FEAT_T>(p.T[src], norm[0], &z, &e);
+    else ok = feature_fast<FEAT_P>(p.p[src], norm[1], &z, &e);
+    __syncwarp();
+    if (!valid) X[r * ld + d] = __float2bfloat16(0.0f);
+    take(EY + lane, r, d, valid, ok, z, e);
+  }
+  constexpr int U = kFeatureBatch;
+#pragma unroll 1
+  for (int e0 = 0; e0 < EY; e0 += 32 * U) {
+    double v[U];
 #pragma unroll
-  for (int mt = 0; mt < 2; ++mt)
+    for (int j = 0; j < U; ++j) {
+      const int i = e0 + j * 32 + lane;
+      if (TRAIN) {
+        const int r = (int)((uint32_t)min(i, EY - 1) * inv_k >> 20);
+        const int64_t row = __shfl_sync(0xffffffffu, src, r);
+        v[j] = i < EY && r < nr ? p.Y[(size_t)row * K + (i - r * K)] : 1.0;
+      } else {
+        v[j] = i < nr * K ? __ldcs(p.Y + (size_t)(p.row0 + r0) * K + i) : 1.0;
+      }
+    }
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
+    for (int j = 0; j < U; ++j) {
+      const int i = e0 + j * 32 + lane;
+      const int r = (int)((uint32_t)min(i, EY - 1) * inv_k >> 20), k = min(i, EY - 1) - r * K;
+      float z, e;
+      const bool ok = feature_fast<FEAT_Y>(v[j], norm[2 + k], &z, &e);
+      if (i < EY && r >= nr) X[r * ld + 2 + k] = __float2bfloat16(0.0f);
+      take(i, r, 2 + k, i < EY && r < nr, ok, z, e);
+    }
+    if (cnt > 32 || (cnt > 0 && e0 + 32 * U >= EY)) listed();
+  }
+  __syncwarp();
+  return __reduce_or_sync(0xffffffffu, far);
+}
+
+// out[o][i] (+)= sum over the CTA's 64 rows of A[row][o] B[row][i], o in the warp's 32, i < cols
+__device__ __forceinline__ void weight_gradient(const bf16* A, int a_step, const bf16* B, int ldb, int cols, int warp,
+                                                int lane, bool add, float* out) {
+  const int ar = (lane & 7) + ((lane >> 4) << 3), am = ((lane >> 3) & 1) * 8;
+  const int br = lane & 15, bn = (lane >> 4) * 8;
+  const int pad = (cols + 15) / 16 * 16;
+#pragma unroll 1
+  for (int mt = 0; mt < 2; ++mt) {
+    const int o0 = warp * 32 + mt * 16;
+#pragma unroll 1
+    for (int c0 = 0; c0 < pad; c0 += 64) {
+      float acc[8][4] = {};
 #pragma unroll
-      for (int hf = 0; hf < 2; ++hf)
+      for (int kt = 0; kt < 4; ++kt) {
+        uint32_t a[4];
+        ldsm_t(a, A + kt * a_step + ar * kLd + o0 + am);
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const int m = m0 + wm * 32 + mt * 16 + g + hf * 8;
-          const int n = n0 + wn * 32 + nt * 8 + t4 * 2 + j;
-          if (m >= p.M || n >= p.N) continue;
-          const float v = acc[mt][nt][hf * 2 + j];
-          if (p.mode == 0) {
-            p.C[(long long)blockIdx.z * p.zstride + (long long)m * p.ldc + n] = v;
-          } else if (p.mode == 1) {
-            const float z = v + p.bias[n];
-            if (p.Zout) p.Zout[(long long)m * p.N + n] = z;
-            p.Hout[(long long)m * p.N + n] = __float2bfloat16(gelu(z));
-          } else {
-            p.dZout[(long long)m * p.N + n] = __float2bfloat16(v * gelu_grad(p.Zin[(long long)m * p.N + n]));
+        for (int np = 0; np < 4; ++np) {
+          if (c0 + np * 16 < pad) {
+            uint32_t b[4];
+            ldsm_t(b, B + (kt * 16 + br) * ldb + c0 + np * 16 + bn);
+            mma_bf16(acc[2 * np], a, b[0], b[1]);
+            mma_bf16(acc[2 * np + 1], a, b[2], b[3]);
           }
         }
-}
-
-// ---------------------------------------------------------------------------
-// output head (128 -> 2), one warp per row. Training: loss, dZ2, per-warp partial
-// gradients of W3/b3. Prediction: denormalised outputs.
-// ---------------------------------------------------------------------------
-struct HeadP {
-  const bf16* H2;
-  const float* Z2;
-  const bf16* W3;   // [2][128] bf16
-  const float* b3;  // [2]
-  const float* Tb;  // standardised targets [rows][2] (training)
-  int rows;
-  float inv_B;
-  bf16* dZ2;
-  float* part;      // [warps][2*128 + 2 + 1]
-  const float* norm_t;  // mu_t[2], sd_t[2] (prediction)
-  float* ln_cost;
-  float* ln_h0;
-  float* cost;      // exp(ln_cost)
-  double* h0;       // max(exp(ln_h0), 1e-14); NaN for a row flagged in out_of_range
-  unsigned char* out_of_range;  // [rows] rows with a feature beyond the range (cleared here)
-  int64_t out0;     // output row offset
-};
-
-__global__ void k_head(const HeadP p, int train) {
-  const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int nw = (gridDim.x * blockDim.x) >> 5;
-  float w0[4], w1[4];
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    w0[j] = __bfloat162float(p.W3[lane * 4 + j]);
-    w1[j] = __bfloat162float(p.W3[kH + lane * 4 + j]);
-  }
-  float gW0[4] = {0, 0, 0, 0}, gW1[4] = {0, 0, 0, 0}, gb0 = 0, gb1 = 0, loss = 0;
-  for (int r = gw; r < p.rows; r += nw) {
-    float h[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) h[j] = __bfloat162float(p.H2[(size_t)r * kH + lane * 4 + j]);
-    float o0 = 0, o1 = 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      o0 += h[j] * w0[j];
-      o1 += h[j] * w1[j];
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-      o0 += __shfl_xor_sync(0xffffffffu, o0, o);
-      o1 += __shfl_xor_sync(0xffffffffu, o1, o);
-    }
-    o0 += p.b3[0];
-    o1 += p.b3[1];
-    if (train) {
-      const float r0 = o0 - p.Tb[2 * r], r1 = o1 - p.Tb[2 * r + 1];
-      loss += 0.5f * (r0 * r0 + r1 * r1) * p.inv_B;
-      const float d0 = r0 * p.inv_B, d1 = r1 * p.inv_B;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float z = p.Z2[(size_t)r * kH + lane * 4 + j];
-        p.dZ2[(size_t)r * kH + lane * 4 + j] = __float2bfloat16((d0 * w0[j] + d1 * w1[j]) * gelu_grad(z));
-        gW0[j] += d0 * h[j];
-        gW1[j] += d1 * h[j];
       }
-      gb0 += d0;
-      gb1 += d1;
-    } else if (lane == 0) {
-      const float l0 = o0 * p.norm_t[2] + p.norm_t[0];
-      const float l1 = o1 * p.norm_t[3] + p.norm_t[1];
-      const int64_t q = p.out0 + r;
-      if (p.ln_cost) p.ln_cost[q] = l0;
-      if (p.ln_h0) p.ln_h0[q] = l1;
-      if (p.cost) p.cost[q] = expf(fminf(l0, 80.0f));
-      bool far = false;
-      if (p.out_of_range && p.out_of_range[r]) {
-        far = true;
-        p.out_of_range[r] = 0;
-      }
-      if (p.h0) p.h0[q] = far ? __longlong_as_double(0x7ff8000000000000LL) : fmax(exp((double)l1), 1e-14);
-    }
-  }
-  if (train) {
-    float* pp = p.part + (size_t)gw * (2 * kH + 3);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      pp[lane * 4 + j] = gW0[j];
-      pp[kH + lane * 4 + j] = gW1[j];
-    }
-    if (lane == 0) {
-      pp[2 * kH] = gb0;
-      pp[2 * kH + 1] = gb1;
-      pp[2 * kH + 2] = loss;
+      for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int o = o0 + (lane >> 2) + (q >> 1) * 8, i = c0 + nt * 8 + (lane & 3) * 2 + (q & 1);
+          if (i < cols) {
+            float* w = out + (size_t)o * cols + i;
+            *w = add ? *w + acc[nt][q] : acc[nt][q];
+          }
+        }
     }
   }
 }
 
-// out[j] = sum_s part[s * stride + j], j < len (fixed order)
-__global__ void k_reduce(const float* part, int S, int stride, int len, float* out) {
-  for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < len; j += gridDim.x * blockDim.x) {
-    float s = 0.0f;
-    for (int i = 0; i < S; ++i) s += part[(size_t)i * stride + j];
-    out[j] = s;
+template <bool TRAIN>
+__global__ void __launch_bounds__((TRAIN ? kTrainWarps : kPredictWarps) * 32, TRAIN ? 1 : 2) k_mlp(const MlpP p) {
+  constexpr int WARPS = TRAIN ? kTrainWarps : kPredictWarps, NT = WARPS * 32;
+  extern __shared__ __align__(16) unsigned char sm[];
+  const MlpSmem L = mlp_smem(p.Dp, WARPS, TRAIN);
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = lane >> 2, t4 = lane & 3, ld1 = p.Dp + 8;
+  bf16* W1 = reinterpret_cast<bf16*>(sm);
+  bf16* W2 = reinterpret_cast<bf16*>(sm + L.W2);
+  bf16* Xc = reinterpret_cast<bf16*>(sm + L.X);
+  bf16* X = Xc + warp * 16 * ld1;
+  float2* norm = reinterpret_cast<float2*>(sm + L.norm);
+  float* b1 = reinterpret_cast<float*>(sm + L.vec);
+  float *b2 = b1 + kH, *w30 = b2 + kH, *w31 = w30 + kH;
+  bf16* H1c = reinterpret_cast<bf16*>(sm + L.H1);
+  bf16* H2c = reinterpret_cast<bf16*>(sm + L.H2);
+  bf16* dZ2c = reinterpret_cast<bf16*>(sm + L.dZ2);
+  float* g1 = reinterpret_cast<float*>(sm + L.g1) + warp * 16 * kH;  // GELU'(Z1), by lane; then dZ1
+  bf16* dZ1c = reinterpret_cast<bf16*>(sm + L.g1);
+  uint16_t* list = TRAIN ? reinterpret_cast<uint16_t*>(g1) : reinterpret_cast<uint16_t*>(sm + L.list) + warp * kListed;
+  float* dc = reinterpret_cast<float*>(sm + L.d);  // [rows]: d0, d1, loss
+#pragma unroll 4
+  for (int r = warp; r < kH; r += WARPS)
+    for (int k = lane; k < p.Dp; k += 32) W1[r * ld1 + k] = k < p.D ? p.wb[r * p.D + k] : __float2bfloat16(0.0f);
+#pragma unroll 8
+  for (int i = tid; i < kH * kH / 8; i += NT)
+    *reinterpret_cast<uint4*>(W2 + (i >> 4) * kLd + (i & 15) * 8) = reinterpret_cast<const uint4*>(p.wb + p.oW2)[i];
+  for (int d = tid; d < p.D; d += NT) norm[d] = make_float2(p.norm[d], 1.0f / p.norm[p.D + d]);
+  for (int i = tid; i < kH; i += NT) {
+    b1[i] = p.w[p.ob1 + i];
+    b2[i] = p.w[p.ob2 + i];
+    w30[i] = __bfloat162float(p.wb[p.oW3 + i]);
+    w31[i] = __bfloat162float(p.wb[p.oW3 + kH + i]);
+  }
+  for (int i = lane; i < 16 * (p.Dp - p.D); i += 32) X[(i & 15) * ld1 + p.D + (i >> 4)] = __float2bfloat16(0.0f);
+  __syncthreads();
+  const float b30 = p.w[p.ob3], b31 = p.w[p.ob3 + 1];
+  const float* nt = p.norm + 2 * p.D;
+  const int64_t tiles = (p.n + 15) / 16;
+  // prediction: a warp's tiles one after the other; training: the CTA's warps stay together
+  bool add = false;
+#pragma unroll 1
+  for (int64_t tile0 = (int64_t)blockIdx.x * WARPS; tile0 < tiles; tile0 += (int64_t)gridDim.x * WARPS) {
+    const int64_t r0 = (tile0 + warp) * 16;
+    const int nr = (int)max((int64_t)0, min((int64_t)16, p.n - r0));
+    if (!TRAIN && nr == 0) break;
+    const uint32_t far = feature_tile<TRAIN>(p, X, ld1, norm, list, nr ? r0 : 0, nr, lane);
+    float acc[16][4] = {};
+#pragma unroll 1
+    for (int k0 = 0; k0 < p.Dp; k0 += 16) {
+      uint32_t a[4];
+      ldsm(a, X + (lane & 15) * ld1 + k0 + (lane >> 4) * 8);
+      rows_times_wt(acc, a, W1, ld1, k0, lane);
+    }
+    // hidden layer 1 as the A fragments of the next product
+    uint32_t h[8][4];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const float2 b = *reinterpret_cast<const float2*>(b1 + j * 8 + t4 * 2);
+      float v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float z = acc[j][q] + (q & 1 ? b.y : b.x);
+        v[q] = gelu(z);
+        if (TRAIN) g1[(j * 4 + q) * 32 + lane] = gelu_grad(z);
+      }
+      h[j >> 1][(j & 1) * 2] = pack_bf16(v[0], v[1]);
+      h[j >> 1][(j & 1) * 2 + 1] = pack_bf16(v[2], v[3]);
+      if (TRAIN) {
+        uint32_t* row = reinterpret_cast<uint32_t*>(H1c + (warp * 16 + g) * kLd + j * 8 + t4 * 2);
+        row[0] = h[j >> 1][(j & 1) * 2];
+        row[4 * kLd] = h[j >> 1][(j & 1) * 2 + 1];
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[j][q] = 0.0f;
+#pragma unroll
+    for (int kt = 0; kt < 8; ++kt) rows_times_wt(acc, h[kt], W2, kLd, kt * 16, lane);
+    // hidden layer 2 and the output head: rows g (o[0], o[1]) and g + 8 (o[2], o[3])
+    float o[4] = {};
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const int c = j * 8 + t4 * 2;
+      const float2 b = *reinterpret_cast<const float2*>(b2 + c);
+      const float2 u0 = *reinterpret_cast<const float2*>(w30 + c), u1 = *reinterpret_cast<const float2*>(w31 + c);
+#pragma unroll
+      for (int q = 0; q < 4; q += 2) {
+        const float z0 = acc[j][q] + b.x, z1 = acc[j][q + 1] + b.y;
+        const __nv_bfloat162 hh = __floats2bfloat162_rn(gelu(z0), gelu(z1));
+        const float2 f = __bfloat1622float2(hh);
+        o[q] += f.x * u0.x + f.y * u0.y;
+        o[q + 1] += f.x * u1.x + f.y * u1.y;
+        if (TRAIN) {
+          *reinterpret_cast<__nv_bfloat162*>(H2c + (warp * 16 + g + q * 4) * kLd + c) = hh;
+          acc[j][q] = gelu_grad(z0);
+          acc[j][q + 1] = gelu_grad(z1);
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      o[q] += __shfl_xor_sync(0xffffffffu, o[q], 1);
+      o[q] += __shfl_xor_sync(0xffffffffu, o[q], 2);
+      o[q] += q & 1 ? b31 : b30;
+    }
+    if (!TRAIN) {
+      const int r = g + (t4 & 1) * 8;
+      if (t4 < 2 && r < nr) {
+        const float l0 = (t4 ? o[2] : o[0]) * nt[2] + nt[0];
+        const float l1 = (t4 ? o[3] : o[1]) * nt[3] + nt[1];
+        const int64_t q = p.row0 + r0 + r;
+        if (p.ln_cost) p.ln_cost[q] = l0;
+        if (p.ln_h0) p.ln_h0[q] = l1;
+        if (p.cost) p.cost[q] = expf(fminf(l0, 80.0f));
+        if (p.h0)
+          p.h0[q] = far >> r & 1 ? __longlong_as_double(0x7ff8000000000000LL) : fmax(exp((double)l1), 1e-14);
+      }
+      __syncwarp();
+      continue;
+    }
+    // standardised targets: lanes 0 - 15 the cost of row `lane`, lanes 16 - 31 the first step
+    float ts = 0.0f;
+    if ((lane & 15) < nr) {
+      const int64_t q = p.row0 + r0 + (lane & 15);
+      const int64_t src = p.perm ? (int64_t)p.perm[q] : q;
+      const double t = log(lane < 16 ? fmax((double)p.sub[src], 1.0) : fmax(p.hf[src], 1e-300));
+      ts = (float)((t - nt[lane >> 4]) / nt[2 + (lane >> 4)]);
+    }
+    float d[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = g + (q >> 1) * 8;
+      const float res = o[q] - __shfl_sync(0xffffffffu, ts, r + (q & 1) * 16);
+      d[q] = r < nr ? res * p.inv_B : 0.0f;
+      o[q] = r < nr ? res : 0.0f;
+    }
+    if (t4 < 2) {
+      float* e = dc + (warp * 16 + g + t4 * 8) * 3;
+      const float d0 = t4 ? d[2] : d[0], d1 = t4 ? d[3] : d[1], e0 = t4 ? o[2] : o[0], e1 = t4 ? o[3] : o[1];
+      e[0] = d0;
+      e[1] = d1;
+      e[2] = 0.5f * (e0 * e0 + e1 * e1) * p.inv_B;
+    }
+    // dZ2, and dZ1 = (dZ2 W2) GELU'(Z1)
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      const int c = j * 8 + t4 * 2;
+      const float2 u0 = *reinterpret_cast<const float2*>(w30 + c), u1 = *reinterpret_cast<const float2*>(w31 + c);
+#pragma unroll
+      for (int q = 0; q < 4; q += 2) {
+        const uint32_t z = pack_bf16((d[q] * u0.x + d[q + 1] * u1.x) * acc[j][q],
+                                     (d[q] * u0.y + d[q + 1] * u1.y) * acc[j][q + 1]);
+        h[j >> 1][(j & 1) * 2 + q / 2] = z;
+        *reinterpret_cast<uint32_t*>(dZ2c + (warp * 16 + g + q * 4) * kLd + c) = z;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[j][q] = 0.0f;
+#pragma unroll
+    for (int kt = 0; kt < 8; ++kt) {
+      const bf16* w = W2 + (kt * 16 + (lane & 15)) * kLd + (lane >> 4) * 8;
+#pragma unroll
+      for (int np = 0; np < 8; ++np) {
+        uint32_t b[4];
+        ldsm_t(b, w + np * 16);
+        mma_bf16(acc[2 * np], h[kt], b[0], b[1]);
+        mma_bf16(acc[2 * np + 1], h[kt], b[2], b[3]);
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[j][q] *= g1[(j * 4 + q) * 32 + lane];
+    __syncwarp();
+    bf16* dZ1 = reinterpret_cast<bf16*>(g1);
+#pragma unroll
+    for (int j = 0; j < 16; ++j)
+#pragma unroll
+      for (int q = 0; q < 4; q += 2)
+        *reinterpret_cast<uint32_t*>(dZ1 + (g + q * 4) * kLd + j * 8 + t4 * 2) = pack_bf16(acc[j][q], acc[j][q + 1]);
+    __syncthreads();
+    // the CTA's contribution to the gradient
+    float* part = p.part + blockIdx.x * p.part_stride;
+    const int z1_step = 16 * kH * 2;  // dZ1's 16 rows of a warp lie in its g1 area
+    weight_gradient(dZ2c, 16 * kLd, H1c, kLd, kH, warp, lane, add, part + p.oW2);
+    weight_gradient(dZ1c, z1_step, Xc, ld1, p.D, warp, lane, add, part);
+    float s[4] = {};
+#pragma unroll 8
+    for (int r = 0; r < WARPS * 16; ++r) {
+      const float h2 = __bfloat162float(H2c[r * kLd + tid]);
+      s[0] += __bfloat162float(dZ1c[(r >> 4) * z1_step + (r & 15) * kLd + tid]);
+      s[1] += __bfloat162float(dZ2c[r * kLd + tid]);
+      s[2] += dc[r * 3] * h2;
+      s[3] += dc[r * 3 + 1] * h2;
+    }
+    const int64_t at[4] = {p.ob1 + tid, p.ob2 + tid, p.oW3 + tid, p.oW3 + kH + tid};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) part[at[q]] = add ? part[at[q]] + s[q] : s[q];
+    if (tid < 3) {  // b3's gradient and the loss
+      float v = 0.0f;
+      for (int r = 0; r < WARPS * 16; ++r) v += dc[r * 3 + tid];
+      float* w = part + p.ob3 + tid;
+      *w = add ? *w + v : v;
+    }
+    add = true;
+    __syncthreads();
   }
 }
 
-// column sums of a [rows][128] bf16 matrix into part[chunk][128]
-__global__ void k_colsum(const bf16* Z, int rows, int rows_per_block, float* part) {
-  const int col = threadIdx.x;
-  const int r0 = blockIdx.x * rows_per_block, r1 = min(rows, r0 + rows_per_block);
+// out[j] = sum over the S partials of part[s][j] in a fixed order, j <= nw; entry nw is the loss.
+// 128 entries a CTA, the partials dealt to eight groups of threads: all loads of a thread
+// are independent.
+__global__ void __launch_bounds__(1024) k_reduce(const float* part, int S, int64_t stride, int64_t nw, float* out,
+                                                 float* loss) {
+  __shared__ float sh[8][128];
+  const int64_t j = (int64_t)blockIdx.x * 128 + threadIdx.x;
   float s = 0.0f;
-  for (int r = r0; r < r1; ++r) s += __bfloat162float(Z[(size_t)r * kH + col]);
-  part[(size_t)blockIdx.x * kH + col] = s;
+  if (j <= nw) {
+#pragma unroll 8
+    for (int i = threadIdx.y; i < S; i += 8) s += part[i * stride + j];
+  }
+  sh[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.y == 0 && j <= nw) {
+    for (int i = 1; i < 8; ++i) s += sh[i][threadIdx.x];
+    if (j < nw) out[j] = s;
+    else *loss = s;
+  }
 }
 
 __global__ void k_adam(float* w, const float* g, float* m, float* v, bf16* wb, int64_t n, float lr, float b1,
@@ -373,12 +604,12 @@ struct chem_mlp_s {
   float* norm = nullptr;          // device: mu_x[D], sd_x[D], mu_t[2], sd_t[2]
   std::vector<float> norm_h;      // host copy
   int64_t adam_t = 0;
-  // scratch
-  int64_t cap = 0;
-  bf16 *X = nullptr, *H1 = nullptr, *H2 = nullptr, *dZ2 = nullptr, *dZ1 = nullptr;
-  float *Z1 = nullptr, *Z2 = nullptr, *Tb = nullptr, *part = nullptr;
-  int64_t part_cap = 0;
-  unsigned char* out_of_range = nullptr;  // [kChunk] per-row range flags (kept zero between calls)
+  // kept between calls: the CTAs' partial gradients, the gradient and loss on the host
+  float* part = nullptr;   // [num_sms][part_stride]
+  float* loss = nullptr;
+  float* host = nullptr;   // pinned, [nw + 1]
+  int64_t part_stride = 0;
+  int num_sms = 0;
   std::string err;
 };
 
@@ -394,41 +625,12 @@ static chem_status mlp_cuda(chem_mlp m, cudaError_t e, const char* what) {
     if (s_ != CHEM_OK) return s_;                           \
   } while (0)
 
-static void mlp_free_scratch(chem_mlp m) {
-  for (void* p : {(void*)m->X, (void*)m->H1, (void*)m->H2, (void*)m->dZ2, (void*)m->dZ1, (void*)m->Z1, (void*)m->Z2,
-                  (void*)m->Tb})
-    if (p) cudaFree(p);
-  m->X = m->H1 = m->H2 = m->dZ2 = m->dZ1 = nullptr;
-  m->Z1 = m->Z2 = m->Tb = nullptr;
-  m->cap = 0;
-}
-
-static chem_status mlp_scratch(chem_mlp m, int64_t rows, bool train) {
-  if (rows <= m->cap && (!train || m->Z1)) return CHEM_OK;
-  cudaDeviceSynchronize();
-  mlp_free_scratch(m);
-  const int64_t r = std::max<int64_t>(rows, 1024);
-  MLP_TRY(m, cudaMalloc(&m->X, r * m->D * sizeof(bf16)));
-  MLP_TRY(m, cudaMalloc(&m->H1, r * kH * sizeof(bf16)));
-  MLP_TRY(m, cudaMalloc(&m->H2, r * kH * sizeof(bf16)));
-  if (train) {
-    MLP_TRY(m, cudaMalloc(&m->dZ2, r * kH * sizeof(bf16)));
-    MLP_TRY(m, cudaMalloc(&m->dZ1, r * kH * sizeof(bf16)));
-    MLP_TRY(m, cudaMalloc(&m->Z1, r * kH * sizeof(float)));
-    MLP_TRY(m, cudaMalloc(&m->Z2, r * kH * sizeof(float)));
-    MLP_TRY(m, cudaMalloc(&m->Tb, r * 2 * sizeof(float)));
-  }
-  m->cap = r;
-  return CHEM_OK;
-}
-
-static chem_status mlp_part(chem_mlp m, int64_t floats) {
-  if (floats <= m->part_cap) return CHEM_OK;
-  cudaDeviceSynchronize();
-  if (m->part) cudaFree(m->part);
-  m->part = nullptr;
-  MLP_TRY(m, cudaMalloc(&m->part, floats * sizeof(float)));
-  m->part_cap = floats;
+// what a gradient needs beside the weights; allocated with the first one
+static chem_status mlp_train_scratch(chem_mlp m) {
+  if (m->host) return CHEM_OK;
+  if (!m->part) MLP_TRY(m, cudaMalloc(&m->part, m->num_sms * m->part_stride * sizeof(float)));
+  if (!m->loss) MLP_TRY(m, cudaMalloc(&m->loss, sizeof(float)));
+  MLP_TRY(m, cudaMallocHost(&m->host, (m->nw + 1) * sizeof(float)));
   return CHEM_OK;
 }
 
@@ -461,7 +663,15 @@ extern "C" chem_status chem_mlp_create(int32_t n_species, uint64_t seed, chem_ml
   m->norm_h.assign(2 * D + 4, 0.0f);
   for (int d = 0; d < D; ++d) m->norm_h[D + d] = 1.0f;
   m->norm_h[2 * D + 2] = m->norm_h[2 * D + 3] = 1.0f;
-  cudaError_t e = cudaMalloc(&m->w, m->nw * 4);
+  m->part_stride = (m->nw + 32) / 32 * 32;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&m->num_sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_mlp<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemMlp);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_mlp<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmemMlp);
+  if (e == cudaSuccess) e = cudaMalloc(&m->w, m->nw * 4);
   if (e == cudaSuccess) e = cudaMalloc(&m->g, m->nw * 4);
   if (e == cudaSuccess) e = cudaMalloc(&m->m, m->nw * 4);
   if (e == cudaSuccess) e = cudaMalloc(&m->v, m->nw * 4);
@@ -486,10 +696,10 @@ extern "C" chem_status chem_mlp_create(int32_t n_species, uint64_t seed, chem_ml
 extern "C" chem_status chem_mlp_destroy(chem_mlp m) {
   if (!m) return CHEM_ERR_INVALID_ARG;
   cudaDeviceSynchronize();
-  mlp_free_scratch(m);
   for (void* p : {(void*)m->w, (void*)m->g, (void*)m->m, (void*)m->v, (void*)m->wb, (void*)m->norm, (void*)m->part,
-                  (void*)m->out_of_range})
+                  (void*)m->loss})
     if (p) cudaFree(p);
+  if (m->host) cudaFreeHost(m->host);
   delete m;
   return CHEM_OK;
 }
@@ -532,87 +742,36 @@ extern "C" chem_status chem_mlp_set_params(chem_mlp m, const float* buf, int64_t
 // ---------------------------------------------------------------------------
 // building blocks
 // ---------------------------------------------------------------------------
-// returns the number of K splits used
-static int gemm(cudaStream_t st, const bf16* A, long long sam, long long sak, const bf16* B, long long sbn,
-                 long long sbk, int M, int N, int K, int splits, int mode, float* C, long long ldc,
-                 const float* bias, float* Zout, bf16* Hout, const float* Zin, bf16* dZout) {
-  GemmP p;
-  p.A = A;
-  p.sam = sam;
-  p.sak = sak;
-  p.B = B;
-  p.sbn = sbn;
-  p.sbk = sbk;
-  p.M = M;
-  p.N = N;
-  p.K = K;
-  p.kchunk = ((K + splits - 1) / splits + 31) / 32 * 32;
-  p.mode = mode;
-  p.C = C;
-  p.ldc = ldc;
-  p.zstride = (long long)M * ldc;
-  p.bias = bias;
-  p.Zout = Zout;
-  p.Hout = Hout;
-  p.Zin = Zin;
-  p.dZout = dZout;
-  dim3 grid((M + 63) / 64, (N + 63) / 64, (K + p.kchunk - 1) / p.kchunk);
-  k_gemm<<<grid, 128, 0, st>>>(p);
-  return (int)grid.z;
+static MlpP mlp_args(chem_mlp m, int64_t n, const double* T, const double* p, const double* Y) {
+  MlpP a{};
+  a.T = T;
+  a.p = p;
+  a.Y = Y;
+  a.n = n;
+  a.K = m->K;
+  a.D = m->D;
+  a.Dp = (m->D + 15) / 16 * 16;
+  a.norm = m->norm;
+  a.wb = m->wb;
+  a.w = m->w;
+  a.ob1 = m->ob1;
+  a.oW2 = m->oW2;
+  a.ob2 = m->ob2;
+  a.oW3 = m->oW3;
+  a.ob3 = m->ob3;
+  a.nw = m->nw;
+  return a;
 }
 
-// forward of `rows` standardised rows in m->X; training keeps Z1, Z2
-static void forward(chem_mlp m, int rows, bool train, cudaStream_t st) {
-  const int D = m->D;
-  gemm(st, m->X, D, 1, m->wb + m->oW1, D, 1, rows, kH, D, 1, 1, nullptr, 0, m->w + m->ob1, train ? m->Z1 : nullptr,
-       m->H1, nullptr, nullptr);
-  gemm(st, m->H1, kH, 1, m->wb + m->oW2, kH, 1, rows, kH, kH, 1, 1, nullptr, 0, m->w + m->ob2,
-       train ? m->Z2 : nullptr, m->H2, nullptr, nullptr);
-}
-
-static int head_warps(int rows) { return std::max(1, std::min(1024, (rows + 31) / 32)); }
-
-// forward + backward of the batch in m->X / m->Tb; gradient into m->g; returns device loss in part tail
-static chem_status fwd_bwd(chem_mlp m, int rows, cudaStream_t st, float* loss_dev) {
-  const int D = m->D;
-  forward(m, rows, true, st);
-  const int hw = head_warps(rows);
-  const int splits = std::max(1, std::min(64, rows / 256));
-  const int colblocks = std::max(1, std::min(256, rows / 64));
-  const int64_t need = std::max<int64_t>({(int64_t)hw * (2 * kH + 3), (int64_t)splits * kH * std::max(D, kH),
-                                          (int64_t)colblocks * kH});
-  chem_status s = mlp_part(m, need);
-  if (s != CHEM_OK) return s;
-  HeadP hp{};
-  hp.H2 = m->H2;
-  hp.Z2 = m->Z2;
-  hp.W3 = m->wb + m->oW3;
-  hp.b3 = m->w + m->ob3;
-  hp.Tb = m->Tb;
-  hp.rows = rows;
-  hp.inv_B = 1.0f / (float)rows;
-  hp.dZ2 = m->dZ2;
-  hp.part = m->part;
-  k_head<<<(hw * 32 + 255) / 256, 256, 0, st>>>(hp, 1);
-  // W3, b3 gradient and the loss
-  k_reduce<<<2, 128, 0, st>>>(m->part, hw, 2 * kH + 3, 2 * kH + 2, m->g + m->oW3);
-  k_reduce<<<1, 32, 0, st>>>(m->part + 2 * kH + 2, hw, 2 * kH + 3, 1, loss_dev);
-  // dW2 = dZ2^T H1 (split-K over the batch), db2 = column sums of dZ2
-  const int S2 = gemm(st, m->dZ2, 1, kH, m->H1, 1, kH, kH, kH, rows, splits, 0, m->part, kH, nullptr, nullptr,
-                      nullptr, nullptr, nullptr);
-  k_reduce<<<64, 256, 0, st>>>(m->part, S2, kH * kH, kH * kH, m->g + m->oW2);
-  const int rpb = (rows + colblocks - 1) / colblocks;
-  k_colsum<<<colblocks, kH, 0, st>>>(m->dZ2, rows, rpb, m->part);
-  k_reduce<<<1, kH, 0, st>>>(m->part, colblocks, kH, kH, m->g + m->ob2);
-  // dZ1 = (dZ2 W2) * GELU'(Z1)
-  gemm(st, m->dZ2, kH, 1, m->wb + m->oW2, 1, kH, rows, kH, kH, 1, 2, nullptr, 0, nullptr, nullptr, nullptr, m->Z1,
-       m->dZ1);
-  // dW1 = dZ1^T X, db1 = column sums of dZ1
-  const int S1 = gemm(st, m->dZ1, 1, kH, m->X, 1, D, kH, D, rows, splits, 0, m->part, D, nullptr, nullptr, nullptr,
-                      nullptr, nullptr);
-  k_reduce<<<64, 256, 0, st>>>(m->part, S1, kH * D, kH * D, m->g + m->oW1);
-  k_colsum<<<colblocks, kH, 0, st>>>(m->dZ1, rows, rpb, m->part);
-  k_reduce<<<1, kH, 0, st>>>(m->part, colblocks, kH, kH, m->g + m->ob1);
+// gradient (into m->g) and loss (device) of the rows [b0, b0 + rows) of the order `perm`
+static chem_status fwd_bwd(chem_mlp m, MlpP a, cudaStream_t st, float* loss_dev) {
+  a.inv_B = 1.0f / (float)a.n;
+  a.part = m->part;
+  a.part_stride = m->part_stride;
+  const int rows = kTrainWarps * 16;
+  const int grid = (int)std::min<int64_t>((a.n + rows - 1) / rows, m->num_sms);
+  k_mlp<true><<<grid, kTrainWarps * 32, mlp_smem(a.Dp, kTrainWarps, true).total, st>>>(a);
+  k_reduce<<<(int)((m->nw + 128) / 128), dim3(128, 8), 0, st>>>(m->part, grid, m->part_stride, m->nw, m->g, loss_dev);
   return mlp_cuda(m, cudaGetLastError(), "mlp backward");
 }
 
@@ -661,26 +820,20 @@ extern "C" chem_status chem_mlp_train(chem_mlp m, int64_t n, const double* T, co
     return CHEM_ERR_INVALID_ARG;
   if (n > 2147483647LL) return CHEM_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const int D = m->D;
   chem_status s = set_normalisation(m, n, T, p, Y, substeps, h_first, st);
   if (s != CHEM_OK) return s;
-  // standardised features and targets of all samples
-  bf16* Xall = nullptr;
-  float* Tall = nullptr;
+  s = mlp_train_scratch(m);
+  if (s != CHEM_OK) return s;
   int* perm_d = nullptr;
   float* loss_d = nullptr;
-  MLP_TRY(m, cudaMalloc(&Xall, (size_t)n * D * sizeof(bf16)));
-  MLP_TRY(m, cudaMalloc(&Tall, (size_t)n * 2 * sizeof(float)));
   MLP_TRY(m, cudaMalloc(&perm_d, (size_t)n * sizeof(int)));
   const int B = (int)std::min<int64_t>(batch, n);
   const int nb = (int)((n + B - 1) / B);
   MLP_TRY(m, cudaMalloc(&loss_d, (size_t)nb * sizeof(float)));
-  const int gridE = (int)std::min<int64_t>(((int64_t)n * D + 255) / 256, 4096);
-  k_features<<<gridE, 256, 0, st>>>(T, p, Y, m->K, 0, n, m->norm, Xall);
-  k_targets<<<(int)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, st>>>(substeps, h_first, n, m->norm + 2 * D,
-                                                                            Tall);
-  s = mlp_scratch(m, B, true);
-  if (s != CHEM_OK) return s;
+  MlpP a = mlp_args(m, 0, T, p, Y);
+  a.sub = substeps;
+  a.hf = h_first;
+  a.perm = perm_d;
   std::vector<int> perm(n);
   std::mt19937_64 rng(seed);
   std::vector<float> batch_losses(nb);
@@ -690,10 +843,9 @@ extern "C" chem_status chem_mlp_train(chem_mlp m, int64_t n, const double* T, co
     std::shuffle(perm.begin(), perm.end(), rng);
     MLP_TRY(m, cudaMemcpyAsync(perm_d, perm.data(), n * sizeof(int), cudaMemcpyHostToDevice, st));
     for (int bi = 0; bi < nb; ++bi) {
-      const int64_t b0 = (int64_t)bi * B;
-      const int rows = (int)std::min<int64_t>(B, n - b0);
-      k_gather<<<256, 256, 0, st>>>(Xall, Tall, perm_d, b0, rows, D, m->X, m->Tb);
-      s = fwd_bwd(m, rows, st, loss_d + bi);
+      a.row0 = (int64_t)bi * B;
+      a.n = std::min<int64_t>(B, n - a.row0);
+      s = fwd_bwd(m, a, st, loss_d + bi);
       if (s != CHEM_OK) return s;
       ++m->adam_t;
       float c1, c2;
@@ -710,8 +862,6 @@ extern "C" chem_status chem_mlp_train(chem_mlp m, int64_t n, const double* T, co
     }
   }
   MLP_TRY(m, cudaStreamSynchronize(st));
-  cudaFree(Xall);
-  cudaFree(Tall);
   cudaFree(perm_d);
   cudaFree(loss_d);
   return mlp_cuda(m, cudaGetLastError(), "chem_mlp_train");
@@ -722,23 +872,18 @@ extern "C" chem_status chem_mlp_gradient(chem_mlp m, int64_t n, const double* T,
                                          float* grad_host, void* stream) {
   if (!m || n < 1 || n > 1 << 20 || !T || !p || !Y || !substeps || !h_first) return CHEM_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const int D = m->D;
-  chem_status s = mlp_scratch(m, n, true);
+  chem_status s = mlp_train_scratch(m);
   if (s != CHEM_OK) return s;
-  const int gridE = (int)std::min<int64_t>(((int64_t)n * D + 255) / 256, 4096);
-  k_features<<<gridE, 256, 0, st>>>(T, p, Y, m->K, 0, n, m->norm, m->X);
-  k_targets<<<(int)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, st>>>(substeps, h_first, n, m->norm + 2 * D,
-                                                                            m->Tb);
-  float* loss_d = nullptr;
-  MLP_TRY(m, cudaMalloc(&loss_d, sizeof(float)));
-  s = fwd_bwd(m, (int)n, st, loss_d);
+  MlpP a = mlp_args(m, n, T, p, Y);
+  a.sub = substeps;
+  a.hf = h_first;
+  s = fwd_bwd(m, a, st, m->loss);
   if (s != CHEM_OK) return s;
-  float l = 0.0f;
-  MLP_TRY(m, cudaMemcpyAsync(&l, loss_d, 4, cudaMemcpyDeviceToHost, st));
-  if (grad_host) MLP_TRY(m, cudaMemcpyAsync(grad_host, m->g, m->nw * 4, cudaMemcpyDeviceToHost, st));
+  MLP_TRY(m, cudaMemcpyAsync(m->host + m->nw, m->loss, 4, cudaMemcpyDeviceToHost, st));
+  if (grad_host) MLP_TRY(m, cudaMemcpyAsync(m->host, m->g, m->nw * 4, cudaMemcpyDeviceToHost, st));
   MLP_TRY(m, cudaStreamSynchronize(st));
-  cudaFree(loss_d);
-  if (loss_host) *loss_host = l;
+  if (grad_host) std::memcpy(grad_host, m->host, m->nw * 4);
+  if (loss_host) *loss_host = m->host[m->nw];
   return CHEM_OK;
 }
 
@@ -760,34 +905,16 @@ extern "C" chem_status chem_mlp_apply_gradient(chem_mlp m, const float* grad_hos
 // deviations get a NaN initial step (the integrator then takes its heuristic).
 static chem_status predict_into(chem_mlp m, int64_t n, const double* T, const double* p, const double* Y, float* ln_cost,
                                 float* ln_h0, float* cost, double* h0, cudaStream_t st, float zmax = 0.0f) {
-  const int D = m->D;
-  chem_status s = mlp_scratch(m, std::min<int64_t>(n, kChunk), false);
-  if (s != CHEM_OK) return s;
-  if (zmax > 0.0f && h0 && !m->out_of_range) {
-    MLP_TRY(m, cudaMalloc(&m->out_of_range, kChunk));
-    MLP_TRY(m, cudaMemsetAsync(m->out_of_range, 0, kChunk, st));
-  }
-  if (!h0) zmax = 0.0f;
-  for (int64_t r0 = 0; r0 < n; r0 += kChunk) {
-    const int rows = (int)std::min<int64_t>(kChunk, n - r0);
-    const int gridE = (int)std::min<int64_t>(((int64_t)rows * D + 255) / 256, 4096);
-    k_features<<<gridE, 256, 0, st>>>(T, p, Y, m->K, r0, rows, m->norm, m->X, zmax, m->out_of_range);
-    forward(m, rows, false, st);
-    HeadP hp{};
-    hp.H2 = m->H2;
-    hp.W3 = m->wb + m->oW3;
-    hp.b3 = m->w + m->ob3;
-    hp.rows = rows;
-    hp.norm_t = m->norm + 2 * D;
-    hp.ln_cost = ln_cost;
-    hp.ln_h0 = ln_h0;
-    hp.cost = cost;
-    hp.h0 = h0;
-    hp.out_of_range = zmax > 0.0f ? m->out_of_range : nullptr;
-    hp.out0 = r0;
-    const int hw = head_warps(rows);
-    k_head<<<(hw * 32 + 255) / 256, 256, 0, st>>>(hp, 0);
-  }
+  MlpP a = mlp_args(m, n, T, p, Y);
+  a.zmax = h0 ? zmax : 0.0f;
+  a.ln_cost = ln_cost;
+  a.ln_h0 = ln_h0;
+  a.cost = cost;
+  a.h0 = h0;
+  const size_t smem = mlp_smem(a.Dp, kPredictWarps, false).total;
+  const int64_t ctas = (n + kPredictWarps * 16 - 1) / (kPredictWarps * 16);
+  const int grid = (int)std::min<int64_t>(ctas, (int64_t)m->num_sms * (2 * (smem + 1024) <= 233472 ? 2 : 1));
+  k_mlp<false><<<grid, kPredictWarps * 32, smem, st>>>(a);
   return mlp_cuda(m, cudaGetLastError(), "chem_mlp_predict");
 }
 
