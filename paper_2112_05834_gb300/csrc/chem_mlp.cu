@@ -20,6 +20,7 @@
 
 #include "chem.h"
 #include "chem_capi_internal.h"
+#include "chem_fixed.cuh"
 #include "chem_mlp.h"
 #include "chem_mlp_internal.h"
 
@@ -85,17 +86,22 @@ __global__ void k_target_stats(const int32_t* sub, const double* hf, int64_t n, 
 // ---------------------------------------------------------------------------
 // forward pass (and backward pass) of a batch in one kernel
 //
-// A warp takes 16 rows through the whole model: it standardises their features into its own
-// BF16 tile in shared memory, and since the accumulator fragment of one m16n8k16 product is
-// laid out like the A fragment of the next, both hidden layers stay in registers; the
-// weights are read from shared memory, where each CTA loads them once.
+// Everything between the features and the results stays in shared memory and registers; the
+// weights are loaded once per CTA. A layer is computed 32 columns at a time, so that the code
+// of its product and its GELUs (16 a lane) exists once: with all 128 columns in registers it
+// was 64 KB long, twice the instruction cache, at 128 registers a thread.
+// Prediction: each warp takes 16 rows through the model on its own. Training: a CTA takes 64
+// rows, four warps to 16 of them, each with 32 columns of every layer, so that the dependent
+// layers are short and an SM has 16 warps although a minibatch is one tile per SM.
 //
 // Four kernels per pass with one FP64 logarithm and division per feature took 527 us for
 // 65,536 rows of 54 species and were bound by the FP64 pipe (3.5 M logarithms of some 25
 // operations at 19 cycles per warp and SM: 180 us) and by element-wise strided operand
-// loads. Training keeps what the backward pass needs in shared memory: a CTA's 64 rows give
-// both weight gradients as products of tiles that never leave the SM (334 us for 8,192 rows
-// in 17 launches before, with two passes over the activations in global memory per layer).
+// loads; this kernel takes 47 us. It is bound by issue and dependent instructions (0.56 warp
+// instructions per cycle and scheduler): half of its 7,800 instructions per 16 rows are the
+// 256 x 16 GELUs' erff. The gradient of 8,192 rows took 332 us in 17 launches, with two passes
+// over the activations in global memory per layer, copies and an allocation; now 61 us, of
+// which this kernel has 31 (one tile per SM: the layers' chain) and the reduction 6.
 // ---------------------------------------------------------------------------
 struct MlpP {
   const double *T, *p, *Y;
@@ -119,29 +125,28 @@ struct MlpP {
 };
 
 constexpr int kLd = kH + 8;  // row length of the 128-wide tiles (rows 16 bytes off in banks: no conflicts)
-constexpr int kPredictWarps = 8, kTrainWarps = 4;
+constexpr int kPredictWarps = 16, kTrainWarps = 16, kTrainRows = 64;
 constexpr size_t kMaxSmemMlp = 232448;
-constexpr int kFeatureBatch = 8;                      // loads in flight per lane
-constexpr int kListed = 32 + 32 * kFeatureBatch;  // features a warp may have waiting for FP64
+constexpr int kFeatureBatch = 14;                // loads in flight per lane
+constexpr int kListed = 32 + 32 * kFeatureBatch;  // features a warp may have listed
 
 struct MlpSmem {  // byte offsets
-  int W2, X, norm, vec, list, H1, H2, dZ2, g1, d, total;
+  int W2, norm, vec, X, H1, H2, dZ2, dZ1, head, total;
 };
-__host__ __device__ inline MlpSmem mlp_smem(int Dp, int warps, bool train) {
+// rows: of the CTA's tiles
+__host__ __device__ inline MlpSmem mlp_smem(int Dp, int rows, bool train) {
   MlpSmem o;
-  const int ld1 = Dp + 8;
+  const int ld1 = Dp + 8, tile = rows * kLd * 2;
   o.W2 = kH * ld1 * 2;
-  o.X = o.W2 + kH * kLd * 2;
-  o.norm = o.X + warps * 16 * ld1 * 2;
+  o.norm = o.W2 + kH * kLd * 2;
   o.vec = o.norm + Dp * 8;
-  o.list = o.vec + 4 * kH * 4;
-  o.H1 = o.list + (train ? 0 : warps * kListed * 2);  // training: in the g1 area, unused by then
-  const int tile = train ? warps * 16 * kLd * 2 : 0;
+  o.X = o.vec + 4 * kH * 4;
+  o.H1 = o.X + rows * ld1 * 2;
   o.H2 = o.H1 + tile;
-  o.dZ2 = o.H2 + tile;
-  o.g1 = o.dZ2 + tile;
-  o.d = o.g1 + (train ? warps * 16 * kH * 4 : 0);
-  o.total = o.d + (train ? warps * 16 * 12 : 0);
+  o.dZ2 = o.H2 + (train ? tile : 0);
+  o.dZ1 = o.dZ2 + (train ? tile : 0);
+  o.head = o.dZ1 + (train ? tile : 0);
+  o.total = o.head + (train ? rows * 13 * 4 : 0);
   return o;
 }
 
@@ -167,16 +172,28 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-// acc[16 rows][128] += A (fragments of kt16 x 16 columns) W^T for W stored [128][k]
-__device__ __forceinline__ void rows_times_wt(float (&acc)[16][4], const uint32_t (&a)[4], const bf16* W, int ld,
-                                              int k0, int lane) {
-  const bf16* w = W + ((lane & 7) + ((lane >> 4) << 3)) * ld + k0 + ((lane >> 3) & 1) * 8;
+// acc[16 rows][32 columns] += A B over ksteps x 16: A [row][k], B stored [column][k], or with
+// BT [k][column]
+template <bool BT>
+__device__ __forceinline__ void product(float (&acc)[4][4], const bf16* A, int lda, const bf16* B, int ldb, int ksteps,
+                                        int lane) {
+  A += (lane & 15) * lda + (lane >> 4) * 8;
+  B += BT ? (lane & 15) * ldb + (lane >> 4) * 8 : ((lane & 7) + ((lane >> 4) << 3)) * ldb + ((lane >> 3) & 1) * 8;
+  const int kb = BT ? 16 * ldb : 16, nb = BT ? 16 : 16 * ldb;
+#pragma unroll 4
+  for (int k = 0; k < ksteps; ++k) {
+    uint32_t a[4], b[2][4];
+    ldsm(a, A + k * 16);
 #pragma unroll
-  for (int np = 0; np < 8; ++np) {
-    uint32_t b[4];
-    ldsm(b, w + np * 16 * ld);
-    mma_bf16(acc[2 * np], a, b[0], b[1]);
-    mma_bf16(acc[2 * np + 1], a, b[2], b[3]);
+    for (int h = 0; h < 2; ++h) {
+      if (BT) ldsm_t(b[h], B + k * kb + h * nb);
+      else ldsm(b[h], B + k * kb + h * nb);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      mma_bf16(acc[2 * h], a, b[h][0], b[h][1]);
+      mma_bf16(acc[2 * h + 1], a, b[h][2], b[h][3]);
+    }
   }
 }
 
@@ -212,16 +229,42 @@ __device__ __forceinline__ bool feature_fast(double v, float2 norm, float* z, fl
   return ok && fabsf(*z) > 1e-30f && fabsf(*z) < 1e30f;
 }
 
-// One warp's 16 x D feature tile (BF16); rows beyond nr are zero. The BF16 value is that of
-// the FP64 formula: where the FP32 value's error bound reaches across a rounding boundary (or
-// across zmax), some one element in a thousand, the element is put on a list and the warp
-// goes through the formula for all of those side by side. Returns the rows beyond zmax.
-template <bool TRAIN>
+// Whether every value in [z - e, z + e] rounds to the same BF16 and lies on one side of zmax
+// (zmax 0: none); the bounds are formed from z's two parts.
+__device__ __forceinline__ bool feature_settled(float z, float zl, float e, float zmax) {
+  const uint32_t h = pack_bf16(z + (zl - e), z + (zl + e));
+  return !((h ^ (h >> 16)) & 0xffffu) && !(zmax > 0.0f && fabsf(fabsf(z) - zmax) <= fabsf(zl) + e);
+}
+
+// The same with the logarithm in 64-bit fixed point (52 fractional bits, within 2^-51): the
+// quotient to twice FP32's precision, z + zl, with a bound e on its error.
+__device__ __forceinline__ bool feature_fixed(double s, float mu, float sd, float* z, float* zl, float* e) {
+  const int ex = __double2hiint(s) >> 20;
+  if (ex < 1 || ex >= 2047 || !(fabsf(mu) < 512.0f)) return false;  // also negative s
+  const long long t = chem::fx_log(s, 52) - chem::fx_from_double((double)mu);
+  const float th = (float)t, inv = 1.0f / sd;
+  const float tl = (float)(t - (long long)th);
+  constexpr float kUnit = 2.220446049250313e-16f;  // 2^-52
+  const float q = th * inv;
+  *z = q * kUnit;
+  *zl = (fmaf(-q, sd, th) + tl) * inv * kUnit;
+  *e = fmaf(fabsf(*z), 1e-12f, fmaf(fabsf(mu), 2.0f, 3.0f) * kUnit * fabsf(inv));  // with the formula's own rounding
+  return fabsf(*z) > 1e-18f && fabsf(*z) < 1e18f;
+}
+
+// A warp's R x D feature tile (BF16); rows beyond nr are zero. The BF16 value is that of the
+// FP64 formula: where the FP32 value's error bound reaches across a rounding boundary (or
+// across zmax), some one element in 500 and a pressure that is the same everywhere, the
+// element is put on a list, and the warp goes through those side by side: in fixed point,
+// and where even that does not settle the rounding, by the formula itself. (By the formula
+// for all of the list, its 66 FP64 instructions per warp took a quarter of the kernel's time.)
+// Returns the rows beyond zmax.
+template <bool TRAIN, int R>
 __device__ __forceinline__ uint32_t feature_tile(const MlpP& p, bf16* X, int ld, const float2* norm, uint16_t* list,
                                                  int64_t r0, int nr, int lane) {
-  const int K = p.K, EY = 16 * K;
+  const int K = p.K, EY = R * K;
   const uint32_t inv_k = (1u << 20) / (uint32_t)K + 1;  // e / K for e < 16 K, K < 256
-  const int64_t mine = p.row0 + r0 + ((lane & 15) < nr ? lane & 15 : 0);
+  const int64_t mine = p.row0 + r0 + ((lane & (R - 1)) < nr ? lane & (R - 1) : 0);
   const int64_t src = TRAIN && p.perm ? (int64_t)p.perm[mine] : mine;
   uint32_t far = 0;
   int cnt = 0;
@@ -234,18 +277,22 @@ __device__ __forceinline__ uint32_t feature_tile(const MlpP& p, bf16* X, int ld,
     for (int i0 = 0; i0 < cnt; i0 += 32) {
       const int c = list[min(i0 + lane, cnt - 1)];
       const int q = c - EY;
-      const int r = q >= 0 ? q & 15 : (int)((uint32_t)c * inv_k >> 20);
-      const int d = q >= 0 ? q >> 4 : c - r * K + 2;
+      const int r = q >= 0 ? q & (R - 1) : (int)((uint32_t)c * inv_k >> 20);
+      const int d = q >= 0 ? q / R : c - r * K + 2;
       const int64_t row = __shfl_sync(0xffffffffu, src, r);
-      const double x = feature(p.T, p.p, p.Y, K, row, d);
-      put(r, d, (float)((x - p.norm[d]) / p.norm[p.D + d]));
+      const float mu = p.norm[d], sd = p.norm[p.D + d];
+      float z = 0.0f, zl = 0.0f, e = 0.0f;
+      bool ok = d > 0 && feature_fixed(d == 1 ? p.p[row] : p.Y[(size_t)row * K + (d - 2)] + 1e-20, mu, sd, &z, &zl, &e);
+      ok = ok && feature_settled(z, zl, e, p.zmax);
+      z += zl;
+      if (!ok) z = (float)((feature(p.T, p.p, p.Y, K, row, d) - mu) / sd);
+      put(r, d, z);
     }
     __syncwarp();
     cnt = 0;
   };
   auto take = [&](int code, int r, int d, bool valid, bool ok, float z, float e) {
-    const uint32_t h = pack_bf16(z - e, z + e);
-    const bool slow = valid && (!ok || ((h ^ (h >> 16)) & 0xffffu) || (p.zmax > 0.0f && fabsf(fabsf(z) - p.zmax) <= e));
+    const bool slow = valid && (!ok || !feature_settled(z, 0.0f, e, p.zmax));
     if (valid && !slow) put(r, d, z);
     const uint32_t m = __ballot_sync(0xffffffffu, slow);
     if (m) {
@@ -254,17 +301,17 @@ __device__ __forceinline__ uint32_t feature_tile(const MlpP& p, bf16* X, int ld,
     }
   };
   {
-    const int r = lane & 15, d = lane >> 4;
-    const bool valid = r < nr;
+    const int r = lane & (R - 1), d = lane / R;  // lanes from 2 R on have no element
+    const bool valid = d < 2 && r < nr;
     float z, e;
     bool ok;
     if (d == 0) ok = feature_fast<FEAT_T>(p.T[src], norm[0], &z, &e);
     else ok = feature_fast<FEAT_P>(p.p[src], norm[1], &z, &e);
     __syncwarp();
-    if (!valid) X[r * ld + d] = __float2bfloat16(0.0f);
+    if (d < 2 && !valid) X[r * ld + d] = __float2bfloat16(0.0f);
     take(EY + lane, r, d, valid, ok, z, e);
   }
-  constexpr int U = kFeatureBatch;
+  constexpr int U = R == 16 ? kFeatureBatch : 8;
 #pragma unroll 1
   for (int e0 = 0; e0 < EY; e0 += 32 * U) {
     double v[U];
@@ -281,6 +328,7 @@ __device__ __forceinline__ uint32_t feature_tile(const MlpP& p, bf16* X, int ld,
     }
 #pragma unroll
     for (int j = 0; j < U; ++j) {
+      if (e0 + j * 32 >= EY) break;
       const int i = e0 + j * 32 + lane;
       const int r = (int)((uint32_t)min(i, EY - 1) * inv_k >> 20), k = min(i, EY - 1) - r * K;
       float z, e;
@@ -294,71 +342,69 @@ __device__ __forceinline__ uint32_t feature_tile(const MlpP& p, bf16* X, int ld,
   return __reduce_or_sync(0xffffffffu, far);
 }
 
-// out[o][i] (+)= sum over the CTA's 64 rows of A[row][o] B[row][i], o in the warp's 32, i < cols
-__device__ __forceinline__ void weight_gradient(const bf16* A, int a_step, const bf16* B, int ldb, int cols, int warp,
-                                                int lane, bool add, float* out) {
+// out[o][i] (+)= sum over the CTA's 64 rows of A[row][o] B[row][i], o < 128, i < cols, in pieces
+// of 16 x 32 dealt to the warps
+__device__ __forceinline__ void weight_gradient(const bf16* A, const bf16* B, int ldb, int cols, int warp, int lane,
+                                                bool add, float* out) {
   const int ar = (lane & 7) + ((lane >> 4) << 3), am = ((lane >> 3) & 1) * 8;
   const int br = lane & 15, bn = (lane >> 4) * 8;
-  const int pad = (cols + 15) / 16 * 16;
+  const int chunks = (cols + 31) / 32;
+  const bool pairs = cols % 2 == 0;
 #pragma unroll 1
-  for (int mt = 0; mt < 2; ++mt) {
-    const int o0 = warp * 32 + mt * 16;
-#pragma unroll 1
-    for (int c0 = 0; c0 < pad; c0 += 64) {
-      float acc[8][4] = {};
+  for (int u = warp; u < 8 * chunks; u += kTrainWarps) {
+    const int o0 = (u & 7) * 16, c0 = (u >> 3) * 32;
+    const bool second = c0 + 16 < cols;
+    float acc[4][4] = {};
 #pragma unroll
-      for (int kt = 0; kt < 4; ++kt) {
-        uint32_t a[4];
-        ldsm_t(a, A + kt * a_step + ar * kLd + o0 + am);
+    for (int kt = 0; kt < kTrainRows / 16; ++kt) {
+      uint32_t a[4], b[4];
+      ldsm_t(a, A + (kt * 16 + ar) * kLd + o0 + am);
+      ldsm_t(b, B + (kt * 16 + br) * ldb + c0 + bn);
+      mma_bf16(acc[0], a, b[0], b[1]);
+      mma_bf16(acc[1], a, b[2], b[3]);
+      if (second) {
+        ldsm_t(b, B + (kt * 16 + br) * ldb + c0 + 16 + bn);
+        mma_bf16(acc[2], a, b[0], b[1]);
+        mma_bf16(acc[3], a, b[2], b[3]);
+      }
+    }
 #pragma unroll
-        for (int np = 0; np < 4; ++np) {
-          if (c0 + np * 16 < pad) {
-            uint32_t b[4];
-            ldsm_t(b, B + (kt * 16 + br) * ldb + c0 + np * 16 + bn);
-            mma_bf16(acc[2 * np], a, b[0], b[1]);
-            mma_bf16(acc[2 * np + 1], a, b[2], b[3]);
-          }
+    for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+      for (int q = 0; q < 4; q += 2) {
+        const int i = c0 + nt * 8 + (lane & 3) * 2;
+        float* w = out + (size_t)(o0 + (lane >> 2) + q * 4) * cols + i;
+        if (pairs && i < cols) {
+          float2* w2 = reinterpret_cast<float2*>(w);
+          const float2 old = add ? *w2 : make_float2(0.0f, 0.0f);
+          *w2 = make_float2(old.x + acc[nt][q], old.y + acc[nt][q + 1]);
+        } else {
+          if (i < cols) *w = add ? *w + acc[nt][q] : acc[nt][q];
+          if (i + 1 < cols) w[1] = add ? w[1] + acc[nt][q + 1] : acc[nt][q + 1];
         }
       }
-#pragma unroll
-      for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int o = o0 + (lane >> 2) + (q >> 1) * 8, i = c0 + nt * 8 + (lane & 3) * 2 + (q & 1);
-          if (i < cols) {
-            float* w = out + (size_t)o * cols + i;
-            *w = add ? *w + acc[nt][q] : acc[nt][q];
-          }
-        }
-    }
   }
 }
 
 template <bool TRAIN>
-__global__ void __launch_bounds__((TRAIN ? kTrainWarps : kPredictWarps) * 32, TRAIN ? 1 : 2) k_mlp(const MlpP p) {
-  constexpr int WARPS = TRAIN ? kTrainWarps : kPredictWarps, NT = WARPS * 32;
+__global__ void __launch_bounds__((TRAIN ? kTrainWarps : kPredictWarps) * 32, 1) k_mlp(const MlpP p) {
   extern __shared__ __align__(16) unsigned char sm[];
-  const MlpSmem L = mlp_smem(p.Dp, WARPS, TRAIN);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int NT = TRAIN ? kTrainWarps * 32 : blockDim.x, warps = NT / 32;
+  const int rows = TRAIN ? kTrainRows : warps * 16;  // of the CTA's tiles
+  const MlpSmem L = mlp_smem(p.Dp, rows, TRAIN);
   const int g = lane >> 2, t4 = lane & 3, ld1 = p.Dp + 8;
   bf16* W1 = reinterpret_cast<bf16*>(sm);
   bf16* W2 = reinterpret_cast<bf16*>(sm + L.W2);
-  bf16* Xc = reinterpret_cast<bf16*>(sm + L.X);
-  bf16* X = Xc + warp * 16 * ld1;
   float2* norm = reinterpret_cast<float2*>(sm + L.norm);
   float* b1 = reinterpret_cast<float*>(sm + L.vec);
   float *b2 = b1 + kH, *w30 = b2 + kH, *w31 = w30 + kH;
-  bf16* H1c = reinterpret_cast<bf16*>(sm + L.H1);
-  bf16* H2c = reinterpret_cast<bf16*>(sm + L.H2);
-  bf16* dZ2c = reinterpret_cast<bf16*>(sm + L.dZ2);
-  float* g1 = reinterpret_cast<float*>(sm + L.g1) + warp * 16 * kH;  // GELU'(Z1), by lane; then dZ1
-  bf16* dZ1c = reinterpret_cast<bf16*>(sm + L.g1);
-  uint16_t* list = TRAIN ? reinterpret_cast<uint16_t*>(g1) : reinterpret_cast<uint16_t*>(sm + L.list) + warp * kListed;
-  float* dc = reinterpret_cast<float*>(sm + L.d);  // [rows]: d0, d1, loss
+  bf16* X = reinterpret_cast<bf16*>(sm + L.X);
+  bf16* H1 = reinterpret_cast<bf16*>(sm + L.H1);
 #pragma unroll 4
-  for (int r = warp; r < kH; r += WARPS)
+  for (int r = warp; r < kH; r += warps)
     for (int k = lane; k < p.Dp; k += 32) W1[r * ld1 + k] = k < p.D ? p.wb[r * p.D + k] : __float2bfloat16(0.0f);
-#pragma unroll 8
+#pragma unroll 4
   for (int i = tid; i < kH * kH / 8; i += NT)
     *reinterpret_cast<uint4*>(W2 + (i >> 4) * kLd + (i & 15) * 8) = reinterpret_cast<const uint4*>(p.wb + p.oW2)[i];
   for (int d = tid; d < p.D; d += NT) norm[d] = make_float2(p.norm[d], 1.0f / p.norm[p.D + d]);
@@ -368,84 +414,63 @@ __global__ void __launch_bounds__((TRAIN ? kTrainWarps : kPredictWarps) * 32, TR
     w30[i] = __bfloat162float(p.wb[p.oW3 + i]);
     w31[i] = __bfloat162float(p.wb[p.oW3 + kH + i]);
   }
-  for (int i = lane; i < 16 * (p.Dp - p.D); i += 32) X[(i & 15) * ld1 + p.D + (i >> 4)] = __float2bfloat16(0.0f);
+  for (int i = tid; i < rows * (p.Dp - p.D); i += NT) X[(i % rows) * ld1 + p.D + i / rows] = __float2bfloat16(0.0f);
   __syncthreads();
   const float b30 = p.w[p.ob3], b31 = p.w[p.ob3 + 1];
   const float* nt = p.norm + 2 * p.D;
-  const int64_t tiles = (p.n + 15) / 16;
-  // prediction: a warp's tiles one after the other; training: the CTA's warps stay together
-  bool add = false;
-#pragma unroll 1
-  for (int64_t tile0 = (int64_t)blockIdx.x * WARPS; tile0 < tiles; tile0 += (int64_t)gridDim.x * WARPS) {
-    const int64_t r0 = (tile0 + warp) * 16;
-    const int nr = (int)max((int64_t)0, min((int64_t)16, p.n - r0));
-    if (!TRAIN && nr == 0) break;
-    const uint32_t far = feature_tile<TRAIN>(p, X, ld1, norm, list, nr ? r0 : 0, nr, lane);
-    float acc[16][4] = {};
-#pragma unroll 1
-    for (int k0 = 0; k0 < p.Dp; k0 += 16) {
-      uint32_t a[4];
-      ldsm(a, X + (lane & 15) * ld1 + k0 + (lane >> 4) * 8);
-      rows_times_wt(acc, a, W1, ld1, k0, lane);
-    }
-    // hidden layer 1 as the A fragments of the next product
-    uint32_t h[8][4];
+  // a layer's 32 columns c0 .. c0 + 31 of the warp's 16 rows, as the lane's pairs of columns
+  // c0 + 8 j + 2 t4 in rows g and g + 8: z = acc + bias, h = GELU(z) rounded, slope = GELU'(z)
+  auto layer = [&](const bf16* A, int lda, const bf16* W, int ldw, int ksteps, const float* bias, int c0, bf16* H,
+                   float (&slope)[4][4], float (&o)[4], bool head) {
+    float acc[4][4] = {};
+    product<false>(acc, A, lda, W + c0 * ldw, ldw, ksteps, lane);
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const float2 b = *reinterpret_cast<const float2*>(b1 + j * 8 + t4 * 2);
-      float v[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float z = acc[j][q] + (q & 1 ? b.y : b.x);
-        v[q] = gelu(z);
-        if (TRAIN) g1[(j * 4 + q) * 32 + lane] = gelu_grad(z);
-      }
-      h[j >> 1][(j & 1) * 2] = pack_bf16(v[0], v[1]);
-      h[j >> 1][(j & 1) * 2 + 1] = pack_bf16(v[2], v[3]);
-      if (TRAIN) {
-        uint32_t* row = reinterpret_cast<uint32_t*>(H1c + (warp * 16 + g) * kLd + j * 8 + t4 * 2);
-        row[0] = h[j >> 1][(j & 1) * 2];
-        row[4 * kLd] = h[j >> 1][(j & 1) * 2 + 1];
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 16; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[j][q] = 0.0f;
-#pragma unroll
-    for (int kt = 0; kt < 8; ++kt) rows_times_wt(acc, h[kt], W2, kLd, kt * 16, lane);
-    // hidden layer 2 and the output head: rows g (o[0], o[1]) and g + 8 (o[2], o[3])
-    float o[4] = {};
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int c = j * 8 + t4 * 2;
-      const float2 b = *reinterpret_cast<const float2*>(b2 + c);
-      const float2 u0 = *reinterpret_cast<const float2*>(w30 + c), u1 = *reinterpret_cast<const float2*>(w31 + c);
+    for (int j = 0; j < 4; ++j) {
+      const int c = c0 + j * 8 + t4 * 2;
+      const float2 b = *reinterpret_cast<const float2*>(bias + c);
 #pragma unroll
       for (int q = 0; q < 4; q += 2) {
         const float z0 = acc[j][q] + b.x, z1 = acc[j][q + 1] + b.y;
         const __nv_bfloat162 hh = __floats2bfloat162_rn(gelu(z0), gelu(z1));
-        const float2 f = __bfloat1622float2(hh);
-        o[q] += f.x * u0.x + f.y * u0.y;
-        o[q + 1] += f.x * u1.x + f.y * u1.y;
+        if (TRAIN || !head) *reinterpret_cast<__nv_bfloat162*>(H + (g + q * 4) * kLd + c) = hh;
         if (TRAIN) {
-          *reinterpret_cast<__nv_bfloat162*>(H2c + (warp * 16 + g + q * 4) * kLd + c) = hh;
-          acc[j][q] = gelu_grad(z0);
-          acc[j][q + 1] = gelu_grad(z1);
+          slope[j][q] = gelu_grad(z0);
+          slope[j][q + 1] = gelu_grad(z1);
+        }
+        if (head) {
+          const float2 f = __bfloat1622float2(hh);
+          const float2 u0 = *reinterpret_cast<const float2*>(w30 + c), u1 = *reinterpret_cast<const float2*>(w31 + c);
+          o[q] += f.x * u0.x + f.y * u0.y;
+          o[q + 1] += f.x * u1.x + f.y * u1.y;
         }
       }
     }
+  };
+  if (!TRAIN) {
+    X += warp * 16 * ld1;
+    H1 += warp * 16 * kLd;
+    const int64_t tiles = (p.n + 15) / 16;
+#pragma unroll 1
+    for (int64_t tile = (int64_t)warp * gridDim.x + blockIdx.x; tile < tiles; tile += (int64_t)gridDim.x * warps) {
+      const int64_t r0 = tile * 16;
+      const int nr = (int)min((int64_t)16, p.n - r0);
+      const uint32_t far = feature_tile<false, 16>(p, X, ld1, norm, reinterpret_cast<uint16_t*>(H1), r0, nr, lane);
+      float slope[4][4], o[4] = {};
+#pragma unroll 1
+      for (int c0 = 0; c0 < kH; c0 += 32) layer(X, ld1, W1, ld1, p.Dp / 16, b1, c0, H1, slope, o, false);
+      __syncwarp();
+#pragma unroll 1
+      for (int c0 = 0; c0 < kH; c0 += 32) layer(H1, kLd, W2, kLd, kH / 16, b2, c0, H1, slope, o, true);
+      // rows g (o[0], o[1]) and g + 8 (o[2], o[3])
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      o[q] += __shfl_xor_sync(0xffffffffu, o[q], 1);
-      o[q] += __shfl_xor_sync(0xffffffffu, o[q], 2);
-      o[q] += q & 1 ? b31 : b30;
-    }
-    if (!TRAIN) {
+      for (int q = 0; q < 4; ++q) {
+        o[q] += __shfl_xor_sync(0xffffffffu, o[q], 1);
+        o[q] += __shfl_xor_sync(0xffffffffu, o[q], 2);
+      }
       const int r = g + (t4 & 1) * 8;
       if (t4 < 2 && r < nr) {
-        const float l0 = (t4 ? o[2] : o[0]) * nt[2] + nt[0];
-        const float l1 = (t4 ? o[3] : o[1]) * nt[3] + nt[1];
+        const float l0 = ((t4 ? o[2] : o[0]) + b30) * nt[2] + nt[0];
+        const float l1 = ((t4 ? o[3] : o[1]) + b31) * nt[3] + nt[1];
         const int64_t q = p.row0 + r0 + r;
         if (p.ln_cost) p.ln_cost[q] = l0;
         if (p.ln_h0) p.ln_h0[q] = l1;
@@ -454,91 +479,108 @@ __global__ void __launch_bounds__((TRAIN ? kTrainWarps : kPredictWarps) * 32, TR
           p.h0[q] = far >> r & 1 ? __longlong_as_double(0x7ff8000000000000LL) : fmax(exp((double)l1), 1e-14);
       }
       __syncwarp();
-      continue;
     }
-    // standardised targets: lanes 0 - 15 the cost of row `lane`, lanes 16 - 31 the first step
-    float ts = 0.0f;
-    if ((lane & 15) < nr) {
-      const int64_t q = p.row0 + r0 + (lane & 15);
-      const int64_t src = p.perm ? (int64_t)p.perm[q] : q;
-      const double t = log(lane < 16 ? fmax((double)p.sub[src], 1.0) : fmax(p.hf[src], 1e-300));
-      ts = (float)((t - nt[lane >> 4]) / nt[2 + (lane >> 4)]);
+    return;
+  }
+  bf16* H2 = reinterpret_cast<bf16*>(sm + L.H2);
+  bf16* dZ2 = reinterpret_cast<bf16*>(sm + L.dZ2);
+  bf16* dZ1 = reinterpret_cast<bf16*>(sm + L.dZ1);
+  float* po = reinterpret_cast<float*>(sm + L.head);  // [rows][4 column groups][2] outputs
+  float* ts = po + 8 * kTrainRows;                     // [rows][2] standardised targets
+  float* dc = ts + 2 * kTrainRows;                     // [rows][3] d0, d1, loss
+  const int rt = warp >> 2, c0 = (warp & 3) * 32;      // the warp's 16 rows and 32 columns
+  bool add = false;
+#pragma unroll 1
+  for (int64_t base = (int64_t)blockIdx.x * kTrainRows; base < p.n; base += (int64_t)gridDim.x * kTrainRows) {
+    constexpr int R = kTrainRows / kTrainWarps;  // rows of features per warp
+    {
+      const int64_t r0 = base + warp * R;
+      const int nr = (int)max((int64_t)0, min((int64_t)R, p.n - r0));
+      feature_tile<true, R>(p, X + warp * R * ld1, ld1, norm, reinterpret_cast<uint16_t*>(H1) + warp * kListed,
+                            nr ? r0 : 0, nr, lane);
     }
-    float d[4];
+    if (warp < kTrainRows * 2 / 32) {  // one target a lane: rows' cost, then their first step
+      const int r = tid >> 1, w = tid & 1;
+      float v = 0.0f;
+      if (base + r < p.n) {
+        const int64_t q = p.row0 + base + r;
+        const int64_t src = p.perm ? (int64_t)p.perm[q] : q;
+        const double t = log(w == 0 ? fmax((double)p.sub[src], 1.0) : fmax(p.hf[src], 1e-300));
+        v = (float)((t - nt[w]) / nt[2 + w]);
+      }
+      ts[tid] = v;
+    }
+    __syncthreads();
+    float s1[4][4], s2[4][4], o[4] = {};
+    layer(X + rt * 16 * ld1, ld1, W1, ld1, p.Dp / 16, b1, c0, H1 + rt * 16 * kLd, s1, o, false);
+    __syncthreads();
+    layer(H1 + rt * 16 * kLd, kLd, W2, kLd, kH / 16, b2, c0, H2 + rt * 16 * kLd, s2, o, true);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int r = g + (q >> 1) * 8;
-      const float res = o[q] - __shfl_sync(0xffffffffu, ts, r + (q & 1) * 16);
-      d[q] = r < nr ? res * p.inv_B : 0.0f;
-      o[q] = r < nr ? res : 0.0f;
+      o[q] += __shfl_xor_sync(0xffffffffu, o[q], 1);
+      o[q] += __shfl_xor_sync(0xffffffffu, o[q], 2);
     }
     if (t4 < 2) {
-      float* e = dc + (warp * 16 + g + t4 * 8) * 3;
-      const float d0 = t4 ? d[2] : d[0], d1 = t4 ? d[3] : d[1], e0 = t4 ? o[2] : o[0], e1 = t4 ? o[3] : o[1];
-      e[0] = d0;
-      e[1] = d1;
-      e[2] = 0.5f * (e0 * e0 + e1 * e1) * p.inv_B;
+      float* e = po + (rt * 16 + g + t4 * 8) * 8 + (warp & 3) * 2;
+      e[0] = t4 ? o[2] : o[0];
+      e[1] = t4 ? o[3] : o[1];
+    }
+    __syncthreads();
+    float d[4];
+#pragma unroll
+    for (int q = 0; q < 4; q += 2) {
+      const int r = rt * 16 + g + q * 4;
+      const float4 ea = *reinterpret_cast<const float4*>(po + r * 8), eb = *reinterpret_cast<const float4*>(po + r * 8 + 4);
+      const bool in = base + r < p.n;
+      const float r0 = in ? ea.x + ea.z + eb.x + eb.z + b30 - ts[2 * r] : 0.0f;
+      const float r1 = in ? ea.y + ea.w + eb.y + eb.w + b31 - ts[2 * r + 1] : 0.0f;
+      d[q] = r0 * p.inv_B;
+      d[q + 1] = r1 * p.inv_B;
+      if ((warp & 3) == 0 && t4 == 0) {
+        dc[r * 3] = d[q];
+        dc[r * 3 + 1] = d[q + 1];
+        dc[r * 3 + 2] = 0.5f * (r0 * r0 + r1 * r1) * p.inv_B;
+      }
     }
     // dZ2, and dZ1 = (dZ2 W2) GELU'(Z1)
 #pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      const int c = j * 8 + t4 * 2;
+    for (int j = 0; j < 4; ++j) {
+      const int c = c0 + j * 8 + t4 * 2;
       const float2 u0 = *reinterpret_cast<const float2*>(w30 + c), u1 = *reinterpret_cast<const float2*>(w31 + c);
 #pragma unroll
-      for (int q = 0; q < 4; q += 2) {
-        const uint32_t z = pack_bf16((d[q] * u0.x + d[q + 1] * u1.x) * acc[j][q],
-                                     (d[q] * u0.y + d[q + 1] * u1.y) * acc[j][q + 1]);
-        h[j >> 1][(j & 1) * 2 + q / 2] = z;
-        *reinterpret_cast<uint32_t*>(dZ2c + (warp * 16 + g + q * 4) * kLd + c) = z;
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 16; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[j][q] = 0.0f;
-#pragma unroll
-    for (int kt = 0; kt < 8; ++kt) {
-      const bf16* w = W2 + (kt * 16 + (lane & 15)) * kLd + (lane >> 4) * 8;
-#pragma unroll
-      for (int np = 0; np < 8; ++np) {
-        uint32_t b[4];
-        ldsm_t(b, w + np * 16);
-        mma_bf16(acc[2 * np], h[kt], b[0], b[1]);
-        mma_bf16(acc[2 * np + 1], h[kt], b[2], b[3]);
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < 16; ++j)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[j][q] *= g1[(j * 4 + q) * 32 + lane];
-    __syncwarp();
-    bf16* dZ1 = reinterpret_cast<bf16*>(g1);
-#pragma unroll
-    for (int j = 0; j < 16; ++j)
-#pragma unroll
       for (int q = 0; q < 4; q += 2)
-        *reinterpret_cast<uint32_t*>(dZ1 + (g + q * 4) * kLd + j * 8 + t4 * 2) = pack_bf16(acc[j][q], acc[j][q + 1]);
+        *reinterpret_cast<uint32_t*>(dZ2 + (rt * 16 + g + q * 4) * kLd + c) =
+            pack_bf16((d[q] * u0.x + d[q + 1] * u1.x) * s2[j][q], (d[q] * u0.y + d[q + 1] * u1.y) * s2[j][q + 1]);
+    }
+    __syncthreads();
+    {
+      float acc[4][4] = {};
+      product<true>(acc, dZ2 + rt * 16 * kLd, kLd, W2 + c0, kLd, kH / 16, lane);
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int q = 0; q < 4; q += 2)
+          *reinterpret_cast<uint32_t*>(dZ1 + (rt * 16 + g + q * 4) * kLd + c0 + j * 8 + t4 * 2) =
+              pack_bf16(acc[j][q] * s1[j][q], acc[j][q + 1] * s1[j][q + 1]);
+    }
     __syncthreads();
     // the CTA's contribution to the gradient
     float* part = p.part + blockIdx.x * p.part_stride;
-    const int z1_step = 16 * kH * 2;  // dZ1's 16 rows of a warp lie in its g1 area
-    weight_gradient(dZ2c, 16 * kLd, H1c, kLd, kH, warp, lane, add, part + p.oW2);
-    weight_gradient(dZ1c, z1_step, Xc, ld1, p.D, warp, lane, add, part);
-    float s[4] = {};
+    weight_gradient(dZ2, H1, kLd, kH, warp, lane, add, part + p.oW2);
+    weight_gradient(dZ1, X, ld1, p.D, warp, lane, add, part);
+    {
+      const int c = tid & (kH - 1), what = tid / kH;  // b1, b2, the rows of W3
+      const bf16* z = what == 0 ? dZ1 : what == 1 ? dZ2 : H2;
+      float s = 0.0f;
 #pragma unroll 8
-    for (int r = 0; r < WARPS * 16; ++r) {
-      const float h2 = __bfloat162float(H2c[r * kLd + tid]);
-      s[0] += __bfloat162float(dZ1c[(r >> 4) * z1_step + (r & 15) * kLd + tid]);
-      s[1] += __bfloat162float(dZ2c[r * kLd + tid]);
-      s[2] += dc[r * 3] * h2;
-      s[3] += dc[r * 3 + 1] * h2;
+      for (int r = 0; r < kTrainRows; ++r)
+        s = fmaf(what < 2 ? 1.0f : dc[r * 3 + (what & 1)], __bfloat162float(z[r * kLd + c]), s);
+      float* w = part + (what == 0 ? p.ob1 : what == 1 ? p.ob2 : p.oW3 + (what & 1) * kH) + c;
+      *w = add ? *w + s : s;
     }
-    const int64_t at[4] = {p.ob1 + tid, p.ob2 + tid, p.oW3 + tid, p.oW3 + kH + tid};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) part[at[q]] = add ? part[at[q]] + s[q] : s[q];
     if (tid < 3) {  // b3's gradient and the loss
       float v = 0.0f;
-      for (int r = 0; r < WARPS * 16; ++r) v += dc[r * 3 + tid];
+      for (int r = 0; r < kTrainRows; ++r) v += dc[r * 3 + tid];
       float* w = part + p.ob3 + tid;
       *w = add ? *w + v : v;
     }
@@ -606,7 +648,6 @@ struct chem_mlp_s {
   int64_t adam_t = 0;
   // kept between calls: the CTAs' partial gradients, the gradient and loss on the host
   float* part = nullptr;   // [num_sms][part_stride]
-  float* loss = nullptr;
   float* host = nullptr;   // pinned, [nw + 1]
   int64_t part_stride = 0;
   int num_sms = 0;
@@ -629,7 +670,6 @@ static chem_status mlp_cuda(chem_mlp m, cudaError_t e, const char* what) {
 static chem_status mlp_train_scratch(chem_mlp m) {
   if (m->host) return CHEM_OK;
   if (!m->part) MLP_TRY(m, cudaMalloc(&m->part, m->num_sms * m->part_stride * sizeof(float)));
-  if (!m->loss) MLP_TRY(m, cudaMalloc(&m->loss, sizeof(float)));
   MLP_TRY(m, cudaMallocHost(&m->host, (m->nw + 1) * sizeof(float)));
   return CHEM_OK;
 }
@@ -696,8 +736,7 @@ extern "C" chem_status chem_mlp_create(int32_t n_species, uint64_t seed, chem_ml
 extern "C" chem_status chem_mlp_destroy(chem_mlp m) {
   if (!m) return CHEM_ERR_INVALID_ARG;
   cudaDeviceSynchronize();
-  for (void* p : {(void*)m->w, (void*)m->g, (void*)m->m, (void*)m->v, (void*)m->wb, (void*)m->norm, (void*)m->part,
-                  (void*)m->loss})
+  for (void* p : {(void*)m->w, (void*)m->g, (void*)m->m, (void*)m->v, (void*)m->wb, (void*)m->norm, (void*)m->part})
     if (p) cudaFree(p);
   if (m->host) cudaFreeHost(m->host);
   delete m;
@@ -763,15 +802,14 @@ static MlpP mlp_args(chem_mlp m, int64_t n, const double* T, const double* p, co
   return a;
 }
 
-// gradient (into m->g) and loss (device) of the rows [b0, b0 + rows) of the order `perm`
-static chem_status fwd_bwd(chem_mlp m, MlpP a, cudaStream_t st, float* loss_dev) {
+// gradient and loss of the rows of `a`
+static chem_status fwd_bwd(chem_mlp m, MlpP a, cudaStream_t st, float* grad, float* loss) {
   a.inv_B = 1.0f / (float)a.n;
   a.part = m->part;
   a.part_stride = m->part_stride;
-  const int rows = kTrainWarps * 16;
-  const int grid = (int)std::min<int64_t>((a.n + rows - 1) / rows, m->num_sms);
-  k_mlp<true><<<grid, kTrainWarps * 32, mlp_smem(a.Dp, kTrainWarps, true).total, st>>>(a);
-  k_reduce<<<(int)((m->nw + 128) / 128), dim3(128, 8), 0, st>>>(m->part, grid, m->part_stride, m->nw, m->g, loss_dev);
+  const int grid = (int)std::min<int64_t>((a.n + kTrainRows - 1) / kTrainRows, m->num_sms);
+  k_mlp<true><<<grid, kTrainWarps * 32, mlp_smem(a.Dp, kTrainRows, true).total, st>>>(a);
+  k_reduce<<<(int)((m->nw + 128) / 128), dim3(128, 8), 0, st>>>(m->part, grid, m->part_stride, m->nw, grad, loss);
   return mlp_cuda(m, cudaGetLastError(), "mlp backward");
 }
 
@@ -845,7 +883,7 @@ extern "C" chem_status chem_mlp_train(chem_mlp m, int64_t n, const double* T, co
     for (int bi = 0; bi < nb; ++bi) {
       a.row0 = (int64_t)bi * B;
       a.n = std::min<int64_t>(B, n - a.row0);
-      s = fwd_bwd(m, a, st, loss_d + bi);
+      s = fwd_bwd(m, a, st, m->g, loss_d + bi);
       if (s != CHEM_OK) return s;
       ++m->adam_t;
       float c1, c2;
@@ -877,10 +915,9 @@ extern "C" chem_status chem_mlp_gradient(chem_mlp m, int64_t n, const double* T,
   MlpP a = mlp_args(m, n, T, p, Y);
   a.sub = substeps;
   a.hf = h_first;
-  s = fwd_bwd(m, a, st, m->loss);
+  // the reduction writes the result to the pinned buffer itself
+  s = fwd_bwd(m, a, st, m->host, m->host + m->nw);
   if (s != CHEM_OK) return s;
-  MLP_TRY(m, cudaMemcpyAsync(m->host + m->nw, m->loss, 4, cudaMemcpyDeviceToHost, st));
-  if (grad_host) MLP_TRY(m, cudaMemcpyAsync(m->host, m->g, m->nw * 4, cudaMemcpyDeviceToHost, st));
   MLP_TRY(m, cudaStreamSynchronize(st));
   if (grad_host) std::memcpy(grad_host, m->host, m->nw * 4);
   if (loss_host) *loss_host = m->host[m->nw];
@@ -911,10 +948,13 @@ static chem_status predict_into(chem_mlp m, int64_t n, const double* T, const do
   a.ln_h0 = ln_h0;
   a.cost = cost;
   a.h0 = h0;
-  const size_t smem = mlp_smem(a.Dp, kPredictWarps, false).total;
-  const int64_t ctas = (n + kPredictWarps * 16 - 1) / (kPredictWarps * 16);
-  const int grid = (int)std::min<int64_t>(ctas, (int64_t)m->num_sms * (2 * (smem + 1024) <= 233472 ? 2 : 1));
-  k_mlp<false><<<grid, kPredictWarps * 32, smem, st>>>(a);
+  // a CTA per SM, with no more warps than there are tiles of 16 rows for it or memory
+  const int64_t tiles = (n + 15) / 16;
+  const int grid = (int)std::min<int64_t>(tiles, m->num_sms);
+  int warps = std::max(4, (int)std::min<int64_t>((tiles + grid - 1) / grid, kPredictWarps));
+  while (mlp_smem(a.Dp, warps * 16, false).total > (int)kMaxSmemMlp) --warps;
+  const size_t smem = mlp_smem(a.Dp, warps * 16, false).total;
+  k_mlp<false><<<grid, warps * 32, smem, st>>>(a);
   return mlp_cuda(m, cudaGetLastError(), "chem_mlp_predict");
 }
 
