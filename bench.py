@@ -968,10 +968,9 @@ def main():
     if "phases" in hd:
         line["phase_share"] = hd["phases"]
         line["phase_roofline"] = phase_rooflines(m, hd, n, mlp_ms)
-    # per step: the integration kernel, plus (learned form) per 65,536-cell chunk the
-    # feature, two GEMM and head kernels of the MLP, and 3 counting-sort kernels
-    chunks = (n + 65535) // 65536
-    line["gpu_launches"] = args.steps * (1 + ((4 * chunks + 3) if learned else 0))
+    # per step: the integration kernel, plus (learned form) the model's kernel and 3
+    # counting-sort kernels
+    line["gpu_launches"] = args.steps * (1 + (4 if learned else 0))
     extra = []
     if world == 1 and not args.no_cpu_baseline:
         cb = cpu_baseline(m, st, dt, args.cpu_seconds)
