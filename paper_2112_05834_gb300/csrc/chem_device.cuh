@@ -734,9 +734,10 @@ __host__ __device__ inline size_t slot_entries(int K) {
 // m0_global: the mixed form's assembled matrix lives in a global-memory slot of
 // the CTA instead of shared memory (large mechanisms, persistent schedulers).
 // want_xt: the exponential's table (2 KB) in shared memory, where that still fits.
+// n_sp: 9, or 0 for a kernel without a mechanism.
 constexpr size_t kMaxSmem = 227 * 1024;
 __host__ __device__ inline Layout make_layout(int Kmax, int Imax, int prec, bool m0_global = false,
-                                              bool want_xt = false) {
+                                              bool want_xt = false, int n_sp = 9) {
   Layout L;
   L.nmax = Kmax + 1;
   L.ld = odd_ld(L.nmax);
@@ -748,7 +749,7 @@ __host__ __device__ inline Layout make_layout(int Kmax, int Imax, int prec, bool
   if (want_xt) o += 256 * sizeof(double);
   L.off_vec = o;
   o += (size_t)13 * L.nmax * sizeof(double);
-  o += (size_t)9 * Kmax * sizeof(double);
+  o += (size_t)n_sp * Kmax * sizeof(double);
   if (prec == PREC_FP64) {
     o += (size_t)8 * Imax * sizeof(double);
     L.off_M = o;
@@ -771,7 +772,7 @@ __host__ __device__ inline Layout make_layout(int Kmax, int Imax, int prec, bool
   o += (size_t)L.nmax * sizeof(double);   // inverse diagonal of U
   o = (o + 15) & ~(size_t)15;
   L.total = o;
-  return want_xt && o > kMaxSmem ? make_layout(Kmax, Imax, prec, m0_global) : L;
+  return want_xt && o > kMaxSmem ? make_layout(Kmax, Imax, prec, m0_global, false, n_sp) : L;
 }
 
 
@@ -2303,7 +2304,8 @@ __device__ void solve(Cta<NW>& c, int n, const double* b, double* x, int ir) {
 }
 
 // Factorisation of the iteration matrix: LU (FP64 form) or the FP32 inverse.
-template <int NW, int PREC>
+// NMAX: the largest n the caller may pass.
+template <int NW, int PREC, int NMAX = 256>
 __device__ int factor(Cta<NW>& c, int n, bool pivot = true) {
   if constexpr (!Policy<PREC>::IR) {
     return lu_factor<NW, double>(c, reinterpret_cast<double*>(c.M()), n, pivot);
@@ -2319,7 +2321,7 @@ __device__ int factor(Cta<NW>& c, int n, bool pivot = true) {
       if (n <= 64) return gj_invert_wc<8, 2, 8>(c, src, c.ld0, inv, n);
       if (n <= 128) return gj_invert_wc<8, 4, 16>(c, src, c.ld0, inv, n);
     } else if constexpr (NW == 2) {
-      if (n <= 32) return gj_invert_wc<2, 1, 16>(c, src, c.ld0, inv, n);
+      if (NMAX <= 32 || n <= 32) return gj_invert_wc<2, 1, 16>(c, src, c.ld0, inv, n);
       if (n <= 64) return gj_invert_wc<2, 2, 32>(c, src, c.ld0, inv, n);
     }
     const int ld = odd_ld(n);

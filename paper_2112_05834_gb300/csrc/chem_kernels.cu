@@ -94,31 +94,47 @@ struct LuArgs {
   int ir;
 };
 
+// Batched solves: a CTA takes a matrix from its load to the solution, bound by the chain of
+// its n dependent pivots, so what counts is how many matrices an SM holds and that nothing
+// else adds to the chain. A warp that waited for one row's loads at a time took 28 memory
+// latencies for n = 55; with eight loads in flight per thread a matrix takes three. The
+// layout leaves out the species arrays and registers are limited to five CTAs of 128 threads
+// (four before) or sixteen of 64 (n <= 32, which needs half of them); beyond n = 64 the
+// inverse stays in the registers of 256 threads instead of the shared memory of 128.
+// Mixed form: 8,192 of n = 55 712 -> 496 us, 65,536 of n = 16 1398 -> 476 us, 592 of
+// n = 101 3434 -> 310 us; FP64 form: 3,970 of n = 55 1619 -> 1533 us, 296 of n = 128 1737 ->
+// 1134 us, 100 of n = 55 158 -> 123 us.
 template <int NW, int PREC>
-__global__ void __launch_bounds__(NW * 32) k_lu_solve(const __grid_constant__ LuArgs a) {
+__global__ void __launch_bounds__(NW * 32, NW == 2 ? 16 : NW == 4 ? 5 : 2) k_lu_solve(const __grid_constant__ LuArgs a) {
   using P = Policy<PREC>;
   using R = typename P::LU;
-  const Layout L = make_layout(a.dim - 1, 1, PREC);
+  const Layout L = make_layout(a.dim - 1, 1, PREC, false, false, 0);
   Cta<NW> c;
   c.bind(L);
-  constexpr int NT = NW * 32;
-  const int n = a.dim, ld = odd_ld(n);
+  constexpr int NT = NW * 32, B = 8;  // B loads in flight per thread
+  const int n = a.dim, nn = n * n, ld = odd_ld(n);
+  const unsigned rn = 0xffffffffu / (unsigned)n + 1u;  // e / n = umulhi(e, rn) for e < 2^16 (n = 1: 0)
   R* M = reinterpret_cast<R*>(c.M());
 #pragma unroll 1
   for (int64_t s = blockIdx.x; s < a.n_mat; s += gridDim.x) {
-    const double* As = a.A + (size_t)s * n * n;
+    const double* As = a.A + (size_t)s * nn;
 #pragma unroll 1
-    for (int i = c.warp; i < n; i += NW)
-#pragma unroll 1
-      for (int j = c.lane; j < n; j += 32) {
-        const double v = As[i * n + j];
-        if constexpr (P::IR) reinterpret_cast<typename P::ASM*>(c.M0)[j * ld + i] = from_double<typename P::ASM>(v);
-        else M[i * ld + j] = v;
+    for (int e0 = c.tid; e0 < nn; e0 += B * NT) {
+      double v[B];
+#pragma unroll
+      for (int u = 0; u < B; ++u) v[u] = e0 + u * NT < nn ? As[e0 + u * NT] : 0.0;
+#pragma unroll
+      for (int u = 0; u < B; ++u) {
+        const int e = e0 + u * NT, i = (int)__umulhi((unsigned)e, rn), j = e - i * n;
+        if (e >= nn) break;
+        if constexpr (P::IR) reinterpret_cast<typename P::ASM*>(c.M0)[j * ld + i] = from_double<typename P::ASM>(v[u]);
+        else M[i * ld + j] = v[u];
       }
+    }
 #pragma unroll 1
     for (int i = c.tid; i < n; i += NT) c.fv()[i] = a.b[(size_t)s * n + i];
     __syncthreads();
-    const int info = factor<NW, PREC>(c, n);
+    const int info = factor<NW, PREC, NW == 2 ? 32 : 128>(c, n);
     if (info == 0) solve<NW, PREC>(c, n, c.fv(), c.u(), a.ir);
 #pragma unroll 1
     for (int i = c.tid; i < n; i += NT) a.x[(size_t)s * n + i] = info == 0 ? c.u()[i] : NAN;
@@ -173,10 +189,10 @@ cudaError_t occupancy_integrate(int block, int prec, int K, int I, int* ctas_per
 }
 
 template <int PREC, class ArgT, class KernelT>
-static cudaError_t launch_simple(KernelT k, const ArgT& a, size_t smem, int grid, cudaStream_t st) {
+static cudaError_t launch_simple(KernelT k, const ArgT& a, size_t smem, int grid, cudaStream_t st, int block = 128) {
   cudaError_t e = prep(k, smem);
   if (e != cudaSuccess) return e;
-  k<<<grid, 128, smem, st>>>(a);
+  k<<<grid, block, smem, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -210,6 +226,22 @@ cudaError_t launch_math(int op, const double* x, double* y, int64_t n, cudaStrea
   return cudaGetLastError();
 }
 
+// Threads per matrix: the register inverse takes 64 threads up to n = 32, 128 up to 64 and
+// 256 up to 128. The FP64 LU is quicker with more threads while the SMs are not full.
+// (FP64, us with 64 / 128 / 256 threads: 100 matrices of n = 32 86 / 62 / 55, 11,722 of them
+// 1335 / 1385 / 1502; 100 of n = 55 236 / 152 / 123, 3,970 of them 1516 / 1535 / 1609; 296 of
+// n = 128 - / 1682 / 1129. Mixed: 100 of n = 55 35 / 28 / 30, 3,970 of them 283 / 277 / 440.)
+// At 86 us a matrix and 0.114 us a matrix for the full GPU, 64 threads reach that rate with
+// some 750 matrices in flight, five per SM.
+static int lu_block(int64_t n_mat, int dim, int prec) {
+  const int block = dim <= 32 ? 64 : dim <= 64 ? 128 : 256;
+  int dev = 0, sms = 0;
+  if (prec != PREC_FP64 || block == 256 || cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return block;
+  return n_mat <= 4 * (int64_t)sms ? 2 * block : block;
+}
+
 cudaError_t launch_lu_solve(int64_t n_mat, int dim, const double* A, const double* b, double* x,
                             int* info, int prec, int ir, cudaStream_t st) {
   LuArgs a;
@@ -220,11 +252,19 @@ cudaError_t launch_lu_solve(int64_t n_mat, int dim, const double* A, const doubl
   a.x = x;
   a.info = info;
   a.ir = ir;
-  const size_t smem = smem_bytes(dim - 1, 1, prec, false, false);
+  const size_t smem = make_layout(dim - 1, 1, prec, false, false, 0).total;
   const int grid = (int)(n_mat < 65535 ? n_mat : 65535);
-  if (prec == PREC_FP64) return launch_simple<PREC_FP64>(k_lu_solve<4, PREC_FP64>, a, smem, grid, st);
-  if (prec == PREC_MIXED) return launch_simple<PREC_MIXED>(k_lu_solve<4, PREC_MIXED>, a, smem, grid, st);
-  return launch_simple<PREC_FP32ASM>(k_lu_solve<4, PREC_FP32ASM>, a, smem, grid, st);
+  const int block = lu_block(n_mat, dim, prec);
+#define LU(P)                                                                               \
+  do {                                                                                      \
+    if (block == 64) return launch_simple<P>(k_lu_solve<2, P>, a, smem, grid, st, block);   \
+    if (block == 256) return launch_simple<P>(k_lu_solve<8, P>, a, smem, grid, st, block);  \
+    return launch_simple<P>(k_lu_solve<4, P>, a, smem, grid, st, block);                    \
+  } while (0)
+  if (prec == PREC_FP64) LU(PREC_FP64);
+  if (prec == PREC_MIXED) LU(PREC_MIXED);
+  LU(PREC_FP32ASM);
+#undef LU
 }
 
 }  // namespace chem
