@@ -2687,9 +2687,9 @@ __device__ void integrate_cell(const Job& job, int64_t cell, const IntegrateArgs
 // ---------------------------------------------------------------------------
 // Launch bounds: 128 registers a thread for four CTAs of 128 threads (FP64 form: its
 // shared-memory footprint allows no more up to ~60 species), eight of 64 or two of 256;
-// the mixed form with 128 threads takes 96 registers for five CTAs per SM, which its
-// global-memory matrix slot makes room for (measured on 54 species: 7 % faster than
-// four CTAs; six and seven CTAs spill too much in the register Gauss-Jordan).
+// the mixed form with 128 threads takes 168 registers for three CTAs per SM: it is bound by
+// the latency of its phases, which spills lengthen (16,384 cells of 54 species: 415 ms;
+// four CTAs with 128 registers 487 ms, five with 96 registers 531 ms).
 template <int NW, int PREC, int MTH>
 __global__ void __launch_bounds__(NW * 32, NW == 4 ? (PREC == PREC_MIXED ? 3 : 4) : NW == 2 ? 8 : 2) k_integrate(const __grid_constant__ IntegrateArgs args) {
   __shared__ long long s_work;
