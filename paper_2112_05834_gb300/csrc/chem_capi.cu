@@ -589,7 +589,7 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
   // the efficiencies species-major as well: the rate evaluation's [M] sums read one
   // species for 32 consecutive reactions at a time (coalesced), the assembly one
   // reaction for 32 consecutive species
-  std::vector<double> effT(eff.size() + (size_t)8 * n_tb, 0.0);  // + 8 rows that the batched loads may reach
+  std::vector<double> effT((size_t)eff_rows(K) * n_tb, 0.0);
   for (int r = 0; r < n_tb; ++r)
     for (int k = 0; k < K; ++k) effT[(size_t)k * n_tb + r] = eff[(size_t)r * K + k];
   const std::vector<float> effT_ff = split(effT);

@@ -1119,8 +1119,8 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
     double S;
     if (FF) {
       // eight terms at a time, the next eight efficiencies loaded while these are summed
-      // (the table's padding rows make the loads past the last species harmless)
-      constexpr int B = 8;
+      // (the loads past the last species reach the table's padding, eff_rows)
+      constexpr int B = kEffBatch;
       const ff2* ef = m.effT_ff + r;
       ff_sum acc;
       ff2 e[B];

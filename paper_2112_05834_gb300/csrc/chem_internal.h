@@ -46,6 +46,11 @@ struct MethodTab {
 // Reaction kinds after the host sorts reactions by kind (warp-uniform branches).
 enum RxnKind { RK_ELEM = 0, RK_TB = 1, RK_LIND = 2, RK_TROE = 3 };
 
+// Species whose efficiencies the mixed forms' third-body sums load at a time, one batch ahead
+// of the sum: the sums touch the rows of every started batch and of the one after the last.
+constexpr int kEffBatch = 8;
+constexpr int eff_rows(int K) { return (K + kEffBatch - 1) / kEffBatch * kEffBatch + kEffBatch; }
+
 // Device-resident struct-of-arrays tables of one mechanism. Reactions are stored
 // sorted by kind; species keep the caller's order.
 struct DevMech {
@@ -85,8 +90,9 @@ struct DevMech {
   const double* fo;     // [n_fo][8]: ln(A0/A), b0 - b, Ea0_R - Ea_R, alpha, 1/T***, 1/T*, T**, 0
   const double* eff;    // [n_tb][K] (row r belongs to reaction i_tb0 + r)
   const struct ff2* eff_ff;  // the same efficiencies as float-float pairs (hi, lo)
-  const double* effT;        // [K][n_tb]: the efficiencies species-major
-  const struct ff2* effT_ff;  // the same as float-float pairs
+  // the efficiencies species-major; float-float pairs with eff_rows(K) rows, zero from row K on
+  const double* effT;        // [K][n_tb]
+  const struct ff2* effT_ff;  // [eff_rows(K)][n_tb]
   // Production sums on a CTA of 64, 128 or 256 threads (table v): ps_g[v] adjacent lanes
   // share a species, ps_passes[v] passes cover them all, ps_quads[v] loads per pass. Load r
   // of a pass holds four 16-bit entries of thread t, at (pass ps_quads + r) NT + t: reaction
