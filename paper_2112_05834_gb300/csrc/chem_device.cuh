@@ -1840,7 +1840,9 @@ __device__ int lu_factor(Cta<NW>& c, R* a, int n, bool pivot = true) {
   for (int k = 0; k < n; ++k) {
     int p = pivot ? pivot_reduce<NW>(c, pmax, pidx, n) : k;  // no pivoting: the diagonal
     if (p >= n) p = k;  // a column of NaN: the zero-pivot path below
-    if (c.tid == 0) {
+    // the reciprocal on the thread that also interchanges column k: it reads the pivot
+    // before its own store to that place, which no barrier separates from other threads
+    if (c.tid == (k & (NT - 1))) {
       c.piv()[k] = p;
       const double pv = (double)a[p * ld + k];
       spinv[0] = pv != 0.0 && isfinite(pv) ? 1.0 / pv : 0.0;
