@@ -1943,7 +1943,7 @@ __device__ void lu_solve_warp(const R* a, int n, const double* invd, R* x, int l
 // In-place Gauss-Jordan inverse (FP32) with partial pivoting: row interchange to
 // the largest |a_ik| (lowest row index on ties), the normalised pivot row kept in a
 // copy while every other row is eliminated (the next pivot search is fused into
-// that elimination: two CTA barriers per column); the inverse is completed by the
+// that elimination: three CTA barriers per column); the inverse is completed by the
 // column interchanges in reverse order. Returns 0 or 1 + k for a zero pivot.
 template <int NW>
 __device__ int gj_invert(Cta<NW>& c, float* a, int n) {
@@ -1972,6 +1972,7 @@ __device__ int gj_invert(Cta<NW>& c, float* a, int n) {
     const float pinv = (pv != 0.0f && isfinite(pv)) ? 1.0f / pv : 0.0f;
     if (pinv == 0.0f && info == 0) info = k + 1;
     if (c.tid == 0) c.piv()[k] = p;
+    __syncthreads();  // every thread has read the pivot: the interchange overwrites it
     // interchange rows k and p; the new row k, normalised, goes to the copy
 #pragma unroll 1
     for (int j = c.tid; j < n; j += NT) {
