@@ -2045,7 +2045,15 @@ __device__ int gj_invert(Cta<NW>& c, float* a, int n) {
 // search by the owner alone took 540 of these.) The inverse is written as
 // inv[Pinv[i]][P[j]] = W[i][j] (P = pivot rows in step order). Requires n <= 32 RS
 // and n <= NW CC. src: the matrix by columns, leading dimension ld0. Returns 0 or 1 + k
-// for a zero pivot.
+// for a zero pivot, or kRowRange.
+// A row that waits for its factor is larger or smaller than the normalised row by its pivot,
+// and so are its multipliers. Pivots within 2^80 of each other and of 1 leave FP32 2^48 on
+// either side of that (the integrator's lie between 1 and about 2^60). Beyond, or where no
+// pivot is left, the result is kRowRange and nothing is written: gj_invert, whose pivot rows
+// are normalised, takes the matrix. (Row sizes 40 decades apart gave infinities. 8,192 solves
+// of n = 55 take 520 us without the test of the range, 525 with it, 531 with it on the
+// factors in registers; scaling pivot rows once a step finds the range exceeded takes 563 us.)
+constexpr int kRowRange = -1;
 template <int NW, int RS, int CC, class A>
 __device__ int gj_invert_wc(Cta<NW>& c, const A* src, int ld0, float* inv, int n) {
   const int ld = odd_ld(n);
@@ -2111,7 +2119,10 @@ __device__ int gj_invert_wc(Cta<NW>& c, const A* src, int ld0, float* inv, int n
     const int ps = RS > 1 ? __shfl_sync(FULLMASK, bs, pl) : 0;
     const int p = pl + 32 * ps;  // (a column of NaN: some row in range, zero pivot)
     if (pinv == 0.0f && info == 0) info = k + 1;
-    if (c.tid == 0) c.piv()[k] = p;
+    if (c.tid == 0) {
+      c.piv()[k] = p;
+      reinterpret_cast<unsigned*>(c.invd())[k] = __float_as_uint(fabsf(pinv));
+    }
     float fp[RS];  // multipliers over the pivot: a_ij -= (a_ik / a_pk) a_pj
     bool isp[RS];
 #pragma unroll
@@ -2174,6 +2185,17 @@ __device__ int gj_invert_wc(Cta<NW>& c, const A* src, int ld0, float* inv, int n
     }
   }
   __syncthreads();
+  {
+    // smallest and largest of the pivots' factors and 1 (0: no pivot)
+    unsigned lo = 0x3f800000u, hi = lo;
+#pragma unroll
+    for (int s = 0; s < RS; ++s) {
+      const unsigned e = lane + 32 * s < n ? reinterpret_cast<unsigned*>(c.invd())[lane + 32 * s] : 0x3f800000u;
+      lo = min(lo, e);
+      hi = max(hi, e);
+    }
+    if (__reduce_max_sync(FULLMASK, hi) - __reduce_min_sync(FULLMASK, lo) > 80u << 23) return kRowRange;
+  }
   // inverse permutation of the pivot rows, then the scatter into the true inverse
 #pragma unroll 1
   for (int k = c.tid; k < n; k += NW * 32) c.perm()[c.piv()[k]] = k;
@@ -2316,17 +2338,19 @@ __device__ int factor(Cta<NW>& c, int n, bool pivot = true) {
     using A = typename Policy<PREC>::ASM;
     float* inv = reinterpret_cast<float*>(c.M());
     const A* src = reinterpret_cast<const A*>(c.M0) + c.i0;
+    int info = kRowRange;
     if constexpr (NW == 4) {
-      if (n <= 32) return gj_invert_wc<4, 1, 8>(c, src, c.ld0, inv, n);
-      if (n <= 56) return gj_invert_wc<4, 2, 14>(c, src, c.ld0, inv, n);
-      if (n <= 64) return gj_invert_wc<4, 2, 16>(c, src, c.ld0, inv, n);
+      if (n <= 32) info = gj_invert_wc<4, 1, 8>(c, src, c.ld0, inv, n);
+      else if (n <= 56) info = gj_invert_wc<4, 2, 14>(c, src, c.ld0, inv, n);
+      else if (n <= 64) info = gj_invert_wc<4, 2, 16>(c, src, c.ld0, inv, n);
     } else if constexpr (NW == 8) {
-      if (n <= 64) return gj_invert_wc<8, 2, 8>(c, src, c.ld0, inv, n);
-      if (n <= 128) return gj_invert_wc<8, 4, 16>(c, src, c.ld0, inv, n);
+      if (n <= 64) info = gj_invert_wc<8, 2, 8>(c, src, c.ld0, inv, n);
+      else if (n <= 128) info = gj_invert_wc<8, 4, 16>(c, src, c.ld0, inv, n);
     } else if constexpr (NW == 2) {
-      if (NMAX <= 32 || n <= 32) return gj_invert_wc<2, 1, 16>(c, src, c.ld0, inv, n);
-      if (n <= 64) return gj_invert_wc<2, 2, 32>(c, src, c.ld0, inv, n);
+      if (NMAX <= 32 || n <= 32) info = gj_invert_wc<2, 1, 16>(c, src, c.ld0, inv, n);
+      else if (n <= 64) info = gj_invert_wc<2, 2, 32>(c, src, c.ld0, inv, n);
     }
+    if (info != kRowRange) return info;
     const int ld = odd_ld(n);
 #pragma unroll 1
     for (int j = c.warp; j < n; j += NW)
