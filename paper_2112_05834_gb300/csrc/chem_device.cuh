@@ -164,10 +164,16 @@ __device__ __forceinline__ float to_float(ff2 a) { return a.hi; }
 __device__ __forceinline__ double to_double(float a) { return (double)a; }
 __device__ __forceinline__ double to_double(double a) { return a; }
 __device__ __forceinline__ double to_double(ff2 a) { return ff_value(a); }
+// A pair's hi part is what the FP32 inverse is formed from: a rounded to nearest, where
+// ff_split truncates.
 template <class R>
 __device__ __forceinline__ R from_double(double a) {
-  if constexpr (std::is_same<R, ff2>::value) return ff_split(a);
-  else return (R)a;
+  if constexpr (std::is_same<R, ff2>::value) {
+    const ff2 s = ff_split(a);
+    return fast_two_sum(s.hi, s.lo);
+  } else {
+    return (R)a;
+  }
 }
 
 // ---------------------------------------------------------------------------
