@@ -246,25 +246,70 @@ static double arrhenius_range(double a, double b, double c) {
   return std::fabs(a) + std::fabs(b) * 9.02 + std::fabs(c) / kTmin;
 }
 
-// The lowest temperature from which the fixed-point rate evaluation holds: |G/RT| of
-// every species at most kFxGRT from there to kFxThi. G/RT is scanned on a 0.5 K grid
-// with a threshold 10 below kFxGRT: by d(G/RT)/dT = -(H/RT)/T, |G/RT| changes by at most
-// 0.5 |H/RT| / T between grid points, under 10 while |H/RT| < 20 T (4,000 at 200 K);
-// a mechanism with a larger |H/RT| anywhere in the range does without (1e300).
-static double fixed_point_temperature(const chem_mechanism_desc* d) {
-  const double thr = kFxGRT - 10.0;
-  double Tb = kTmin;
-  for (double T = kFxThi; T >= kTmin; T -= 0.5) {
-    const double lnT = std::log(T), iT = 1.0 / T;
-    for (int k = 0; k < d->n_species; ++k) {
+// The temperatures [*lo, *end) for which the fixed-point rate evaluation holds: the longest run
+// of a 4 K grid over [kTmin, kFxThi] whose points keep G/RT and every exponential's argument
+// inside their bounds (kFxGRT, kFxFalloff, kFxArg) by what they change from a point to the next,
+// d(G/RT)/dT = -(H/RT)/T and d ln k/dT = (b + E/T)/T. *lo = 1e300: nowhere.
+static void fixed_point_range(const chem_mechanism_desc* d, double* lo, double* end) {
+  const int K = d->n_species, I = d->n_reactions;
+  const double step = 4.0;
+  struct Rate {
+    double a, b, E;
+    double at(double lnT, double iT) const { return a + b * lnT - E * iT; }
+    double change(double step, double iT) const { return step * (std::fabs(b) + std::fabs(E) * iT) * iT; }
+  };
+  std::vector<Rate> kf(I), fall(I);
+  for (int i = 0; i < I; ++i) {
+    const bool f = d->rxn_type[i] >= 2;
+    // with the falloff's k0/kinf, ln kf is ln k0
+    fall[i] = f ? Rate{std::log(d->A0[i]) - std::log(d->A[i]), d->b0[i] - d->b[i], d->Ea0_R[i] - d->Ea_R[i]} : Rate{0, 0, 0};
+    kf[i] = f ? Rate{std::log(d->A0[i]), d->b0[i], d->Ea0_R[i]} : Rate{std::log(d->A[i]), d->b[i], d->Ea_R[i]};
+  }
+  std::vector<double> g(K), dg(K);
+  *lo = 1e300;
+  *end = 0.0;
+  double first = -1.0;
+  for (int it = 0;; ++it) {
+    const double T = std::min(kTmin + it * step, kFxThi), lnT = std::log(T), iT = 1.0 / T, lnc = std::log(kRc / kP0 * T);
+    bool ok = true;
+    for (int k = 0; k < K && ok; ++k) {
       const double* a = (T < d->T_mid[k] ? d->nasa_lo : d->nasa_hi) + 7 * k;
       const double h = a[0] + T * (a[1] / 2 + T * (a[2] / 3 + T * (a[3] / 4 + T * (a[4] / 5)))) + a[5] * iT;
       const double sr = a[0] * lnT + T * (a[1] + T * (a[2] / 2 + T * (a[3] / 3 + T * (a[4] / 4)))) + a[6];
-      if (!(std::fabs(h) < 20.0 * T)) return 1e300;
-      if (std::fabs(h - sr) > thr) Tb = std::max(Tb, T + 0.5);
+      g[k] = h - sr;
+      dg[k] = step * std::fabs(h) * iT;
+      ok = std::fabs(g[k]) + dg[k] <= kFxGRT;
     }
+    for (int i = 0; i < I && ok; ++i) {
+      double a = kf[i].at(lnT, iT), da = kf[i].change(step, iT);
+      ok = std::fabs(a) + da <= kFxArg && std::fabs(fall[i].at(lnT, iT)) + fall[i].change(step, iT) <= kFxFalloff;
+      if (!d->reversible[i]) continue;
+      int dnu = 0;
+      for (int s = 0; s < 4; ++s) {
+        const int k = s < 2 ? d->reac_idx[2 * i + s] : d->prod_idx[2 * i + s - 2];
+        if (k < 0) continue;
+        const int nu = s < 2 ? -d->reac_nu[2 * i + s] : d->prod_nu[2 * i + s - 2];
+        dnu += nu;
+        a += nu * g[k];
+        da += std::abs(nu) * dg[k];
+      }
+      a += dnu * lnc;
+      ok = ok && std::fabs(a) + da + step * std::abs(dnu) * iT <= kFxArg;
+    }
+    if (!ok) first = -1.0;
+    else if (first < 0.0) first = T;
+    if (ok && T - first > *end - std::min(*lo, *end)) {
+      *lo = first;
+      *end = T;
+    }
+    if (T >= kFxThi) return;
   }
-  return Tb;
+}
+
+// The temperatures [range[0], range[1]) of a mechanism's fixed-point rate evaluation, without
+// a device (for tests; not part of the interface).
+extern "C" void chem_internal_fixed_point_range(const chem_mechanism_desc* d, double* range) {
+  fixed_point_range(d, range, range + 1);
 }
 
 static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
@@ -626,7 +671,9 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
   m.i_tb0 = i_tb0;
   m.i_fo0 = i_fo0;
   m.i_troe0 = i_troe0;
-  m.T_fx = fx_ok ? fixed_point_temperature(d) : 1e300;
+  m.T_fx = 1e300;
+  m.T_fx_end = 0.0;
+  if (fx_ok) fixed_point_range(d, &m.T_fx, &m.T_fx_end);
   m.gfx = reinterpret_cast<const long long*>(b + oGx);
   m.hcp = reinterpret_cast<const double2*>(b + oHc);
   m.T_mid = reinterpret_cast<const double*>(b + oTm);

@@ -990,7 +990,7 @@ struct Scal {
 // Rate constants come from one exponential each: kf from ln A + b ln T - Theta/T
 // (+ the falloff terms), kr from that argument + dG/RT + dnu ln(Rc T/P0).
 // FX: arguments, logarithms and exponentials in 64-bit fixed point (chem_fixed.cuh),
-// for T in [m.T_fx, kFxThi), where every argument fits; otherwise (FX = false, out of
+// for T in [m.T_fx, m.T_fx_end), where every argument fits; otherwise (FX = false, out of
 // line) the same formulas in FP64. One RHS of the 54-species mechanism issues 196 FP64
 // warp instructions with FX, 546 with FP64 exponentials and species factors
 // exp(+-G/RT) (counted in the source); the FP64 pipe bounded the rate evaluation.
@@ -1033,6 +1033,14 @@ template <int NW, bool JAC, bool FF, bool FX>
 __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double p, double* f) {
   constexpr int NT = NW * 32;
   using Arg = typename std::conditional<FX, long long, double>::type;
+  auto sum = [](Arg a, Arg b) -> Arg {
+    if constexpr (FX) return fx_add(a, b);
+    else return a + b;
+  };
+  auto difference = [](Arg a, Arg b) -> Arg {
+    if constexpr (FX) return fx_sub(a, b);
+    else return a - b;
+  };
   const int K = m.K;
   Scal s;
   s.T = y[0];
@@ -1194,7 +1202,7 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
       dnu = a23.y;
       if (!FX) ka = (Arg)(a01.x + a01.y * lgT - a23.x * invT);
     }
-    if constexpr (FX) ka = fx_clamp(rec.lnA + fx_mul(rec.b, LT) - fx_mul(rec.th, IT), 1100);
+    if constexpr (FX) ka = rec.lnA + fx_mul(rec.b, LT) - fx_mul(rec.th, IT);
     const bool two_f = sl.y != 255, two_r = sl.w != 255;
     const double Ca = c.C()[sl.x];
     const double Cb = two_f ? c.C()[sl.y] : 1.0;
@@ -1215,14 +1223,14 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
       Arg fa;
       if constexpr (FX) {
         const long long* x = m.fox + 4 * (i - m.i_fo0);
-        fa = fx_clamp(x[0] + fx_mul(x[1], LT) - fx_mul(x[2], IT), 900);
+        fa = x[0] + fx_mul(x[1], LT) - fx_mul(x[2], IT);
       } else {
         fa = fo[0] + fo[1] * lgT - fo[2] * invT;
       }
       const double Pr = rate_exp<FX>(fa, c.xt()) * Mc;
       red1 = xrcp(1.0 + Pr);
       double dlgF_dL = 0.0, dlnF_dT = 0.0;
-      ka = ka + fa;
+      ka = sum(ka, fa);
       if (i >= m.i_troe0) {
         const double alpha = fo[3];
         // fo[4] = 1/T***, fo[5] = 1/T*
@@ -1271,7 +1279,7 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
           lnF = lF * (den2 * xrcp(fma(x, x, den2)));
         }
         if constexpr (FX) {
-          ka = fx_clamp(ka, 1100) + fx_clamp(fx_from_double(lnF), 900);
+          ka = fx_add(ka, fx_from_double(lnF));
           if ((__double2hiint(lnF) & 0x7ff00000) == 0x7ff00000) red1 = lnF;  // NaN: no valid [M] or Fc
         } else {
           ka += lnF;
@@ -1286,12 +1294,11 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
     const double kfP = rate_exp<FX>(ka, c.xt());
     double krP = 0.0;
     if (rv & 1) {
-      Arg dg = g_RT[sl.z] - g_RT[sl.x];
-      if (two_r) dg += g_RT[sl.w];
-      if (two_f) dg -= g_RT[sl.y];
-      dg += (rv >> 1) == 2 ? lc : (rv >> 1) == 0 ? -lc : Arg(0);
-      if constexpr (FX) krP = fx_exp(fx_clamp(ka, 1100) + fx_clamp(dg, 900), c.xt());
-      else krP = xexp(ka + dg);
+      Arg dg = difference(g_RT[sl.z], g_RT[sl.x]);
+      if (two_r) dg = sum(dg, g_RT[sl.w]);
+      if (two_f) dg = difference(dg, g_RT[sl.y]);
+      dg = sum(dg, (rv >> 1) == 2 ? lc : (rv >> 1) == 0 ? -lc : Arg(0));
+      krP = rate_exp<FX>(sum(ka, dg), c.xt());
     }
     const double Pf = Ca * Cb, Pb = Cc * Cd;
     if constexpr (!JAC) {
@@ -1437,7 +1444,7 @@ __device__ __noinline__ Scal eval_rhs_fp64(const DevMech& m, Cta<NW> c, const do
 // RHS (and with JAC the Jacobian data) of the state y; T = y[0] selects the path.
 template <int NW, bool JAC, bool FF = false>
 __device__ __forceinline__ Scal eval_rhs(const DevMech& m, Cta<NW>& c, const double* y, double p, double* f) {
-  if (!(y[0] >= m.T_fx && y[0] < kFxThi)) return eval_rhs_fp64<NW, JAC, FF>(m, c, y, p, f);
+  if (!(y[0] >= m.T_fx && y[0] < m.T_fx_end)) return eval_rhs_fp64<NW, JAC, FF>(m, c, y, p, f);
   return eval_rhs_t<NW, JAC, FF, true>(m, c, y, p, f);
 }
 

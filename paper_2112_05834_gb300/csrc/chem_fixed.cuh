@@ -225,10 +225,12 @@ __device__ __forceinline__ long long fx_mul(long long a, unsigned long long b) {
   return (long long)(__umul64hi((unsigned long long)a, b) - ((unsigned long long)(a >> 63) & b));
 }
 
-// v limited to about +-lim (its integer part is clamped), Q52.
-__device__ __forceinline__ long long fx_clamp(long long v, int lim) {
-  const int hi = min(max((int)(v >> 32), -(lim << 20)), lim << 20);
-  return ((long long)hi << 32) | (unsigned)v;
+// a + b and a - b modulo the format: partial sums may leave it when the whole sum does not.
+__device__ __forceinline__ long long fx_add(long long a, long long b) {
+  return (long long)((unsigned long long)a + (unsigned long long)b);
+}
+__device__ __forceinline__ long long fx_sub(long long a, long long b) {
+  return (long long)((unsigned long long)a - (unsigned long long)b);
 }
 
 // A positive double's significand (2^52 .. 2^53) shifted left by its exponent plus sh,
@@ -238,7 +240,8 @@ __device__ __forceinline__ unsigned long long fx_scale(double x, int sh) {
   return ((b & 0xfffffffffffffull) | 0x10000000000000ull) << (((int)(b >> 52) - 1023 + sh) & 63);
 }
 
-// exp(x) of x in Q52, as a double; x beyond +-700 is taken as +-700.
+// exp(x) of x in Q52, as a double; results outside the normal numbers are taken as about
+// the smallest or the largest of them.
 // x = N ln2/256 + r with |r| <= ln2/512 (1 + 2^-8), exp(x) = 2^(N/256) (1 + r + r^2/2 +
 // r^3/6 + r^4/24 + r^5/120); r and the bracket in Q62, r^2 from the two halves of r, the
 // cubic tail (below 2^-31) from 32-bit factors. Error before the final rounding below
@@ -248,7 +251,8 @@ __device__ __forceinline__ double fx_exp(long long x, const unsigned long long* 
   constexpr int kInvL = 1549082005;                           // 256/ln2, Q22
   constexpr unsigned long long kL = 0x2c5c85fdf473deull;      // ln2/256, Q62, rounded down
   constexpr unsigned kLlo = 1794275565u;                      // the rest, Q94
-  x = fx_clamp(x, 700);
+  constexpr int kLo = -742798459, kHi = 744254700;  // -708.388, 709.777 in Q20
+  x = (long long)min(max((int)(x >> 32), kLo), kHi) << 32 | (unsigned)x;
   const int N = ((int)(((long long)(int)(x >> 32) * kInvL) >> 32) + 512) >> 10;
   const long long r = (long long)(((unsigned long long)x << 10) - (unsigned long long)(long long)N * kL) -
                       (((long long)N * (long long)kLlo) >> 32);

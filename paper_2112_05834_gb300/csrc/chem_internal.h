@@ -13,11 +13,15 @@ constexpr int kMaxJobs = 8;
 constexpr double kRc = 8.31446261815324e7;  // erg / (mol K)
 constexpr double kP0 = 1.01325e6;           // dyn / cm^2, standard state (1 atm)
 constexpr double kTmin = 200.0, kTmax = 6000.0;
-// Range of the fixed-point rate evaluation (chem_fixed.cuh): T in [kTmin, kFxThi), and
-// |G/RT| of every species at most kFxGRT there, so that the sum of a reaction's four
-// stays inside the format's +-2048.
+// Range of the fixed-point rate evaluation (chem_fixed.cuh): temperatures inside [kTmin, kFxThi)
+// where G/RT of every species stays inside the format's +-2048, and so does the argument of
+// every exponential as a whole: ln k0/kinf up to +-kFxFalloff, ln kf (with the falloff's
+// k0/kinf) and ln kr up to +-kFxArg, which leaves ln F (at most |ln Fcent|, 745) its room.
+// Partial sums may leave the format (fx_add).
 constexpr double kFxThi = 8192.0;
-constexpr double kFxGRT = 400.0;
+constexpr double kFxGRT = 1900.0;
+constexpr double kFxFalloff = 700.0;
+constexpr double kFxArg = 1000.0;
 
 // FP64: everything in FP64.
 // MIXED: Jacobian assembled in float-float arithmetic (about 48 bits, FP32 pipe; kept
@@ -65,7 +69,7 @@ struct DevMech {
   int i_tb0;  // first reaction of kind >= 1 (sorted order)
   int i_fo0;  // first reaction of kind >= 2
   int i_troe0;  // first reaction of kind 3
-  double T_fx;    // the fixed-point rate evaluation holds for T in [T_fx, kFxThi) (1e300: nowhere)
+  double T_fx, T_fx_end;  // the fixed-point rate evaluation holds for T in [T_fx, T_fx_end)
   const long long* gfx;  // [K][16]: G/RT coefficients for range r at 8 r: constant (Q52), of ln T
                          //   (Q58), of 1/T (Q45), of t, t^2, t^3, t^4 (Q52), t = T/2048 (r = 0)
                          //   or T/8192 (r = 1)
