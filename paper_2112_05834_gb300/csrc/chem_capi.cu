@@ -241,11 +241,6 @@ static long long fixed_log(double A, bool* ok) {
   return to_fixed(l, 52, ok) + to_fixed(A / std::exp(l) - 1.0, 52, ok);
 }
 
-// Largest |a + b ln T - c/T| over [kTmin, kFxThi), from above.
-static double arrhenius_range(double a, double b, double c) {
-  return std::fabs(a) + std::fabs(b) * 9.02 + std::fabs(c) / kTmin;
-}
-
 // The temperatures [*lo, *end) for which the fixed-point rate evaluation holds: the longest run
 // of a 4 K grid over [kTmin, kFxThi] whose points keep G/RT and every exponential's argument
 // inside their bounds (kFxGRT, kFxFalloff, kFxArg) by what they change from a point to the next,
@@ -306,10 +301,63 @@ static void fixed_point_range(const chem_mechanism_desc* d, double* lo, double* 
   }
 }
 
+// The fixed-point tables of the rate evaluation (DevMech::gfx, rx, fox) for reactions in the
+// order `rxns` (-1: null) of kinds `kind`; false where a number does not fit its format.
+// Whole arguments are fixed_point_range's matter: their partial sums may leave the format.
+// Formats: a1 and b within +-128 (large alkanes' a1 pass 38 at 12 carbons), a6 and E/R within
+// 262,144 K, a polynomial's scaled coefficients 2,000 in sum. Below T_mid it is one of
+// t = T 2^(fx_low - 12), the smallest range that holds every species' T_mid.
+static bool fixed_point_tables(const chem_mechanism_desc* d, const std::vector<int>& rxns, const std::vector<int>& kind,
+                               std::vector<long long>& gfx, std::vector<long long>& rx, std::vector<long long>& fox,
+                               int* fx_low) {
+  const int K = d->n_species;
+  const double mid = K ? *std::max_element(d->T_mid, d->T_mid + K) : 0.0;
+  *fx_low = mid <= 2048.0 ? 1 : mid <= 4096.0 ? 0 : -1;
+  bool ok = true;
+  for (int k = 0; k < K; ++k)
+    for (int r = 0; r < 2; ++r) {
+      const double* a = (r == 0 ? d->nasa_lo : d->nasa_hi) + 7 * k;
+      long long* o = &gfx[16 * k + 8 * r];
+      const double S = r == 0 ? std::ldexp(1.0, 12 - *fx_low) : 8192.0;
+      // G/RT = (a1 - a7) - a1 ln T + a6/T - a2/2 T - a3/6 T^2 - a4/12 T^3 - a5/20 T^4
+      const double c[4] = {-a[1] / 2.0 * S, -a[2] / 6.0 * S * S, -a[3] / 12.0 * S * S * S, -a[4] / 20.0 * S * S * S * S};
+      if (!(std::fabs(c[0]) + std::fabs(c[1]) + std::fabs(c[2]) + std::fabs(c[3]) < 2000.0)) ok = false;
+      if (!(std::fabs(a[0]) + std::fabs(a[6]) < 2000.0)) ok = false;
+      o[0] = to_fixed(a[0], 52, &ok) - to_fixed(a[6], 52, &ok) + 2;  // + 2: the mean of the products' truncations
+      o[1] = to_fixed(-a[0], 56, &ok);
+      o[2] = to_fixed(a[5], 45, &ok);
+      for (int j = 0; j < 4; ++j) o[3 + j] = to_fixed(c[j], 52, &ok);
+    }
+  auto arrhenius = [&](long long lnA, double b, double E, long long* o) {
+    o[0] = lnA;
+    o[1] = to_fixed(b, 56, &ok);
+    o[2] = to_fixed(E, 45, &ok);
+  };
+  for (size_t i = 0, f = 0; i < rxns.size(); ++i) {
+    const int o = rxns[i];
+    const bool falloff = kind[i] >= 2;
+    if (o >= 0) {
+      const long long lnA = fixed_log(d->A[o], &ok);
+      arrhenius(lnA, d->b[o], d->Ea_R[o], &rx[4 * i]);
+      if (falloff)
+        arrhenius(fixed_log(d->A0[o], &ok) - lnA, d->b0[o] - d->b[o], d->Ea0_R[o] - d->Ea_R[o], &fox[4 * f]);
+    }
+    if (falloff) ++f;
+  }
+  return ok;
+}
+
 // The temperatures [range[0], range[1]) of a mechanism's fixed-point rate evaluation, without
 // a device (for tests; not part of the interface).
 extern "C" void chem_internal_fixed_point_range(const chem_mechanism_desc* d, double* range) {
-  fixed_point_range(d, range, range + 1);
+  std::vector<int> rxns(d->n_reactions);
+  std::iota(rxns.begin(), rxns.end(), 0);
+  const std::vector<int> kind(d->rxn_type, d->rxn_type + d->n_reactions);
+  std::vector<long long> gfx((size_t)16 * d->n_species), rx((size_t)4 * d->n_reactions), fox(rx);
+  int fx_low;
+  range[0] = 1e300;
+  range[1] = 0.0;
+  if (fixed_point_tables(d, rxns, kind, gfx, rx, fox, &fx_low)) fixed_point_range(d, range, range + 1);
 }
 
 static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
@@ -493,44 +541,10 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
     for (int k = 0; k < K; ++k) ptr[k + 1] = ptr[k] + (int)v[k].size();
     for (int k = 0; k < K; ++k) ent.insert(ent.end(), v[k].begin(), v[k].end());
   };
-  // fixed-point copies for the rate evaluation; every argument has to stay inside +-2000
-  bool fx_ok = true;
+  // fixed-point copies for the rate evaluation
   std::vector<long long> gfx((size_t)16 * K, 0), fox(fo.size() / 2, 0);
-  for (int k = 0; k < K; ++k) {
-    if (!(d->T_mid[k] <= 2048.0)) fx_ok = false;  // t = T/2048 below T_mid
-    for (int r = 0; r < 2; ++r) {
-      const double* a = (r == 0 ? d->nasa_lo : d->nasa_hi) + 7 * k;
-      long long* o = &gfx[16 * k + 8 * r];
-      const double S = r == 0 ? 2048.0 : 8192.0;
-      // G/RT = (a1 - a7) - a1 ln T + a6/T - a2/2 T - a3/6 T^2 - a4/12 T^3 - a5/20 T^4
-      const double c[4] = {-a[1] / 2.0 * S, -a[2] / 6.0 * S * S, -a[3] / 12.0 * S * S * S, -a[4] / 20.0 * S * S * S * S};
-      const double c0 = a[0] - a[6];
-      if (!(arrhenius_range(c0, a[0], a[5]) + std::fabs(c[0]) + std::fabs(c[1]) + std::fabs(c[2]) + std::fabs(c[3]) <
-            2000.0))
-        fx_ok = false;
-      o[0] = to_fixed(a[0], 52, &fx_ok) - to_fixed(a[6], 52, &fx_ok) + 2;  // + 2: the mean of the products' truncations
-      o[1] = to_fixed(-a[0], 58, &fx_ok);
-      o[2] = to_fixed(a[5], 45, &fx_ok);
-      for (int j = 0; j < 4; ++j) o[3 + j] = to_fixed(c[j], 52, &fx_ok);
-    }
-  }
-  auto fix_arrhenius = [&](long long lnA, double b, double E, long long* o) {
-    if (!(arrhenius_range(std::ldexp((double)lnA, -52), b, E) < 2000.0)) fx_ok = false;
-    o[0] = lnA;
-    o[1] = to_fixed(b, 58, &fx_ok);
-    o[2] = to_fixed(E, 45, &fx_ok);
-  };
-  for (int i = 0, f = 0; i < Ip; ++i) {
-    const int o = padded[i];
-    const bool falloff = pkind[i] >= 2;
-    if (o >= 0) {
-      const long long lnA = fixed_log(d->A[o], &fx_ok);
-      fix_arrhenius(lnA, d->b[o], d->Ea_R[o], &rx[4 * i]);
-      if (falloff)
-        fix_arrhenius(fixed_log(d->A0[o], &fx_ok) - lnA, d->b0[o] - d->b[o], d->Ea0_R[o] - d->Ea_R[o], &fox[4 * f]);
-    }
-    if (falloff) ++f;
-  }
+  int fx_low = 1;
+  const bool fx_ok = fixed_point_tables(d, padded, pkind, gfx, rx, fox, &fx_low);
   std::vector<int> tr_ptr;
   std::vector<int2> tr_ent;
   flatten2(tr, tr_ptr, tr_ent);
@@ -674,6 +688,7 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
   m.T_fx = 1e300;
   m.T_fx_end = 0.0;
   if (fx_ok) fixed_point_range(d, &m.T_fx, &m.T_fx_end);
+  m.fx_low = fx_low;
   m.gfx = reinterpret_cast<const long long*>(b + oGx);
   m.hcp = reinterpret_cast<const double2*>(b + oHc);
   m.T_mid = reinterpret_cast<const double*>(b + oTm);

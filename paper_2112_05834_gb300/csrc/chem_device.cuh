@@ -1013,7 +1013,7 @@ __device__ __forceinline__ double rate_log(double x) {
   }
 }
 
-// One reaction's record: Arrhenius parameters in fixed point (Q52, Q58, Q45), species
+// One reaction's record: Arrhenius parameters in fixed point (Q52, Q56, Q45), species
 // slots (reactants, products; 255 = empty), rev (DevMech::rx).
 struct RxRec {
   long long lnA, b, th;
@@ -1092,10 +1092,10 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
   const double lgT = c.red()[SC_LOGT];
   s.invT = c.red()[SC_INVT];
   const double T = s.T, invT = s.invT;
-  // ln T (Q58), 1/T (Q71) and ln(Rc T/P0) (Q52), or their FP64 forms
-  const unsigned long long LT = (unsigned long long)__double_as_longlong(lgT);
+  // ln T (Q60), 1/T (Q71) and ln(Rc T/P0) (Q52), or their FP64 forms
+  const unsigned long long LT = (unsigned long long)__double_as_longlong(lgT) << 2;
   const unsigned long long IT = fx_scale(invT, 19);
-  const Arg lc = FX ? (Arg)((long long)(LT >> 6) + kLnRcP0_Q52) : (Arg)(lgT + kLnRcP0);
+  const Arg lc = FX ? (Arg)((long long)(LT >> 8) + kLnRcP0_Q52) : (Arg)(lgT + kLnRcP0);
   Arg* const g_RT = reinterpret_cast<Arg*>(c.g());
   // species: thermo, G/RT, concentrations
   if (c.warp < nsw) s.rho = c.red()[SC_OUT + 1];
@@ -1110,12 +1110,12 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
     c.cpR()[k] = cp;
     c.hRT()[k] = h;
     if constexpr (FX) {
-      // T / 2048 below T_mid, T / 8192 above (Q64)
-      const unsigned long long t = fx_scale(T, low ? 1 : -1);
+      // T 2^(fx_low - 12) below T_mid, T / 8192 above (Q64)
+      const unsigned long long t = fx_scale(T, low ? m.fx_low : -1);
       const longlong2* q = reinterpret_cast<const longlong2*>(m.gfx + 16 * k + (low ? 0 : 8));
       const longlong2 q0 = q[0], q1 = q[1], q2 = q[2], q3 = q[3];
       const long long poly = fx_mul(q1.y + fx_mul(q2.x + fx_mul(q2.y + fx_mul(q3.x, t), t), t), t);
-      g_RT[k] = q0.x + fx_mul(q0.y, LT) + fx_mul(q1.x, IT) + poly;
+      g_RT[k] = fx_add(fx_add(q0.x, fx_mul(q0.y, LT)), fx_add(fx_mul(q1.x, IT), poly));
     } else {
       const double* b = m.nasa + 36 * k + (low ? 0 : 17);
       const double sr = b[11] * lgT + T * (b[12] + T * (b[13] + T * (b[14] + T * b[15]))) + b[16];
@@ -1202,7 +1202,7 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
       dnu = a23.y;
       if (!FX) ka = (Arg)(a01.x + a01.y * lgT - a23.x * invT);
     }
-    if constexpr (FX) ka = rec.lnA + fx_mul(rec.b, LT) - fx_mul(rec.th, IT);
+    if constexpr (FX) ka = fx_sub(fx_add(rec.lnA, fx_mul(rec.b, LT)), fx_mul(rec.th, IT));
     const bool two_f = sl.y != 255, two_r = sl.w != 255;
     const double Ca = c.C()[sl.x];
     const double Cb = two_f ? c.C()[sl.y] : 1.0;
@@ -1223,7 +1223,7 @@ __device__ Scal eval_rhs_t(const DevMech& m, Cta<NW>& c, const double* y, double
       Arg fa;
       if constexpr (FX) {
         const long long* x = m.fox + 4 * (i - m.i_fo0);
-        fa = x[0] + fx_mul(x[1], LT) - fx_mul(x[2], IT);
+        fa = fx_sub(fx_add(x[0], fx_mul(x[1], LT)), fx_mul(x[2], IT));
       } else {
         fa = fo[0] + fo[1] * lgT - fo[2] * invT;
       }

@@ -71,8 +71,9 @@ struct DevMech {
   int i_troe0;  // first reaction of kind 3
   double T_fx, T_fx_end;  // the fixed-point rate evaluation holds for T in [T_fx, T_fx_end)
   const long long* gfx;  // [K][16]: G/RT coefficients for range r at 8 r: constant (Q52), of ln T
-                         //   (Q58), of 1/T (Q45), of t, t^2, t^3, t^4 (Q52), t = T/2048 (r = 0)
-                         //   or T/8192 (r = 1)
+                         //   (Q56), of 1/T (Q45), of t, t^2, t^3, t^4 (Q52), t = T 2^(fx_low - 12)
+                         //   (r = 0) or T/8192 (r = 1)
+  int fx_low;            // 1, 0 or -1: every T_mid up to 2048, 4096 or beyond
   const long long* fox;  // [n_fo][4]: the first three of fo in the formats of rx
   const double* W;      // [K]
   const double* invW;   // [K]
@@ -86,10 +87,10 @@ struct DevMech {
                         //   a4/4, a5/5, a6, S/R coefficients a1, a2, a3/2, a4/3, a5/4, a7;
                         //   [34] = T_mid
   const double* arr;    // [I][4]: ln A, b, Ea_R, dnu
-  // [I] records of 32 bytes: fixed-point ln A (Q52), b (Q58), Ea_R (Q45), then four
+  // [I] records of 32 bytes: fixed-point ln A (Q52), b (Q56), Ea_R (Q45), then four
   // bytes of species slots (reactants 0/1, products 0/1; 255 empty; a coefficient of 2
   // appears as two equal slots) and rev: bit 0 reversible, bits 1-2 dnu + 1 (dnu = -1, 0, 1).
-  // ln T enters as Q58, 1/T as Q71 (a value v in Qn: round(v 2^n)).
+  // ln T enters as Q60, 1/T as Q71 (a value v in Qn: round(v 2^n)).
   const longlong2* rx;
   const double* fo;     // [n_fo][8]: ln(A0/A), b0 - b, Ea0_R - Ea_R, alpha, 1/T***, 1/T*, T**, 0
   const double* eff;    // [n_tb][K] (row r belongs to reaction i_tb0 + r)

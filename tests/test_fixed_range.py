@@ -1,4 +1,5 @@
 """The temperatures for which rates are evaluated in fixed point: every argument fits there."""
+import copy
 import ctypes as C
 import math
 
@@ -6,6 +7,7 @@ import numpy as np
 import pytest
 
 import mechs
+from fuels import fuel_like
 from paper_2112_05834_gb300 import synth
 
 
@@ -66,3 +68,19 @@ def test_a_mechanism_beyond_every_bound_has_no_range(fixed_range):
     m.nasa_lo[1, 6] = m.nasa_hi[1, 6] = 5000.0
     lo, end = fixed_range(m)
     assert not lo < end
+
+
+@pytest.mark.parametrize("a1,T_mid", [(38.5, 1000.0), (60.0, 1000.0), (100.0, 1391.0), (20.0, 2500.0), (5.0, 5000.0)])
+def test_large_fuel_molecules_have_a_range(fixed_range, a1, T_mid):
+    m = copy.deepcopy(synth.mechanism_preset("c_54"))
+    for k in (40, 47):
+        fuel_like(m, k, a1, T_mid)
+    lo, end = fixed_range(m)
+    assert lo == 200.0 and end >= 6000.0
+
+
+@pytest.mark.parametrize("b", [-40.0, 40.0])
+def test_large_temperature_exponents_have_a_range(fixed_range, b):
+    m, _, _ = _one_reaction(1000.0, math.exp(-b * 7.0), 5000.0)
+    m.b[0] = b
+    assert fixed_range(m) == (200.0, 8192.0)
