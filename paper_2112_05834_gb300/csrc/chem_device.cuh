@@ -741,7 +741,7 @@ __host__ __device__ inline size_t slot_entries(int K) {
 // the CTA instead of shared memory (large mechanisms, persistent schedulers).
 // want_xt: the exponential's table (2 KB) in shared memory, where that still fits.
 // n_sp: 9, or 0 for a kernel without a mechanism.
-constexpr size_t kMaxSmem = 227 * 1024;
+constexpr size_t kMaxSmem = 227 * 1024 - 16;  // k_integrate has 16 bytes of static shared memory
 __host__ __device__ inline Layout make_layout(int Kmax, int Imax, int prec, bool m0_global = false,
                                               bool want_xt = false, int n_sp = 9) {
   Layout L;
