@@ -229,8 +229,12 @@ chem_status chem_integrate_jobs(const chem_job* jobs, int32_t n_jobs, double dt,
  *                 not trusted outside the states it was trained on; default 10);
  *                 0 = off
  *   "max_steps"   step budget per cell (default 100000)
- *   "block"       threads per cell: 64, 128 or 256; 0 (default) = the size with
- *                 the most resident warps per SM for the mechanism and precision
+ *   "block"       threads per cell: 64, 128 or 256; 0 (default) = by the call's
+ *                 largest mechanism, 64 up to 31 species, 128 up to 63, 256 beyond,
+ *                 and twice as many (at most 256) when the call has at most one
+ *                 cell per SM. The order of a cell's sums follows the threads, so
+ *                 that a cell's result is the same bit for bit in batches of
+ *                 different sizes only with an explicit size
  *   "ctas_per_sm" resident CTAs per SM for persistent schedulers (0 = maximum)
  *   "graph"       1 = capture the launch sequence in a CUDA graph and replay it
  *                 while arguments repeat
