@@ -224,6 +224,12 @@ struct Pool {
 
 }  // namespace
 
+static int upper_word(double v) {
+  int64_t b;
+  std::memcpy(&b, &v, sizeof b);
+  return (int)(b >> 32);
+}
+
 // v 2^q rounded to an integer; *ok is cleared when it does not stay inside the format.
 static long long to_fixed(double v, int q, bool* ok) {
   const double s = std::ldexp(v, q);
@@ -685,9 +691,9 @@ static chem_status build_tables(chem_handle h, const chem_mechanism_desc* d) {
   m.i_tb0 = i_tb0;
   m.i_fo0 = i_fo0;
   m.i_troe0 = i_troe0;
-  m.T_fx = 1e300;
-  m.T_fx_end = 0.0;
-  if (fx_ok) fixed_point_range(d, &m.T_fx, &m.T_fx_end);
+  double T_fx = 1e300, T_fx_end = 0.0;  // (or multiples of 4 K)
+  if (fx_ok) fixed_point_range(d, &T_fx, &T_fx_end);
+  m.T_fx = make_int2(upper_word(T_fx), upper_word(T_fx_end));
   m.fx_low = fx_low;
   m.gfx = reinterpret_cast<const long long*>(b + oGx);
   m.hcp = reinterpret_cast<const double2*>(b + oHc);

@@ -990,7 +990,7 @@ struct Scal {
 // Rate constants come from one exponential each: kf from ln A + b ln T - Theta/T
 // (+ the falloff terms), kr from that argument + dG/RT + dnu ln(Rc T/P0).
 // FX: arguments, logarithms and exponentials in 64-bit fixed point (chem_fixed.cuh),
-// for T in [m.T_fx, m.T_fx_end), where every argument fits; otherwise (FX = false, out of
+// for T in the range m.T_fx, where every argument fits; otherwise (FX = false, out of
 // line) the same formulas in FP64. One RHS of the 54-species mechanism issues 196 FP64
 // warp instructions with FX, 546 with FP64 exponentials and species factors
 // exp(+-G/RT) (counted in the source); the FP64 pipe bounded the rate evaluation.
@@ -1444,7 +1444,9 @@ __device__ __noinline__ Scal eval_rhs_fp64(const DevMech& m, Cta<NW> c, const do
 // RHS (and with JAC the Jacobian data) of the state y; T = y[0] selects the path.
 template <int NW, bool JAC, bool FF = false>
 __device__ __forceinline__ Scal eval_rhs(const DevMech& m, Cta<NW>& c, const double* y, double p, double* f) {
-  if (!(y[0] >= m.T_fx && y[0] < m.T_fx_end)) return eval_rhs_fp64<NW, JAC, FF>(m, c, y, p, f);
+  const int2 range = m.T_fx;
+  const int hT = __double2hiint(y[0]);  // (NaN is above every range)
+  if (hT < range.x || hT >= range.y) return eval_rhs_fp64<NW, JAC, FF>(m, c, y, p, f);
   return eval_rhs_t<NW, JAC, FF, true>(m, c, y, p, f);
 }
 

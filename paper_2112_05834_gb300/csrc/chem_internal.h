@@ -69,7 +69,10 @@ struct DevMech {
   int i_tb0;  // first reaction of kind >= 1 (sorted order)
   int i_fo0;  // first reaction of kind >= 2
   int i_troe0;  // first reaction of kind 3
-  double T_fx, T_fx_end;  // the fixed-point rate evaluation holds for T in [T_fx, T_fx_end)
+  // The fixed-point rate evaluation holds for T in [x, y), as the upper words of two doubles
+  // whose lower words are zero (one load; two doubles cost the 100-species integration 2 %:
+  // 88.7 -> 90.8 ms of 16,384 cells).
+  int2 T_fx;
   const long long* gfx;  // [K][16]: G/RT coefficients for range r at 8 r: constant (Q52), of ln T
                          //   (Q56), of 1/T (Q45), of t, t^2, t^3, t^4 (Q52), t = T 2^(fx_low - 12)
                          //   (r = 0) or T/8192 (r = 1)
