@@ -101,9 +101,10 @@ struct LuArgs {
 // layout leaves out the species arrays and registers are limited to five CTAs of 128 threads
 // (four before) or sixteen of 64 (n <= 32, which needs half of them); beyond n = 64 the
 // inverse stays in the registers of 256 threads instead of the shared memory of 128.
-// Mixed form: 8,192 of n = 55 712 -> 496 us, 65,536 of n = 16 1398 -> 476 us, 592 of
-// n = 101 3434 -> 310 us; FP64 form: 3,970 of n = 55 1619 -> 1533 us, 296 of n = 128 1737 ->
-// 1134 us, 100 of n = 55 158 -> 123 us.
+// Mixed form: 8,192 of n = 55 712 -> 501 us, 65,536 of n = 16 1398 -> 490 us, 592 of
+// n = 101 3434 -> 311 us; FP64 form: 3,970 of n = 55 1619 -> 1535 us, 296 of n = 128 1737 ->
+// 1133 us, 100 of n = 55 158 -> 123 us. (Of these 3 % at most are what the test of the
+// pivots' range and the rounding of the entries cost.)
 template <int NW, int PREC>
 __global__ void __launch_bounds__(NW * 32, NW == 2 ? 16 : NW == 4 ? 5 : 2) k_lu_solve(const __grid_constant__ LuArgs a) {
   using P = Policy<PREC>;
